@@ -218,6 +218,9 @@ struct CustomMat {
 
 // Internal kind of a custom unitary (outside the tqs_gate range).
 constexpr int kCustomKind = 64;
+// Internal kind of the phase diag(1, phi) that prepare_gates puts before the
+// target of a CNOT: it runs in a pass where its qubit is local, as hi + lo.
+constexpr int kPhaseKind = 65;
 
 // One recorded operation.
 struct Gate {
@@ -276,6 +279,11 @@ struct Program {
   int gen_index = 0;  // basis state the program starts from (leading X gates folded)
   int n_instr = 0;    // measure / reset instructions (one pass each)
   std::vector<float2> coef;  // custom unitaries' coefficients (wide passes)
+  // Factor of the rotations (phases, scales) that the program takes over when
+  // its compile starts; with `defer`, what it has not applied at the end is
+  // left here for the program that follows (else it is applied, and 1).
+  cd carry = 1.0;
+  bool defer = false;
   double cost = 0.0;
   // Empty the program for reuse (keeps the vectors' capacity).
   void reset() {
@@ -288,6 +296,8 @@ struct Program {
     out_scale = 1.0f;
     gen_index = 0;
     n_instr = 0;
+    carry = 1.0;
+    defer = false;
     cost = 0.0;
   }
 };
@@ -299,6 +309,7 @@ struct CompileRaw {
   bool is_h;    // unfused uncontrolled Hadamard
   bool single;  // uncontrolled single-qubit factor
   int t, c;     // physical bits (c = -1: uncontrolled)
+  bool hl;      // a phase to apply as FP32 hi + lo (kPhaseKind)
 };
 
 // Full-state-vector program: per pass the tile bits, the far bits it tests
@@ -331,8 +342,14 @@ constexpr int kMaxHPerPass = 48;
 // circuits of a batch.
 // absorb: fold the trailing permutation gates into the output map (not in
 // the full-state-vector tile programs, whose write-back is the tile's own).
+// prepared: the gates come from a prepare_gates that returned true.
 void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
-                     bool fold_x = true, bool absorb = true);
+                     bool fold_x = true, bool absorb = true, bool prepared = false);
+
+// Fusion of a circuit's single-qubit factors and the move of its phases past
+// one another, in place of gs (new gates live in `store`); see host_compile.cpp.
+bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store, cd& global,
+                   uint32_t* flips);
 
 inline int team_for(int nint) {
   if (nint <= kWarpMaxQ) return TEAM_WARP;

@@ -96,6 +96,7 @@ struct DiagEnt {
 // factor, else two.
 int diag_entries(const FusedOp& op, DiagEnt* e) {
   const int code = op.code;
+  if (code >= OPC_DLN && code < OPC_DLF && op.c) return 0;  // hi + lo: stays as it is
   const bool one = op.d0one != 0;
   const float2 d0 = op.m[0], d1 = op.m[1], r = op.m[2];
   if (code >= OPC_DLN && code < OPC_DLF) {  // local target, uncontrolled
@@ -185,6 +186,102 @@ double single_cost(const Mat2& u, bool is_h) {
       return hadamard_split(u, d2, d1) ? 1.5 : 3.5;
     }
   }
+}
+
+// An uncontrolled single-qubit unitary as the kernel runs it:
+//   u = gamma diag(1, alpha) X^flip scale R diag(1, beta),  R = [[1, -tau], [tau, 1]],
+// with phases alpha, beta, gamma and |tau| the ratio of the small to the large
+// entry, at most 1.  R costs one multiply-add per real part (the dense product
+// with hi + lo coefficients: eight), and scale = (1 + tau^2)^-1/2 is taken
+// from tau as FP32 holds it, so scale R is a rotation exactly: rounding tau
+// turns it by less than 1.5e-8 and leaves the norm alone.
+struct RotSplit {
+  bool flip;
+  float tau;
+  double scale;
+  cd alpha, beta, gamma;
+};
+
+// A phase within 1e-14 of 1, -1, i or -i is that value.
+cd snap_phase(cd z) {
+  const double re = std::round(z.real()), im = std::round(z.imag());
+  return std::abs(z - cd(re, im)) <= 1e-14 ? cd(re, im) : z / std::abs(z);
+}
+
+// real_column: the first column's ratio is known to be real (its computed phase
+// is then rounding, large beside a small entry), so alpha is a sign.
+RotSplit split_rotation(const Mat2& u, bool real_column) {
+  RotSplit r;
+  double c = std::abs(u.m[0]), s = std::abs(u.m[2]);
+  if (s <= 1e-14) s = 0.0;  // rounding of a zero: its phase means nothing
+  if (c <= 1e-14) c = 0.0;
+  r.flip = s > c;
+  // u = gamma diag(p0, p1) [[c, -s beta], [s, c beta]]; with s > c the bracket
+  // is X [[s, c beta], [c, -s beta]] = X [[s, -c beta'], [c, s beta']], beta' = -beta
+  cd p0, p1;  // the phases of the first column, row 0 and row 1
+  if (!r.flip) {
+    p0 = u.m[0] / c;
+    p1 = s > 0.0 ? u.m[2] / s : p0;
+    r.tau = static_cast<float>(s / c);
+    r.beta = u.m[3] / (p1 * std::abs(u.m[3]));
+  } else {
+    p1 = u.m[2] / s;
+    p0 = c > 0.0 ? u.m[0] / c : p1;
+    r.tau = static_cast<float>(c / s);
+    r.beta = u.m[1] / (p0 * std::abs(u.m[1]));
+  }
+  r.beta = snap_phase(r.beta);
+  r.gamma = snap_phase(p0);
+  r.alpha = snap_phase(p1 / p0);
+  if (real_column) r.alpha = r.alpha.real() < 0.0 ? -1.0 : 1.0;
+  if (r.alpha == cd(-1.0)) {  // a sign: the rotation the other way
+    r.alpha = 1.0;
+    r.tau = -r.tau;
+    r.beta = -r.beta;
+    if (r.flip) r.gamma = -r.gamma;
+  }
+  r.scale = 1.0 / std::sqrt(1.0 + double(r.tau) * double(r.tau));
+  return r;
+}
+
+// scale R diag(1, beta): what is left of u with gamma, alpha and X taken out.
+Mat2 rotation_part(const RotSplit& r) {
+  const double c = r.scale, s = r.scale * double(r.tau);
+  return {{c, -s * r.beta, s, c * r.beta}};
+}
+
+// The FP32 pair near z whose modulus is nearest |z|: a value that multiplies
+// every amplitude once.
+float2 to_mod_f2(cd z) {
+  const float2 rn = to_f2(z);
+  const double want = std::norm(z);
+  float xs[2] = {rn.x, rn.x}, ys[2] = {rn.y, rn.y};
+  if (double(rn.x) < z.real()) xs[1] = fstep(rn.x, true);
+  if (double(rn.x) > z.real()) xs[0] = fstep(rn.x, false);
+  if (double(rn.y) < z.imag()) ys[1] = fstep(rn.y, true);
+  if (double(rn.y) > z.imag()) ys[0] = fstep(rn.y, false);
+  float2 best = rn;
+  double best_m = std::abs(double(rn.x) * rn.x + double(rn.y) * rn.y - want);
+  for (int k = 0; k < 4; ++k) {
+    const float x = xs[k & 1], y = ys[k >> 1];
+    const double m = std::abs(double(x) * x + double(y) * y - want);
+    if (m < best_m) {
+      best = make_float2(x, y);
+      best_m = m;
+    }
+  }
+  return best;
+}
+
+// Uncontrolled factor that runs as a rotation: neither diagonal, nor X, nor a
+// Hadamard, nor one between exact phases.
+bool needs_rotation(const Gate& g) {
+  if (g.nq != 1 || is_instruction(g.kind) || is_two_qubit(g.kind) || g.kind == TQS_H) return false;
+  const GClass cls = classify_mat(g.u);
+  if (cls == G_DIAG) return false;
+  if (cls == G_ANTI) return !(exact_phase(g.u.m[1]) && exact_phase(g.u.m[2]));
+  Mat2 d1, d2;
+  return !hadamard_split(g.u, d2, d1);
 }
 
 // Local target position of a non-diagonal op.
@@ -569,8 +666,278 @@ void group_hadamards(std::vector<FusedOp>& ops, size_t begin) {
 
 }  // namespace
 
+// Circuit-wide fusion of single-qubit factors: consecutive uncontrolled
+// single-qubit gates on one qubit (no other gate on it in between; the gates
+// in between act on other qubits and commute) multiply into one factor at the
+// first one's place, by the mixed-product property of the Kronecker product,
+// unless the product runs costlier than the two apart.  Products equal to the
+// identity (H H, X X, ...) disappear; an exact X product is an X gate (an
+// exchange).
+//
+// Then, if a factor needs a rotation (split_rotation), what is left of each
+// factor beside its rotation moves on through the circuit.  A qubit carries a
+// pending factor of one of two kinds, with a phase phi:
+//   Z: diag(1, phi) X^flip, which passes controls and diagonal gates (an X on
+//      a control leaves one on the target, one on a controlled phase its
+//      inverse and a phase);
+//   X: H diag(1, phi) H, which passes the targets of CNOTs;
+// diagonal factors and X join a Z, a Hadamard turns one into the other, and the
+// next non-diagonal factor on the qubit absorbs either in FP64.  The factor u
+// times the pending one is split as
+//   gamma Z [scale R diag(1, beta)]  or  gamma X [scale R diag(1, beta)]
+// (both always exist), of which the bracket stays in the circuit and the left
+// factor becomes pending: X when the gates up to the qubit's next non-diagonal
+// factor are all CNOTs targeting it, else Z.  So a layer of general
+// single-qubit gates costs a phase and a rotation each, and X and Y nothing; a
+// pending factor becomes a gate of its own only before a gate that it does not
+// pass, and at the end.  The gammas multiply `global`; `flips`, if given,
+// receives the qubits whose X is left at the end (else it becomes a gate).
+// Circuits without such a factor (the paper's programs) are left as they are.
+// True when rotations were taken out.
+bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store, cd& global,
+                   uint32_t* flips) {
+  static thread_local std::vector<const Gate*> fl_tls;
+  std::vector<const Gate*>& fl = fl_tls;
+  fl.clear();
+  int open[TQS_MAX_FSV_QUBITS];
+  for (int& o : open) o = -1;
+  for (const Gate* g : gs) {
+    const bool single = g->nq == 1 && !is_instruction(g->kind) && !is_two_qubit(g->kind);
+    if (!single) {
+      fl.push_back(g);
+      for (int i = 0; i < g->nq; ++i) open[g->q[i]] = -1;
+      continue;
+    }
+    const int q = g->q[0];
+    if (open[q] >= 0) {
+      const Gate* pg = fl[static_cast<size_t>(open[q])];
+      const Mat2 uf = mat_mul(g->u, pg->u);
+      if (single_cost(uf, false) <=
+          single_cost(pg->u, pg->kind == TQS_H) + single_cost(g->u, g->kind == TQS_H)) {
+        if (is_identity2(uf)) {
+          fl[static_cast<size_t>(open[q])] = nullptr;
+          open[q] = -1;
+          continue;
+        }
+        store.push_back(*pg);
+        Gate& f = store.back();
+        f.u = uf;
+        f.cm.reset();
+        const bool is_x = uf.m[0] == cd(0.0) && uf.m[3] == cd(0.0) && uf.m[1] == cd(1.0) && uf.m[2] == cd(1.0);
+        f.kind = is_x ? TQS_X : TQS_U3;
+        fl[static_cast<size_t>(open[q])] = &f;
+        continue;
+      }
+    }
+    fl.push_back(g);
+    open[q] = static_cast<int>(fl.size()) - 1;
+  }
+  gs.clear();
+  bool rotations = false;
+  for (const Gate* g : fl)
+    if (g != nullptr) {
+      gs.push_back(g);
+      rotations = rotations || needs_rotation(*g);
+    }
+  if (!rotations) return false;
+  fl.swap(gs);
+  gs.clear();
+  // after[i]: what lies between the single-qubit gate i and the next
+  // non-diagonal one on its qubit
+  enum : uint8_t { kAbsorbed = 0, kZOnly = 1, kXOnly = 2, kOther = 3, kEnd = 4 };
+  static thread_local std::vector<uint8_t> after_tls;
+  std::vector<uint8_t>& after = after_tls;
+  after.assign(fl.size(), kEnd);
+  {
+    uint8_t st[TQS_MAX_FSV_QUBITS];
+    for (uint8_t& v : st) v = kEnd;
+    auto meet = [&](int q, uint8_t b) { st[q] = (st[q] == kAbsorbed || st[q] == kEnd || st[q] == b) ? b : kOther; };
+    for (size_t i = fl.size(); i-- > 0;) {
+      const Gate& g = *fl[i];
+      if (g.kind == TQS_SWAP) {
+        std::swap(st[g.q[0]], st[g.q[1]]);
+      } else if (is_controlled(g.kind)) {
+        meet(g.q[0], kZOnly);
+        const GClass cls = classify_mat(g.u);
+        meet(g.q[1], cls == G_DIAG ? kZOnly : g.kind == TQS_CNOT ? kXOnly : kOther);
+      } else if (g.nq != 1 || is_instruction(g.kind)) {
+        for (int k = 0; k < g.nq; ++k) meet(g.q[k], kOther);
+      } else {
+        after[i] = st[g.q[0]];
+        const GClass cls = classify_mat(g.u);
+        if (cls == G_DENSE) st[g.q[0]] = kAbsorbed;
+        else if (g.kind != TQS_X) meet(g.q[0], kZOnly);
+      }
+    }
+  }
+  struct Pend {
+    cd phi = 1.0;
+    bool x = false;     // kind X
+    bool flip = false;  // kind Z
+  };
+  Pend pend[TQS_MAX_FSV_QUBITS];
+  const Mat2 mat_x = {{0.0, 1.0, 1.0, 0.0}};
+  auto put = [&](int kind, int q, const Mat2& u) {
+    store.emplace_back();
+    Gate& g = store.back();
+    g.kind = kind;
+    for (int& v : g.q) v = q;
+    g.nq = 1;
+    g.u = u;
+    gs.push_back(&g);
+  };
+  auto put_phase = [&](int kind, int q, cd phi) {
+    if (phi != cd(1.0)) put(kind, q, {{1.0, 0.0, 0.0, phi}});
+  };
+  auto pend_mat = [&](const Pend& p) -> Mat2 {
+    if (!p.x) return p.flip ? Mat2{{0.0, 1.0, p.phi, 0.0}} : Mat2{{1.0, 0.0, 0.0, p.phi}};
+    const cd a = 0.5 * (1.0 + p.phi), b = 0.5 * (1.0 - p.phi);
+    return {{a, b, b, a}};
+  };
+  // the rotation of u into the circuit, its left factor pending
+  auto rotate = [&](int q, Mat2 u, bool left_x) {
+    Pend& p = pend[q];
+    p = Pend();
+    if (left_x) {
+      // the X factor that makes the first column real up to a phase, its larger part first
+      const cd w0 = u.m[0] + u.m[2], w1 = u.m[0] - u.m[2];
+      if (std::abs(w0) > 0.0 && std::abs(w1) > 0.0) p.phi = snap_phase((w1 / std::abs(w1)) / (w0 / std::abs(w0)));
+      p.x = true;
+      u = mat_mul(pend_mat({std::conj(p.phi), true, false}), u);
+    }
+    const RotSplit r = split_rotation(u, left_x);
+    global *= r.gamma;
+    if (left_x) {
+      if (r.flip) p.phi = -p.phi;  // X = H diag(1, -1) H
+    } else {
+      p.phi = r.alpha;
+      p.flip = r.flip;
+    }
+    put(TQS_U3, q, rotation_part(r));
+  };
+  // make the pending factor of q one that passes what the flags name: gates
+  // that Z (with its X) passes, those that X passes
+  auto settle = [&](int q, bool z, bool x) {
+    Pend& p = pend[q];
+    if (p.x) {
+      if (p.phi == cd(1.0)) p = Pend();
+      else if (!x) rotate(q, pend_mat(p), false);
+    }
+    if (p.x || z) return;
+    if (x) {
+      // only the phase stops: diag(1, phi) X = X phi diag(1, conj phi)
+      if (p.flip) global *= p.phi;
+      put_phase(kPhaseKind, q, p.flip ? std::conj(p.phi) : p.phi);
+      p.phi = 1.0;
+    } else {
+      if (p.flip) put(TQS_X, q, mat_x);
+      put_phase(kPhaseKind, q, p.phi);
+      p = Pend();
+    }
+  };
+  for (size_t i = 0; i < fl.size(); ++i) {
+    const Gate* g = fl[i];
+    if (g->kind == TQS_SWAP) {
+      std::swap(pend[g->q[0]], pend[g->q[1]]);
+      gs.push_back(g);
+      continue;
+    }
+    if (g->nq != 1 || is_instruction(g->kind)) {
+      if (!is_controlled(g->kind)) {
+        for (int k = 0; k < g->nq; ++k) settle(g->q[k], false, false);
+        gs.push_back(g);
+        continue;
+      }
+      Pend& pc = pend[g->q[0]];
+      Pend& pt = pend[g->q[1]];
+      if (classify_mat(g->u) != G_DIAG) {
+        settle(g->q[0], true, false);
+        if (g->kind != TQS_CNOT && pc.flip) settle(g->q[0], false, false);
+        settle(g->q[1], false, g->kind == TQS_CNOT);
+        if (g->kind == TQS_CNOT && pc.flip) {  // CNOT X_c = X_c X_t CNOT
+          if (pt.x) pt.phi = -pt.phi;
+          else pt.flip = !pt.flip;
+        }
+        gs.push_back(g);
+        continue;
+      }
+      settle(g->q[0], true, false);
+      settle(g->q[1], true, false);
+      if (!pc.flip && !pt.flip) {
+        gs.push_back(g);
+      } else if (g->u.m[0] != cd(1.0)) {
+        settle(g->q[0], false, false);
+        settle(g->q[1], false, false);
+        gs.push_back(g);
+      } else {
+        // the phase w where both bits are 1 after the X: with one X, w on the
+        // other qubit's 1 and w^-1 where both bits before are 1; with two,
+        // w on either's 1, w^-1 on all and w where both bits before are 1
+        const cd w = g->u.m[3];
+        if (pc.flip) pt.phi = snap_phase(pt.phi * w);
+        if (pt.flip) pc.phi = snap_phase(pc.phi * w);
+        if (pc.flip && pt.flip) {
+          global *= std::conj(w);
+          gs.push_back(g);
+        } else {
+          store.push_back(*g);
+          store.back().kind = TQS_CP;
+          store.back().u.m[3] = std::conj(w);
+          gs.push_back(&store.back());
+        }
+      }
+      continue;
+    }
+    const int q = g->q[0];
+    Pend& p = pend[q];
+    if (p.x && p.phi == cd(1.0)) p = Pend();
+    const bool none = p.phi == cd(1.0) && !p.flip;
+    const GClass cls = classify_mat(g->u);
+    if (cls == G_DIAG) {
+      settle(q, true, false);
+      global *= g->u.m[0];
+      p.phi = snap_phase(p.phi * g->u.m[3] / g->u.m[0]);
+    } else if (cls == G_ANTI && p.x && g->kind == TQS_X) {
+      p.phi = -p.phi;
+    } else if (cls == G_ANTI) {
+      // diag(b, c) X diag(1, phi) = b phi diag(1, c / (b phi)) X
+      settle(q, true, false);
+      const cd b = g->u.m[1] * p.phi;
+      global *= b;
+      p.phi = snap_phase(g->u.m[2] / b);
+      p.flip = !p.flip;
+    } else if (g->kind == TQS_H && (none || (p.x && after[i] != kXOnly))) {
+      p.x = !none && !p.x;
+      gs.push_back(g);
+    } else if (g->kind == TQS_H && p.flip && p.phi == cd(1.0)) {
+      p.flip = false;  // H X = Z H
+      p.phi = -1.0;
+      gs.push_back(g);
+    } else if (g->kind == TQS_H && !p.x && !p.flip && (after[i] == kXOnly || after[i] == kAbsorbed)) {
+      p.x = true;
+      gs.push_back(g);
+    } else {
+      rotate(q, mat_mul(g->u, pend_mat(p)), after[i] == kXOnly);
+    }
+  }
+  if (flips) *flips = 0;
+  for (int q = 0; q < n; ++q) {
+    Pend& p = pend[q];
+    settle(q, true, false);
+    if (flips && p.flip) {
+      *flips |= 1u << q;
+      global *= p.phi;
+      p.phi = std::conj(p.phi);
+    } else if (p.flip) {
+      put(TQS_X, q, mat_x);
+    }
+    put_phase(TQS_R, q, p.phi);
+  }
+  return true;
+}
+
 void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
-                      bool fold_x, bool absorb) {
+                     bool fold_x, bool absorb, bool prepared) {
   P.n = n;
   P.nint = std::max(n, 4);
   // scratch reused across calls on this thread (no allocation per circuit)
@@ -635,57 +1002,13 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     }
     gs.swap(xf);
   }
-  // Circuit-wide fusion of single-qubit factors: consecutive uncontrolled
-  // single-qubit gates on one qubit (no other gate on it in between; the
-  // gates in between act on other qubits and commute) multiply into one
-  // factor at the first one's place, by the mixed-product property of the
-  // Kronecker product, unless the product runs costlier than the two apart.
-  // Products equal to the identity (H H, X X, ...) disappear; an exact X
-  // product is an X gate (an exchange).
   static thread_local std::deque<Gate> fused_tls;
-  static thread_local std::vector<const Gate*> fl_tls;
-  std::deque<Gate>& fused = fused_tls;
-  std::vector<const Gate*>& fl = fl_tls;
-  fused.clear();
-  fl.clear();
-  {
-    int open[32];
-    for (int q = 0; q < 32; ++q) open[q] = -1;
-    for (const Gate* g : gs) {
-      const bool single = g->nq == 1 && !is_instruction(g->kind) && !is_two_qubit(g->kind);
-      if (!single) {
-        fl.push_back(g);
-        for (uint32_t m = qubit_mask(*g); m; m &= m - 1) open[__builtin_ctz(m)] = -1;
-        continue;
-      }
-      const int q = g->q[0];
-      if (open[q] >= 0) {
-        const Gate* pg = fl[static_cast<size_t>(open[q])];
-        const Mat2 uf = mat_mul(g->u, pg->u);
-        if (single_cost(uf, false) <=
-            single_cost(pg->u, pg->kind == TQS_H) + single_cost(g->u, g->kind == TQS_H)) {
-          if (is_identity2(uf)) {
-            fl[static_cast<size_t>(open[q])] = nullptr;
-            open[q] = -1;
-            continue;
-          }
-          fused.push_back(*pg);
-          Gate& f = fused.back();
-          f.u = uf;
-          f.cm.reset();
-          const bool is_x = uf.m[0] == cd(0.0) && uf.m[3] == cd(0.0) && uf.m[1] == cd(1.0) && uf.m[2] == cd(1.0);
-          f.kind = is_x ? TQS_X : TQS_U3;
-          fl[static_cast<size_t>(open[q])] = &f;
-          continue;
-        }
-      }
-      fl.push_back(g);
-      open[q] = static_cast<int>(fl.size()) - 1;
-    }
+  bool split = prepared;  // the program runs rotations (split_rotation)
+  uint32_t flips = 0;     // qubits with an X left after the program's gates
+  if (!prepared) {
+    fused_tls.clear();
+    split = prepare_gates(n, gs, fused_tls, P.carry, absorb ? &flips : nullptr);
   }
-  gs.clear();
-  for (const Gate* g : fl)
-    if (g != nullptr) gs.push_back(g);
 
   std::vector<uint32_t>& qmask = qmask_tls;
   std::vector<GClass>& gcls = cls_tls;
@@ -709,9 +1032,15 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
   int last_touch[32];
   int h_in_pass = 0;
   int h_carry = 0;  // Hadamard factors 2^-1/2 not yet applied
+  // The factor (phases and scales of the rotations, and of the Hadamards of a
+  // program that has any) not yet applied: the first pass multiplies the
+  // start by what is left of it at the end, so amplitudes never exceed the
+  // state's norm on the way.
+  cd& carry = P.carry;
+  int grow_in_pass = 0;  // rotations and Hadamards of the pass being built
   auto push_raw = [&](const Gate& g, GClass cls, int t, int c) {
     const bool single = (c < 0);
-    if (single) {
+    if (single && !split) {
       const int last = last_touch[t];
       if (last >= 0 && raw[last].single && raw[last].t == t) {
         // consecutive factors on one qubit multiply (the mixed-product
@@ -730,7 +1059,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     }
     const bool is_h = single && g.kind == TQS_H && h_in_pass < kMaxHPerPass;
     if (is_h) ++h_in_pass;
-    raw.push_back({g.u, cls, is_h, single, t, c});
+    raw.push_back({g.u, cls, is_h, single, t, c, g.kind == kPhaseKind});
     last_touch[t] = static_cast<int>(raw.size()) - 1;
     if (c >= 0) last_touch[c] = static_cast<int>(raw.size()) - 1;
   };
@@ -747,7 +1076,24 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     ps.op_begin = static_cast<uint32_t>(P.ops.size());
     double pass_cost = 6.0;
     int h_count = 0;
-    auto emit_raw = [&](const Raw& r) {
+    // the phase diag(1, alpha) that a rotation leaves on its own target
+    auto emit_phase = [&](cd alpha, int tl) {
+      FusedOp op{};
+      op.c = 1;  // hi + lo, multiplied in at once
+      op.code = static_cast<uint8_t>(OPC_DLN + tl);
+      op.fbit = op.tbit = 0xFF;
+      op.act = 0xFFFF;
+      op.d0one = 1;
+      op.m[0] = make_float2(1.f, 0.f);
+      op.m[1] = op.m[2] = op.hc = to_f2(alpha);
+      op.lo[0] = to_f2(alpha - cd(op.hc.x, op.hc.y));
+      P.ops.push_back(op);
+    };
+    auto emit_raw = [&](const Raw& r, auto&& emit_raw) -> void {
+      if (r.hl) {
+        emit_phase(r.u.m[3], loc[r.t]);
+        return;
+      }
       // a factor that fused to the identity (H H, X X, ...) does nothing
       if (!r.is_h && is_identity2(r.u)) return;
       FusedOp op{};
@@ -764,15 +1110,33 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
         if (cl >= 0) op.act = kLocalControlMask[cl];
         if (r.is_h) {
           op.code = static_cast<uint8_t>(OPC_H + tl);
-          ++h_count;
+          if (split) carry *= std::sqrt(0.5);
+          else ++h_count;
           pass_cost += 0.5;
         } else if (r.cls == G_ANTI && u.m[1] == cd(1.0) && u.m[2] == cd(1.0)) {
           if (r.c < 0) op.code = static_cast<uint8_t>(OPC_X + tl);
           else if (far_c) op.code = static_cast<uint8_t>(OPC_XF + tl);
           else op.code = static_cast<uint8_t>(OPC_XL + 4 * tl + cl);
           pass_cost += 0.5;
-        } else {  // dense, or anti-diagonal other than X (as a dense factor)
-          op.code = static_cast<uint8_t>((r.c < 0 ? OPC_DENSE : OPC_CDENSE) + tl);
+        } else if (r.c < 0) {  // dense, or anti-diagonal other than X: a rotation
+          const RotSplit rs = split_rotation(u, false);
+          carry *= rs.gamma * rs.scale;
+          op.code = static_cast<uint8_t>(OPC_DENSE + tl);
+          op.hc = make_float2(rs.tau, 0.f);
+          const float2 b = to_f2(rs.beta), bl = to_f2(rs.beta - cd(b.x, b.y));
+          op.d0one = rs.beta == cd(1.0) ? 1 : bl.x == 0.f && bl.y == 0.f ? 2 : 0;
+          op.m[0] = make_float2(1.f, 0.f);
+          op.m[1] = make_float2(-rs.tau * b.x, -rs.tau * b.y);
+          op.m[2] = make_float2(rs.tau, 0.f);
+          op.m[3] = b;
+          op.lo[3] = bl;
+          pass_cost += 1.0;
+          P.ops.push_back(op);
+          if (rs.flip) emit_raw({gate_matrix(TQS_X, nullptr), G_ANTI, false, true, r.t, -1, false}, emit_raw);
+          if (rs.alpha != cd(1.0)) emit_phase(rs.alpha, tl);
+          return;
+        } else {  // controlled: hi + lo coefficients
+          op.code = static_cast<uint8_t>(OPC_CDENSE + tl);
           for (int i = 0; i < 4; ++i) {
             op.m[i] = to_f2(u.m[i]);
             const cd hi(op.m[i].x, op.m[i].y);
@@ -813,23 +1177,23 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
       // unscaled Hadamard between exact phase factors instead of a dense
       // butterfly.
       Mat2 d1, d2;
-      if (r.single && !r.is_h && r.cls != G_DIAG && h_count < kMaxHPerPass &&
+      if (!split && r.single && !r.is_h && r.cls != G_DIAG && h_count < kMaxHPerPass &&
           hadamard_split(r.u, d2, d1)) {
-        emit_raw({d2, G_DIAG, false, true, r.t, -1});
-        emit_raw({gate_matrix(TQS_H, nullptr), G_DENSE, true, true, r.t, -1});
-        emit_raw({d1, G_DIAG, false, true, r.t, -1});
+        emit_raw({d2, G_DIAG, false, true, r.t, -1, false}, emit_raw);
+        emit_raw({gate_matrix(TQS_H, nullptr), G_DENSE, true, true, r.t, -1, false}, emit_raw);
+        emit_raw({d1, G_DIAG, false, true, r.t, -1, false}, emit_raw);
         continue;
       }
       // An uncontrolled anti-diagonal factor [[0, b], [c, 0]] other than X
       // with exact phases (Y, X Z, ...) is X diag(c, b): phases, then an
       // exchange.
-      if (r.single && !r.is_h && r.cls == G_ANTI && !(r.u.m[1] == cd(1.0) && r.u.m[2] == cd(1.0)) &&
+      if (!split && r.single && !r.is_h && r.cls == G_ANTI && !(r.u.m[1] == cd(1.0) && r.u.m[2] == cd(1.0)) &&
           exact_phase(r.u.m[1]) && exact_phase(r.u.m[2])) {
-        emit_raw({Mat2{{r.u.m[2], 0.0, 0.0, r.u.m[1]}}, G_DIAG, false, true, r.t, -1});
-        emit_raw({gate_matrix(TQS_X, nullptr), G_ANTI, false, true, r.t, -1});
+        emit_raw({Mat2{{r.u.m[2], 0.0, 0.0, r.u.m[1]}}, G_DIAG, false, true, r.t, -1, false}, emit_raw);
+        emit_raw({gate_matrix(TQS_X, nullptr), G_ANTI, false, true, r.t, -1, false}, emit_raw);
         continue;
       }
-      emit_raw(r);
+      emit_raw(r, emit_raw);
     }
     merge_diagonals(P.ops, ps.op_begin);
     group_hadamards(P.ops, ps.op_begin);
@@ -839,10 +1203,17 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     const int tot = h_carry + h_count;
     ps.scale = std::ldexp(1.0f, -(tot / 2));
     h_carry = tot % 2;
+    // rotations: rescaled only once the factor held back is below 2^-20
+    if (const double left = std::abs(carry); left < 0x1p-20) {
+      const int k = -std::ilogb(left) - 1;
+      ps.scale = std::ldexp(ps.scale, -k);
+      carry *= std::ldexp(1.0, k);
+    }
     P.passes.push_back(ps);
     P.cost += pass_cost * static_cast<double>(1u << nint);
     raw.clear();
     h_in_pass = 0;
+    grow_in_pass = 0;
   };
   // An instruction is a barrier: the gates before it are scheduled (pending),
   // then it becomes a pass of its own, then scheduling resumes after it.
@@ -879,12 +1250,22 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
       const int cq = is_controlled(g.kind) ? g.q[0] : -1;
       const int t = phys[tq];
       const int c = cq >= 0 ? phys[cq] : -1;
-      if (cls != G_DIAG && !((Lmask >> t) & 1)) {
+      if (g.kind == kPhaseKind && !((Lmask >> t) & 1) && idx + 1 < pending.size() &&
+          (qmask[pending[idx + 1]] & blocked)) {
+        // its CNOT (the gate after it) cannot join this pass: neither takes a local position
+        blocked |= qm;
+        still.push_back(pending[idx]);
+        continue;
+      }
+      const bool grows = split && c < 0 && cls == G_DENSE;
+      if (grows && grow_in_pass >= kMaxHPerPass) { blocked |= qm; still.push_back(pending[idx]); continue; }
+      if ((cls != G_DIAG || g.kind == kPhaseKind) && !((Lmask >> t) & 1)) {
         if (nL == 4) { blocked |= qm; still.push_back(pending[idx]); continue; }
         Lmask |= 1u << t;
         ++nL;
       }
       push_raw(g, cls, t, c);
+      grow_in_pass += grows;
     }
     for (; idx < pending.size(); ++idx) still.push_back(pending[idx]);
     emit_pass(Lmask, nL, still.empty());
@@ -932,6 +1313,29 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
   take_segment();
   }
   if (P.passes.empty()) emit_pass(0u, 0, true);
+  // What is left of the rotations' phases and scales multiplies the start (or,
+  // in a full-state-vector pass that is not the last, passes on to the next).
+  if (carry != cd(1.0)) {
+    if (h_carry) carry *= std::sqrt(0.5);
+    h_carry = 0;
+    if (!P.defer) {
+      FusedOp op{};
+      op.code = OPC_DLIST;
+      op.t = 4;
+      op.c = 1;
+      op.fbit = op.tbit = 0xFF;
+      op.act = 0xFFFF;
+      std::memset(&op.hc, 0xFF, sizeof(op.hc));  // every factor always on
+      op.m[0] = to_mod_f2(carry);
+      for (int k = 1; k < 4; ++k) op.m[k] = make_float2(1.f, 0.f);
+      for (float2& v : op.lo) v = make_float2(1.f, 0.f);
+      P.ops.insert(P.ops.begin() + P.passes[0].op_begin, op);
+      ++P.passes[0].op_count;
+      for (size_t i = 1; i < P.passes.size(); ++i)
+        if (P.passes[i].L[0] != kInstrPass && P.passes[i].L[0] != kWidePass) ++P.passes[i].op_begin;
+      carry = 1.0;
+    }
+  }
   // Drop passes left with nothing to do (every factor fused to the identity).
   // The first pass kept generates the start state, so it must be a register
   // pass: an empty one stays in front of a leading instruction or custom
@@ -962,7 +1366,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
   // composed with the relabeling phys.  F(y) = g_1(g_2(... g_k(y))) for the
   // tail g_1 .. g_k: built by F <- F o g for g in order.
   uint32_t fcol[32];
-  uint32_t fv = 0;
+  uint32_t fv = flips;  // an X after the gates and before the tail: F(y) ^ flips
   for (int q = 0; q < 32; ++q) fcol[q] = 1u << q;
   for (const Gate* g : tail) {
     if (g->kind == TQS_X) {

@@ -99,7 +99,7 @@ tqs_status tqs_batch_sample(tqs_batch* b, const double* d_probs, int shots, cons
 // bits, a custom unitary's bits), at most T in all.  Controls and diagonal
 // factors may sit on any bit.  Unused tile slots take the lowest free bits.
 
-static tqs_status compile_fsv(int n, const std::vector<Gate>& gates, int max_gates, int tile_opt,
+static tqs_status compile_fsv(int n, const std::vector<Gate>& circuit, int max_gates, int tile_opt,
                               FsvProgram& P) {
   P = FsvProgram();
   P.max_gates = max_gates;
@@ -117,12 +117,24 @@ static tqs_status compile_fsv(int n, const std::vector<Gate>& gates, int max_gat
       for (int i = 0; i < g.nq; ++i) m |= uint64_t(1) << g.q[i];
       return m;
     }
-    if (classify_mat(g.u) == G_DIAG) return 0;
+    if (classify_mat(g.u) == G_DIAG && g.kind != kPhaseKind) return 0;
     return uint64_t(1) << (is_controlled(g.kind) ? g.q[1] : g.q[0]);
   };
-  for (const Gate& g : gates)
+  for (const Gate& g : circuit)
     if (is_instruction(g.kind))
       return fail(TQS_ERR_UNSUPPORTED, "tqs_simulate_fsv: measure/reset instructions are not supported");
+  // Fusion and the phases' moves see the whole circuit, so that a phase is
+  // applied where it is absorbed and not at the end of every pass (the form
+  // with a bound on the gates per pass counts the circuit's own gates).
+  std::vector<const Gate*> gates;
+  for (const Gate& g : circuit) gates.push_back(&g);
+  std::deque<Gate> store;
+  cd carry = 1.0;
+  const bool split = max_gates == 0 && prepare_gates(n, gates, store, carry, nullptr);
+  if (max_gates == 0 && !split) {
+    gates.clear();
+    for (const Gate& g : circuit) gates.push_back(&g);
+  }
   // One in-order scan per pass: a gate joins the pass if no earlier gate left
   // for a later pass shares a qubit with it (gates on disjoint qubits
   // commute), its non-diagonal bits fit the tile and its other bits fit the
@@ -140,7 +152,7 @@ static tqs_status compile_fsv(int n, const std::vector<Gate>& gates, int max_gat
     for (; i < pending.size() && blocked != all &&
            (max_gates == 0 || cur.size() < static_cast<size_t>(max_gates));
          ++i) {
-      const Gate& g = gates[pending[i]];
+      const Gate& g = *gates[static_cast<size_t>(pending[i])];
       uint64_t qm = 0;
       for (int j = 0; j < g.nq; ++j) qm |= uint64_t(1) << g.q[j];
       const uint64_t need = need_of(g);
@@ -181,7 +193,12 @@ static tqs_status compile_fsv(int n, const std::vector<Gate>& gates, int max_gat
       ptrs[k] = &relabelled[k];
     }
     Program tp;
-    compile_program(T + info.nfar, ptrs, tp, false, false);
+    if (split) {
+      tp.carry = carry;
+      tp.defer = !pending.empty();
+    }
+    compile_program(T + info.nfar, ptrs, tp, false, false, split);
+    carry = tp.carry;
     P.passes.push_back(info);
     P.progs.push_back(std::move(tp));
   }

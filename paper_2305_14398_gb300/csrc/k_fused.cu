@@ -90,27 +90,39 @@ __device__ __forceinline__ float2 sel(bool on, float2 y, float2 x) {
   return make_float2(on ? y.x : x.x, on ? y.y : x.y);
 }
 
-// CTRL = false: every pair (an uncontrolled factor, no selects).
-template <int T, bool CTRL>
+template <int T>
 __device__ __forceinline__ void dense_t(float2 (&a)[16], const Coef& m, unsigned act) {
 #pragma unroll
   for (int p = 0; p < 8; ++p) {
     const int j0 = ((p >> T) << (T + 1)) | (p & ((1 << T) - 1));
     const int j1 = j0 | (1 << T);
     const float2 x0 = a[j0], x1 = a[j1];
-    if (CTRL) {
-      const bool on = (act >> j0) & 1;
-      a[j0] = sel(on, cmac2_hl(m.h[0], m.l[0], x0, m.h[1], m.l[1], x1), x0);
-      a[j1] = sel(on, cmac2_hl(m.h[2], m.l[2], x0, m.h[3], m.l[3], x1), x1);
-    } else {
-      a[j0] = cmac2_hl(m.h[0], m.l[0], x0, m.h[1], m.l[1], x1);
-      a[j1] = cmac2_hl(m.h[2], m.l[2], x0, m.h[3], m.l[3], x1);
-    }
+    const bool on = (act >> j0) & 1;
+    a[j0] = sel(on, cmac2_hl(m.h[0], m.l[0], x0, m.h[1], m.l[1], x1), x0);
+    a[j1] = sel(on, cmac2_hl(m.h[2], m.l[2], x0, m.h[3], m.l[3], x1), x1);
   }
 }
 
-
-
+// Unscaled rotation of every pair: (x0 - tau x1, x1 + tau x0).  One packed
+// multiply-add per amplitude: each part is rounded once.  With its phase (hi +
+// lo, 8 multiply-adds on half the amplitudes) a general gate takes 6 FP32
+// operations per amplitude where the dense product with hi + lo coefficients
+// took 16: 4096 random circuits of 4..14 qubits 885 -> 475 us, 1024 of 14
+// qubits 960 -> 694 us, a 26-qubit tiled state 23.8 -> 20.5 ms; error against
+// FP64 2.1e-7 -> 1.6e-7, 2.8e-7 -> 2.2e-7, 6.3e-7 -> 5.7e-7 (phases in FP32
+// without lo: 6.9e-7).
+template <int T>
+__device__ __forceinline__ void rot_t(float2 (&a)[16], float tau) {
+  const float2 p = make_float2(tau, tau), m = make_float2(-tau, -tau);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int j0 = ((k >> T) << (T + 1)) | (k & ((1 << T) - 1));
+    const int j1 = j0 | (1 << T);
+    const float2 x0 = a[j0], x1 = a[j1];
+    a[j0] = __ffma2_rn(m, x1, x0);
+    a[j1] = __ffma2_rn(p, x0, x1);
+  }
+}
 
 template <int T>
 __device__ __forceinline__ void swap_t(float2 (&a)[16], unsigned act) {
@@ -148,6 +160,27 @@ __device__ __forceinline__ void cmul_in(float2& a, float2 b) {
   const float t = a.y * b.y, u = a.y * b.x;
   a.y = fmaf(a.x, b.y, u);
   a.x = fmaf(a.x, b.x, -t);
+}
+
+// a <- (h + l) a in place: a phase whose FP32 rounding residue l counts (the
+// phases of rotations, about one per general gate).  The last product of each
+// part is with that part itself.
+__device__ __forceinline__ void cmul_hl_in(float2& a, float2 h, float2 l) {
+  float re = l.x * a.x, im = l.x * a.y;
+  re = fmaf(-l.y, a.y, re);
+  im = fmaf(l.y, a.x, im);
+  re = fmaf(-h.y, a.y, re);
+  im = fmaf(h.y, a.x, im);
+  a.x = fmaf(h.x, a.x, re);
+  a.y = fmaf(h.x, a.y, im);
+}
+
+// The amplitudes with local bit T set times h + l.
+template <int T>
+__device__ __forceinline__ void phase_hl_t(float2 (&a)[16], float2 h, float2 l) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j)
+    if ((j >> T) & 1) cmul_hl_in(a[j], h, l);
 }
 
 template <int B>
@@ -221,19 +254,17 @@ __device__ __forceinline__ void pend_mul(Pending& pd, int b, float2 v) {
   pd.dirty |= 1u << b;
 }
 
-__device__ __forceinline__ void pend_flush(float2 (&a)[16], Pending& pd, int b) {
-  if (!((pd.dirty >> b) & 1)) return;
+// Multiply in the pending phases of the positions in `mask`.
+__device__ __forceinline__ void pend_flush(float2 (&a)[16], Pending& pd, unsigned mask) {
+  const unsigned m = pd.dirty & mask;
+  if (m == 0) return;
   const float2 one = make_float2(1.f, 0.f);
-  switch (b) {
-    case 0: scale_bit<0>(a, pd.p[0]); pd.p[0] = one; break;
-    case 1: scale_bit<1>(a, pd.p[1]); pd.p[1] = one; break;
-    case 2: scale_bit<2>(a, pd.p[2]); pd.p[2] = one; break;
-    default: scale_bit<3>(a, pd.p[3]); pd.p[3] = one; break;
-  }
-  pd.dirty &= ~(1u << b);
+  if (m & 1) { scale_bit<0>(a, pd.p[0]); pd.p[0] = one; }
+  if (m & 2) { scale_bit<1>(a, pd.p[1]); pd.p[1] = one; }
+  if (m & 4) { scale_bit<2>(a, pd.p[2]); pd.p[2] = one; }
+  if (m & 8) { scale_bit<3>(a, pd.p[3]); pd.p[3] = one; }
+  pd.dirty &= ~m;
 }
-
-
 
 __device__ __forceinline__ float2 f2(unsigned x, unsigned y) {
   return make_float2(__uint_as_float(x), __uint_as_float(y));
@@ -242,11 +273,14 @@ __device__ __forceinline__ float2 f2(unsigned x, unsigned y) {
 // Apply the ops of one pass to the 16 amplitudes of one group, then the
 // pass's exact power-of-two scale.  The next op's header is fetched while the
 // current one runs.
-// SPLIT_DENSE: uncontrolled dense factors take a select-free copy of the
-// butterfly (more code; the full-state-vector tiles and the CTA-sized teams,
-// dominated by dense single-qubit factors, use it; the warp and pair teams
-// keep one copy, measured faster on the paper-shaped circuits).
-template <bool SPLIT_DENSE>
+// Bound by instruction issue, and in the warp teams by instruction fetch:
+// their warps are all at different ops, and with separate copies of the flush,
+// the exchange and the phase per op kind they stalled 12 cycles per
+// instruction on fetch (2048 random circuits of 9..11 qubits: 488 us, with
+// one place each 314 us).  SMALL keeps also the hi + lo phase in one place;
+// the other teams' warps run the same ops at about the same time and take one
+// branch less instead (n = 14 batch 702 -> 694 us).
+template <bool SMALL>
 __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restrict__ ops,
                                         uint32_t count, int base, float scale) {
   Pending pd;
@@ -263,51 +297,83 @@ __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restri
     const int code = q0.x & 0xff;
     const int fbit = (q0.y >> 8) & 0xff;
     if (fbit != 0xff && !((base >> fbit) & 1)) continue;  // a far control is 0 here
-    if (code < OPC_DLN) {
-      // non-diagonal: target local position t
+    // a phase that a rotation left on its target: hi + lo, at once
+    const bool phase_op = code >= OPC_DLN && code < OPC_DFL && ((q0.x >> 16) & 0xff);
+    if (code < OPC_DLN || phase_op) {
+      // target local position t, or the mask hm of a Hadamard's positions;
+      // exchanges act on the pairs in `act`
       int t = code & 3;
       unsigned act = q0.y >> 16;
+      const bool had = code < OPC_X || code == OPC_HMASK;
+      const bool rot = code >= OPC_DENSE && code < OPC_CDENSE;
+      unsigned hm = 1u << t;
+      if (code == OPC_HMASK) hm = (q0.x >> 8) & 15;
       if (code >= OPC_XL && code < OPC_ANTI) {
         t = (code - OPC_XL) >> 2;
         act = bit_mask((code - OPC_XL) & 3);
+        hm = 1u << t;
+      } else if (code == OPC_XP) {
+        // under a parity of local and far bits
+        t = (q0.x >> 8) & 3;
+        if (__popc(static_cast<unsigned>(base) & q0.z) & 1) act ^= 0xFFFFu;
+        hm = 1u << t;
       }
-      if (code < OPC_X) {
-        pend_flush(a, pd, t);
-        switch (t) {
-          case 0: h_t<0>(a); break;
-          case 1: h_t<1>(a); break;
-          case 2: h_t<2>(a); break;
-          default: h_t<3>(a); break;
-        }
-      } else if (code < OPC_ANTI) {
-        pend_flush(a, pd, t);
+      float2 bh = f2(q0.z, q0.w), bl = make_float2(0.f, 0.f);
+      const int kind = phase_op ? 0 : q0.y & 0xff;  // a rotation's phase: 0 hi + lo, 1 none, 2 exact
+      if (rot && kind != 1) {
+        const uint4 qh = __ldg(rec + 2), ql = __ldg(rec + 4);
+        bh = f2(qh.z, qh.w);
+        bl = f2(ql.z, ql.w);
+        if (kind == 2) pend_mul(pd, t, bh);
+      }
+      pend_flush(a, pd, hm);
+      if (had) {
+        if (hm & 1) h_t<0>(a);
+        if (hm & 2) h_t<1>(a);
+        if (hm & 4) h_t<2>(a);
+        if (hm & 8) h_t<3>(a);
+      } else if (code < OPC_DENSE) {
         switch (t) {
           case 0: swap_t<0>(a, act); break;
           case 1: swap_t<1>(a, act); break;
           case 2: swap_t<2>(a, act); break;
           default: swap_t<3>(a, act); break;
         }
-      } else if (code == OPC_HMASK) {
-        // Hadamards on several local positions, one dispatch
-        const int hm = (q0.x >> 8) & 15;
-        if (hm & 1) { pend_flush(a, pd, 0); h_t<0>(a); }
-        if (hm & 2) { pend_flush(a, pd, 1); h_t<1>(a); }
-        if (hm & 4) { pend_flush(a, pd, 2); h_t<2>(a); }
-        if (hm & 8) { pend_flush(a, pd, 3); h_t<3>(a); }
-      } else if (code == OPC_XP) {
-        // exchanges on one position under a parity of local and far bits
-        const int tt = (q0.x >> 8) & 3;
-        unsigned act2 = q0.y >> 16;
-        if (__popc(static_cast<unsigned>(base) & q0.z) & 1) act2 ^= 0xFFFFu;
-        pend_flush(a, pd, tt);
-        switch (tt) {
-          case 0: swap_t<0>(a, act2); break;
-          case 1: swap_t<1>(a, act2); break;
-          case 2: swap_t<2>(a, act2); break;
-          default: swap_t<3>(a, act2); break;
+      } else if (!SMALL && rot) {
+        const float tau = __uint_as_float(q0.z);
+        switch (kind == 0 ? 4 + t : t) {
+          case 0: rot_t<0>(a, tau); break;
+          case 1: rot_t<1>(a, tau); break;
+          case 2: rot_t<2>(a, tau); break;
+          case 3: rot_t<3>(a, tau); break;
+          case 4: phase_hl_t<0>(a, bh, bl); rot_t<0>(a, tau); break;
+          case 5: phase_hl_t<1>(a, bh, bl); rot_t<1>(a, tau); break;
+          case 6: phase_hl_t<2>(a, bh, bl); rot_t<2>(a, tau); break;
+          default: phase_hl_t<3>(a, bh, bl); rot_t<3>(a, tau); break;
+        }
+      } else if (rot || phase_op) {
+        if (kind == 0) {
+          if (phase_op) {
+            const uint4 ql = __ldg(rec + 3);
+            bl = f2(ql.x, ql.y);
+          }
+          switch (t) {
+            case 0: phase_hl_t<0>(a, bh, bl); break;
+            case 1: phase_hl_t<1>(a, bh, bl); break;
+            case 2: phase_hl_t<2>(a, bh, bl); break;
+            default: phase_hl_t<3>(a, bh, bl); break;
+          }
+        }
+        if (SMALL && rot) {
+          const float tau = __uint_as_float(q0.z);
+          switch (t) {
+            case 0: rot_t<0>(a, tau); break;
+            case 1: rot_t<1>(a, tau); break;
+            case 2: rot_t<2>(a, tau); break;
+            default: rot_t<3>(a, tau); break;
+          }
         }
       } else {
-        pend_flush(a, pd, t);
         const uint4 q1 = __ldg(rec + 1);
         const uint4 q2 = __ldg(rec + 2);
         const uint4 q3 = __ldg(rec + 3);
@@ -321,20 +387,11 @@ __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restri
         m.l[1] = f2(q3.z, q3.w);
         m.l[2] = f2(q4.x, q4.y);
         m.l[3] = f2(q4.z, q4.w);
-        if (SPLIT_DENSE && code < OPC_CDENSE) {
-          switch (t) {
-            case 0: dense_t<0, false>(a, m, act); break;
-            case 1: dense_t<1, false>(a, m, act); break;
-            case 2: dense_t<2, false>(a, m, act); break;
-            default: dense_t<3, false>(a, m, act); break;
-          }
-        } else {
-          switch (t) {
-            case 0: dense_t<0, true>(a, m, act); break;
-            case 1: dense_t<1, true>(a, m, act); break;
-            case 2: dense_t<2, true>(a, m, act); break;
-            default: dense_t<3, true>(a, m, act); break;
-          }
+        switch (t) {
+          case 0: dense_t<0>(a, m, act); break;
+          case 1: dense_t<1>(a, m, act); break;
+          case 2: dense_t<2>(a, m, act); break;
+          default: dense_t<3>(a, m, act); break;
         }
       }
       continue;
@@ -476,10 +533,7 @@ __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restri
       }
     }
   }
-  pend_flush(a, pd, 0);
-  pend_flush(a, pd, 1);
-  pend_flush(a, pd, 2);
-  pend_flush(a, pd, 3);
+  pend_flush(a, pd, 15u);
   if (sc_set) {
     sc.x *= scale;  // exact: scale is a power of two
     sc.y *= scale;
@@ -748,9 +802,7 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
           a[j] = ld_state<TEAM>(&st[TQS_IX(sb ^ ((j & 1) ? w0 : 0) ^ ((j & 2) ? w1 : 0) ^ ((j & 4) ? w2 : 0) ^ ((j & 8) ? w3 : 0), 1 << nint)]);
         }
       }
-      // select-free dense butterflies where they pay: the CTA-sized teams,
-      // whose random-circuit workloads are dense-gate heavy
-      run_ops<TEAM != TEAM_WARP && TEAM != TEAM_PAIR>(a, ops, count, base, scale);
+      run_ops<TEAM == TEAM_WARP || TEAM == TEAM_PAIR>(a, ops, count, base, scale);
 #pragma unroll
       for (int j = 0; j < 16; ++j)
         st[TQS_IX(sb ^ ((j & 1) ? w0 : 0) ^ ((j & 2) ? w1 : 0) ^ ((j & 4) ? w2 : 0) ^ ((j & 8) ? w3 : 0), 1 << nint)] = a[j];
@@ -950,6 +1002,13 @@ __device__ __forceinline__ uint64_t deposit64(uint64_t v, uint64_t mask) {
 
 constexpr int kFsvHighQ = kFsvTileQ - kFsvLowQ;
 
+// A state amplitude, read once: past L1, which keeps the pass's op records.
+__device__ __forceinline__ float2 ld_stream(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+  return v;
+}
+
 __global__ void __launch_bounds__(kFsvThreads)
     fsv_tile_kernel(const __grid_constant__ FusedLaunch L, const __grid_constant__ FsvTile F) {
   extern __shared__ float4 smem_raw[];
@@ -981,7 +1040,7 @@ __global__ void __launch_bounds__(kFsvThreads)
     int ext = 0;
     for (int v = 0; v < F.nfar; ++v) ext |= static_cast<int>((gbase >> F.far[v]) & 1) << (T + v);
     for (int e = tid; e < NT; e += kFsvThreads)
-      st[TQS_IX(swz(e), NT)] = g[TQS_IX(gbase + hoff[e >> nlow] + (e & lowm), 1ull << F.n)];
+      st[TQS_IX(swz(e), NT)] = ld_stream(&g[TQS_IX(gbase + hoff[e >> nlow] + (e & lowm), 1ull << F.n)]);
     __syncthreads();
     for (int p = 0; p < cd.pass_count; ++p) {
       const uint4 pr = __ldg(reinterpret_cast<const uint4*>(L.passes + cd.pass_begin + p));
@@ -1001,7 +1060,7 @@ __global__ void __launch_bounds__(kFsvThreads)
 #pragma unroll
         for (int q = 0; q < 16; ++q)
           a[q] = st[TQS_IX(sb ^ ((q & 1) ? w0 : 0) ^ ((q & 2) ? w1 : 0) ^ ((q & 4) ? w2 : 0) ^ ((q & 8) ? w3 : 0), NT)];
-        run_ops<true>(a, ops, count, base | ext, scale);
+        run_ops<false>(a, ops, count, base | ext, scale);
 #pragma unroll
         for (int q = 0; q < 16; ++q)
           st[TQS_IX(sb ^ ((q & 1) ? w0 : 0) ^ ((q & 2) ? w1 : 0) ^ ((q & 4) ? w2 : 0) ^ ((q & 8) ? w3 : 0), NT)] = a[q];

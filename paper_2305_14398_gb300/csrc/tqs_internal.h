@@ -35,9 +35,15 @@ namespace tqs {
 //                    XOR the parity of the group's physical bits in the far
 //                    mask (the first 4 bytes of hc) is 1; field c = the local
 //                    control positions (a run of X / CNOT factors on one target)
-//   OPC_DENSE + t    uncontrolled 2x2, coefficients as FP32 hi + lo
+//   OPC_DENSE + t    uncontrolled 2x2 as a rotation after a phase (the rest of
+//                    the gate, its outer phase, X and scale, is carried by the
+//                    compiler): [[1, -tau], [tau, 1]] diag(1, beta); tau in
+//                    hc.x; `d0one` = 1 when beta is exactly 1, 2 when FP32
+//                    holds it, else 0; beta as hi + lo in m[3], lo[3]; m holds
+//                    the product
 //   OPC_CDENSE + t   controlled 2x2 (`act` mask for a local control, `fbit` far)
-//   OPC_DLN + t      diag(d0, d1), local target, uncontrolled
+//   OPC_DLN + t      diag(d0, d1), local target, uncontrolled; field c = 1:
+//                    diag(1, d1) with d1 as hi + lo (hc, lo[0])
 //   OPC_DLF + t      diag(d0, d1), local target, far control `fbit`
 //   OPC_DFL + c      diag(d0, d1), far target bit `tbit`, local control c
 //   OPC_DFF          diag(d0, d1), far target bit `tbit`, no or far control `fbit`
@@ -94,7 +100,7 @@ struct alignas(16) FusedOp {
   float2 hc;       // diagonal ops, in the header so no further load is needed in the
                    // common case: d1/d0 (DLN, DLF) or d1 (DFL, DFF, DLL)
   float2 m[4];     // DENSE: m00 m01 m10 m11 | ANTI: -, m01, m10, - | DIAG: d0, d1, d1/d0, -
-  float2 lo[4];    // DENSE: m - m_fp32 rounded to FP32 (the FP64 matrix is m + lo)
+  float2 lo[4];    // CDENSE: m - m_fp32 rounded to FP32 (the FP64 matrix is m + lo)
 };
 static_assert(sizeof(FusedOp) == 80, "FusedOp layout");
 
