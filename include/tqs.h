@@ -92,7 +92,8 @@ typedef enum {
 
 /* Arithmetic of the circuit-unitary chain (Algorithm 1). */
 typedef enum {
-  TQS_PREC_FP32_SIMT = 0,   /* FP32 CUDA-core complex GEMM (4 real products) */
+  TQS_PREC_FP32_SIMT = 0,   /* FP32 on the CUDA cores: the products' terms with nonzero
+                               entries of S_k only, column by column */
   TQS_PREC_TC_BF16X3 = 1,   /* tcgen05 tensor cores, 3M complex product, each real
                                product as BF16 hi*hi + hi*lo + lo*hi, FP32 accumulate */
   TQS_PREC_TC_TF32X3 = 2    /* as above with TF32 hi/lo splits (kind::tf32) */
@@ -227,7 +228,7 @@ tqs_status tqs_materialize_step(tqs_circuit* c, int step, tqs_c64* d_S, void* st
  * n <= TQS_MAX_DENSE_QUBITS; tensor-core precisions need n >= 7.
  * Scratch (cached on the circuit): 36 * 4^n bytes for TQS_PREC_TC_BF16X3
  * (three matrices of six BF16 planes), 72 * 4^n for TQS_PREC_TC_TF32X3 (FP32
- * words), 24 * 4^n for TQS_PREC_FP32_SIMT.
+ * words), 8 * 4^n + 84 * 2^n for TQS_PREC_FP32_SIMT.
  * The tensor-core form synchronises `stream` before returning and returns
  * TQS_ERR_TIMEOUT if one of its bounded device waits ran out. */
 tqs_status tqs_circuit_unitary(tqs_circuit* c, int prec, tqs_c64* d_U, void* stream);
@@ -246,8 +247,8 @@ tqs_status tqs_circuit_unitary(tqs_circuit* c, int prec, tqs_c64* d_U, void* str
  * of 128 (the tensor-core tile), else TQS_ERR_ARG; a block outside the 2^n
  * columns is TQS_ERR_ARG.  Scratch (cached on the circuit): the step matrix's
  * operands plus two ncols x 2^n chain matrices (BF16x3: 12 * 4^n +
- * 24 * ncols * 2^n bytes; TF32x3 twice that; FP32 SIMT: 8 * 4^n +
- * 16 * ncols * 2^n). */
+ * 24 * ncols * 2^n bytes; TF32x3 twice that; FP32 SIMT: 8 * ncols * 2^n +
+ * 84 * ncols). */
 tqs_status tqs_circuit_unitary_cols(tqs_circuit* c, int prec, int col0, int ncols, tqs_c64* d_U,
                                     int64_t ldu, void* stream);
 

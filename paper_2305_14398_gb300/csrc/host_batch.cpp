@@ -506,9 +506,19 @@ static tqs_status unitary_block(tqs_circuit* c, int prec, int col0, int ncols, t
   if (c->n >= 7 && (col0 % 128 != 0 || ncols % 128 != 0))
     return fail(TQS_ERR_ARG, "%s: for n >= 7, col0 and ncols must be multiples of 128", who);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  float2* U = reinterpret_cast<float2*>(d_U);
+  if (prec == TQS_PREC_FP32_SIMT && c->nsteps > 1) {
+    const Program& P = ensure_program(c);
+    FusedLaunch L{};
+    tqs_status st = c->cols_prog.ensure(P, nullptr, L, s, "tqs_circuit_unitary: upload program");
+    if (st != TQS_OK) return st;
+    TQS_CUDA(c->d_chain.ensure(columns_scratch_bytes(c->n, ncols)), "tqs_circuit_unitary: cudaMalloc");
+    TQS_CUDA(launch_columns(L, c->n, P.nint, col0, ncols, U, ldu, c->d_chain.p, device_sms(), s),
+             "tqs_circuit_unitary: columns");
+    return TQS_OK;
+  }
   tqs_status st = upload_factors(c, s);
   if (st != TQS_OK) return st;
-  float2* U = reinterpret_cast<float2*>(d_U);
   if (c->nsteps <= 1) {
     // Algorithm 1 with at most one step: U = S_1 (or the identity).
     StepDesc d = c->nsteps == 1 ? c->steps[0] : StepDesc{0, 0, (1u << c->n) - 1u, 0};
@@ -524,13 +534,6 @@ static tqs_status unitary_block(tqs_circuit* c, int prec, int col0, int ncols, t
     TQS_CUDA(cudaMemcpy2DAsync(U, size_t(ldu) * sizeof(float2), S + col0, size_t(N) * sizeof(float2),
                                size_t(ncols) * sizeof(float2), size_t(N), cudaMemcpyDeviceToDevice, s),
              "tqs_circuit_unitary: copy block");
-    return TQS_OK;
-  }
-  if (prec == TQS_PREC_FP32_SIMT) {
-    TQS_CUDA(c->d_chain.ensure(chain_simt_scratch_bytes(c->n, ncols)), "tqs_circuit_unitary: cudaMalloc");
-    TQS_CUDA(chain_simt(c->d_factors.as<StepFactor>(), c->steps.data(), c->nsteps, c->n, col0, ncols,
-                        U, ldu, c->d_chain.p, s),
-             "tqs_circuit_unitary: SIMT chain");
     return TQS_OK;
   }
   TQS_CUDA(c->d_chain.ensure(chain_tc_scratch_bytes(c->n, prec, ncols)), "tqs_circuit_unitary: cudaMalloc");

@@ -637,6 +637,55 @@ struct Image {
   }
 };
 
+// Device copy of one program: its FusedCirc, passes, ops and coefficients, then
+// an int32 0 (the job order of a launch of this one circuit).
+struct ProgramUpload {
+  DevBuf buf;
+  bool valid = false;
+  const Program* prog = nullptr;  // what buf holds, and the initial state its FusedCirc names
+  const void* init = nullptr;
+  cudaEvent_t done = nullptr;  // recorded after the upload, on `stream`
+  cudaStream_t stream = nullptr;
+  ~ProgramUpload() {
+    if (done) cudaEventDestroy(done);
+  }
+  // Make buf hold P with initial state `init` (nullptr: a basis state), in
+  // stream order on s; L's program arrays and job order point into it.
+  tqs_status ensure(const Program& P, const float2* d_init, FusedLaunch& L, cudaStream_t s, const char* who) {
+    const size_t order_off = (sizeof(FusedCirc) + P.passes.size() * sizeof(FusedPass) +
+                              P.ops.size() * sizeof(FusedOp) + P.coef.size() * sizeof(float2) + 255) &
+                             ~size_t(255);
+    if (!valid || prog != &P || init != d_init) {
+      valid = false;
+      Image img;
+      img.add(P, 0);
+      img.circs[0].init = d_init;
+      static const int32_t zero_order[1] = {0};
+      TQS_CUDA(buf.ensure(order_off + 256), who);
+      TQS_CUDA(img.upload(buf.p, s), who);
+      TQS_CUDA(cudaMemcpyAsync(buf.as<char>() + order_off, zero_order, sizeof(int32_t), cudaMemcpyHostToDevice, s),
+               who);
+      if (!done) TQS_CUDA(cudaEventCreateWithFlags(&done, cudaEventDisableTiming), who);
+      TQS_CUDA(cudaEventRecord(done, s), who);
+      stream = s;
+      valid = true;
+      prog = &P;
+      init = d_init;
+    } else if (s != stream) {
+      TQS_CUDA(cudaStreamWaitEvent(s, done, 0), who);  // another stream's kernels wait for the upload
+    }
+    char* p = buf.as<char>();
+    L.circs = reinterpret_cast<const FusedCirc*>(p);
+    L.order = reinterpret_cast<const int32_t*>(p + order_off);
+    p += sizeof(FusedCirc);
+    L.passes = reinterpret_cast<const FusedPass*>(p);
+    p += P.passes.size() * sizeof(FusedPass);
+    L.ops = reinterpret_cast<const FusedOp*>(p);
+    L.coef = reinterpret_cast<const float2*>(p + P.ops.size() * sizeof(FusedOp));
+    return TQS_OK;
+  }
+};
+
 struct tqs_circuit {
   int n = 0;
   int n_instr = 0;  // measure / reset instructions
@@ -673,6 +722,7 @@ struct tqs_circuit {
   Image fsv_img;      // their tile programs
   DevBuf d_fsv;       // device copy of fsv_img
   DevBuf d_sample;    // sampling scratch
+  ProgramUpload cols_prog;  // the unitary's columns: `prog`
   // chain scratch
   DevBuf d_chain;
   DevBuf d_err;

@@ -80,6 +80,7 @@ tqs_status tqs_add_gate(tqs_circuit* c, int gate, const int* qubits, int nq, con
   c->nsteps = std::max(c->nsteps, step + 1);
   c->gates.push_back(g);
   c->prog_valid = false;
+  c->cols_prog.valid = false;
   c->prog_init_valid = false;
   c->uploaded = false;
   c->steps_valid = false;
@@ -157,6 +158,7 @@ tqs_status tqs_add_custom(tqs_circuit* c, const char* name, const int* qubits, i
   c->nsteps = std::max(c->nsteps, g.step + 1);
   c->gates.push_back(g);
   c->prog_valid = false;
+  c->cols_prog.valid = false;
   c->prog_init_valid = false;
   c->uploaded = false;
   c->steps_valid = false;
@@ -414,7 +416,7 @@ tqs_status tqs_check_violations(uint32_t* count, int reset) {
   if (!count) return fail(TQS_ERR_ARG, "tqs_check_violations: count is NULL");
   using Counter = cudaError_t (*)(unsigned int*, bool);
   static const Counter counters[] = {violations_fused,  violations_plain,      violations_probs,
-                                     violations_sample, violations_chain_simt, violations_chain_tc};
+                                     violations_sample, violations_columns, violations_chain_tc};
   uint32_t total = 0;
   for (Counter f : counters) {
     unsigned int v = 0;

@@ -237,9 +237,11 @@ size_t chain_tc_scratch_bytes(int n, int prec, int ncols);
 cudaError_t chain_tc(const StepFactor* d_factors, const StepDesc* steps, int nsteps, int n,
                      int prec, int col0, int ncols, float2* d_U, int64_t ldu, void* scratch,
                      int* d_err, int group, int kchunk, int pair, cudaStream_t s);
-size_t chain_simt_scratch_bytes(int n, int ncols);
-cudaError_t chain_simt(const StepFactor* d_factors, const StepDesc* steps, int nsteps, int n,
-                       int col0, int ncols, float2* d_U, int64_t ldu, void* scratch, cudaStream_t s);
+// FP32 form: the columns as a batch of the circuit's fused program, whose
+// arrays L names (L.circs its descriptor).
+size_t columns_scratch_bytes(int n, int ncols);
+cudaError_t launch_columns(FusedLaunch L, int n, int nint, int col0, int ncols, float2* d_U, int64_t ldu,
+                           void* scratch, int sms, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Probabilities / marginals (FP64).
@@ -332,7 +334,7 @@ cudaError_t violations_fused(unsigned int* count, bool reset);
 cudaError_t violations_plain(unsigned int* count, bool reset);
 cudaError_t violations_probs(unsigned int* count, bool reset);
 cudaError_t violations_sample(unsigned int* count, bool reset);
-cudaError_t violations_chain_simt(unsigned int* count, bool reset);
+cudaError_t violations_columns(unsigned int* count, bool reset);
 cudaError_t violations_chain_tc(unsigned int* count, bool reset);
 
 // Process-wide count of kernel launches enqueued by this library.
