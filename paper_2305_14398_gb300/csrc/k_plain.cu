@@ -15,8 +15,9 @@ namespace {
 constexpr int kMatThreads = 256;
 constexpr int kMaxFactors = 16;
 
+// Small matrices (n < kMatExpandQ): one product over the factors per entry.
 __global__ void __launch_bounds__(kMatThreads)
-    materialize_kernel(const StepFactor* __restrict__ factors, int nf, uint32_t idle, int n,
+    materialize_small_kernel(const StepFactor* __restrict__ factors, int nf, uint32_t idle, int n,
                        float2* __restrict__ S) {
   __shared__ StepFactor fs[kMaxFactors];
   for (int i = threadIdx.x; i < nf * static_cast<int>(sizeof(StepFactor) / 8); i += blockDim.x)
@@ -33,6 +34,130 @@ __global__ void __launch_bounds__(kMatThreads)
     const float2 v0 = step_entry(fs, nf, idle, r, c);
     const float2 v1 = step_entry(fs, nf, idle, r, c + 1);
     __stcs(reinterpret_cast<float4*>(S) + TQS_IX(e, pairs), make_float4(v0.x, v0.y, v1.x, v1.y));
+  }
+}
+
+// Larger matrices.  Per entry the product costs a complex multiply and an
+// entry lookup per factor (n = 12, a layer of 12 single-qubit gates: 196 us,
+// 0.68 TB/s written, bound by instruction issue), but entries of a row share
+// their partial products: a row is expanded qubit by qubit, x(c | b << q) =
+// x(c) f_q(r, c | b << q), where f_q is the entry of the factor whose highest
+// qubit is q (1 where q is a lower qubit of its factor, the delta where it
+// is idle).  The last expansion costs two multiplies per entry (one for each
+// parent), all before it half as much again.  A block of 256 threads works 2^14
+// entries (kRows rows, as many as fill it): every thread forms one product
+// over the lowest n - 6 qubits, expands it by 3 qubits into shared memory, and
+// then expands 8 of those by the top 3 qubits into the matrix, two neighbours
+// at once, so that a warp's store covers 512 contiguous bytes.  Same matrix:
+// 29 us, and n = 14 at 6.9 TB/s, the measured copy rate (n = 12, 13: 4.7, 6.3 TB/s).
+constexpr int kMatExpandQ = 10;  // below, 16 or fewer blocks are slower than the small kernel (9 us against 12)
+constexpr int kMatMid = 2048;  // entries of the 2^(n-3)-entry row parts of a block
+
+// How the expansion by qubit q multiplies: the index of the factor whose
+// highest qubit q is, or one of these.
+constexpr int kLevelIdle = -1, kLevelCopy = -2;
+
+__device__ __noinline__ float2 custom_entry(const StepFactor& f, uint32_t r, uint32_t c) {
+  return factor_entry(f, r, c);
+}
+
+// x: the row's value with the qubits from q on left out (at column bits c);
+// out[i]: with the 3 qubits q, q + 1, q + 2 at the bits of i.
+__device__ __forceinline__ void expand3(const StepFactor* fs, const int* level, int q, uint32_t r, uint32_t c,
+                                        float2 x, float2 (&out)[8]) {
+  out[0] = x;
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    const int k = level[TQS_IX(q + l, 16)];
+    const uint32_t bit = 1u << (q + l);
+    if (k < 0) {
+      const bool one = k == kLevelCopy || (r & bit) != 0, zero = k == kLevelCopy || (r & bit) == 0;
+#pragma unroll
+      for (int i = 0; i < (1 << l); ++i) {
+        out[i | (1 << l)] = one ? out[i] : make_float2(0.f, 0.f);
+        out[i] = zero ? out[i] : make_float2(0.f, 0.f);
+      }
+    } else if (fs[k].custom) {
+#pragma unroll
+      for (int i = 0; i < (1 << l); ++i) {
+        const uint32_t ci = c | (static_cast<uint32_t>(i) << q);
+        out[i | (1 << l)] = step_cmul(out[i], custom_entry(fs[k], r, ci | bit));
+        out[i] = step_cmul(out[i], custom_entry(fs[k], r, ci));
+      }
+    } else if (fs[k].nq == 1) {
+      const float2* m = fs[k].m + ((r & bit) ? 2 : 0);
+      const float2 f0 = m[0], f1 = m[1];
+#pragma unroll
+      for (int i = 0; i < (1 << l); ++i) {
+        out[i | (1 << l)] = step_cmul(out[i], f1);
+        out[i] = step_cmul(out[i], f0);
+      }
+    } else {
+      // the row's entries at this qubit's bit, for both bits of the partner
+      const int q0 = fs[k].q0, q1 = fs[k].q1, part = q0 == q + l ? q1 : q0;
+      const float2* m = fs[k].m + 4 * ((((r >> q0) & 1) << 1) | ((r >> q1) & 1));
+      const int sb = q0 == q + l ? 2 : 1, sp = 3 - sb;
+      const float2 f00 = m[0], f01 = m[sb], f10 = m[sp], f11 = m[3];
+#pragma unroll
+      for (int i = 0; i < (1 << l); ++i) {
+        const bool p = ((c | (static_cast<uint32_t>(i) << q)) >> part) & 1;
+        const float2 f0 = make_float2(p ? f10.x : f00.x, p ? f10.y : f00.y);
+        const float2 f1 = make_float2(p ? f11.x : f01.x, p ? f11.y : f01.y);
+        out[i | (1 << l)] = step_cmul(out[i], f1);
+        out[i] = step_cmul(out[i], f0);
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kMatThreads)
+    materialize_kernel(const StepFactor* __restrict__ factors, int nf, uint32_t idle, int n,
+                       float2* __restrict__ S) {
+  __shared__ StepFactor fs[kMaxFactors];
+  __shared__ int level[16];
+  __shared__ float2 mid[kMatMid];
+  const int t = threadIdx.x;
+  for (int i = t; i < nf * static_cast<int>(sizeof(StepFactor) / 8); i += blockDim.x)
+    reinterpret_cast<float2*>(fs)[TQS_IX(i, int(sizeof(fs) / 8))] =
+        reinterpret_cast<const float2*>(factors)[i];
+  if (t < 16) level[t] = ((idle >> t) & 1) ? kLevelIdle : kLevelCopy;
+  __syncthreads();
+  if (t < nf) level[31 - __clz(factor_qubits(fs[t]))] = t;
+  __syncthreads();
+  // 2^rq rows of 2^(n-3) mid entries in the block, from row r0
+  const int mq = n - 3, rq = 11 - mq;
+  const uint32_t r0 = blockIdx.x << rq;
+  {
+    // one product over the lowest n - 6 qubits, expanded by the next 3
+    const int lq = n - 6;
+    const uint32_t row = static_cast<uint32_t>(t) >> lq, c = static_cast<uint32_t>(t) & ((1u << lq) - 1);
+    const uint32_t r = r0 + row;
+    float2 x = make_float2(((r ^ c) & idle & ((1u << lq) - 1)) ? 0.f : 1.f, 0.f);
+    for (int q = 0; q < lq; ++q)
+      if (level[q] >= 0) x = step_cmul(x, custom_entry(fs[level[q]], r, c));
+    float2 o[8];
+    expand3(fs, level, lq, r, c, x, o);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      mid[TQS_IX((row << mq) | (static_cast<uint32_t>(i) << lq) | c, kMatMid)] = o[i];
+  }
+  __syncthreads();
+  const size_t NN = size_t(1) << (2 * n);
+#pragma unroll 1
+  for (int e = t; e < kMatMid / 2; e += kMatThreads) {
+    const uint32_t row = static_cast<uint32_t>(2 * e) >> mq, c = static_cast<uint32_t>(2 * e) & ((1u << mq) - 1);
+    const uint32_t r = r0 + row;
+    const float4 m = reinterpret_cast<const float4*>(mid)[TQS_IX(e, kMatMid / 2)];
+    float2 a[8], b[8];
+    expand3(fs, level, mq, r, c, make_float2(m.x, m.y), a);
+    expand3(fs, level, mq, r, c + 1, make_float2(m.z, m.w), b);
+    float2* out = S + (static_cast<size_t>(r) << n) + c;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      (void)TQS_IX((static_cast<size_t>(r) << n) + c + (static_cast<size_t>(i) << mq) + 1, NN);
+      __stcs(reinterpret_cast<float4*>(out + (static_cast<size_t>(i) << mq)),
+             make_float4(a[i].x, a[i].y, b[i].x, b[i].y));
+    }
   }
 }
 
@@ -91,13 +216,19 @@ int sm_count() {
 cudaError_t launch_materialize(const StepFactor* d_factors, StepDesc step, int n, float2* d_S,
                                cudaStream_t s) {
   if (step.f_count > kMaxFactors) return cudaErrorInvalidValue;
+  if (n >= kMatExpandQ) {
+    materialize_kernel<<<1 << (2 * n - 14), kMatThreads, 0, s>>>(d_factors + step.f_begin, step.f_count,
+                                                                 step.idle, n, d_S);
+    count_launches(1);
+    return cudaGetLastError();
+  }
   const int64_t N = int64_t(1) << n;
   const int64_t pairs = (N * N) >> 1;
   int64_t blocks = (pairs + kMatThreads - 1) / kMatThreads;
   const int64_t cap = int64_t(sm_count()) * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
-  materialize_kernel<<<static_cast<int>(blocks), kMatThreads, 0, s>>>(
+  materialize_small_kernel<<<static_cast<int>(blocks), kMatThreads, 0, s>>>(
       d_factors + step.f_begin, step.f_count, step.idle, n, d_S);
   count_launches(1);
   return cudaGetLastError();
