@@ -65,6 +65,43 @@ TQS_HD uint64_t sq_f32_as_f64_bits_general(uint32_t xbits) {
   return (static_cast<uint64_t>(E + 1023) << 52) | frac;
 }
 
+// The FP64 bits of x^2 + y^2 correctly rounded (round to nearest, ties to
+// even: the FP64 sum of the exact squares above), integers only.  The larger
+// square, m^2 < 2^48 for the 24-bit significand m, is placed with its low bit
+// at bit 15 of a 64-bit sum, the other aligned to it (what falls below bit 0
+// only matters as "something": it is or-ed into bit 0, which is below the
+// rounding position), and the sum, in [2^61, 2^64), is rounded to 53 bits.
+TQS_HD uint64_t sq_sum_bits(uint32_t xbits, uint32_t ybits) {
+  const uint32_t ax = xbits & 0x7fffffffu, ay = ybits & 0x7fffffffu;
+  const uint32_t hi = ax > ay ? ax : ay, lo = ax > ay ? ay : ax;
+  if (hi < 0x00800000u) {
+    // both zero or subnormal: m < 2^23 at 2^-149 each, the sum is exact
+    const uint64_t s = static_cast<uint64_t>(hi) * hi + static_cast<uint64_t>(lo) * lo;
+    if (s == 0) return 0;
+    const uint32_t sh = static_cast<uint32_t>(s >> 32);
+    const int lz = sh ? clz32(sh) : 32 + clz32(static_cast<uint32_t>(s));
+    return (static_cast<uint64_t>(1023 - 298 + 62 - lz) << 52) + (s << (lz - 11));
+  }
+  const int eh = static_cast<int>(hi >> 23);
+  const bool sub = lo < 0x00800000u;
+  const int el = sub ? 1 : static_cast<int>(lo >> 23);
+  const uint32_t mh = (hi & 0x7fffffu) | 0x800000u, ml = (lo & 0x7fffffu) | (sub ? 0u : 0x800000u);
+  const uint64_t B = static_cast<uint64_t>(ml) * ml;
+  const int r = 2 * (eh - el) - 15;  // bits B moves right
+  uint64_t b;
+  if (r <= 0) {
+    b = B << -r;
+  } else {
+    b = r < 63 ? B >> r : 0;
+    b |= (r < 63 ? (b << r) != B : B != 0) ? 1 : 0;
+  }
+  const uint64_t s = ((static_cast<uint64_t>(mh) * mh) << 15) + b;
+  const uint32_t top = static_cast<uint32_t>(s >> 32);
+  const int k = 9 + (top >= 0x40000000u ? 1 : 0) + (top >= 0x80000000u ? 1 : 0);  // bits rounded off
+  const uint64_t q = (s + ((uint64_t(1) << (k - 1)) - 1) + ((s >> k) & 1)) >> k;
+  return (static_cast<uint64_t>(2 * eh + 759 + k) << 52) + q;
+}
+
 #if defined(__CUDACC__)
 // |x + iy|^2 correctly rounded to FP64 (bit-identical to (double)x * x +
 // (double)y * y): the two squares are exact FP64 values built with integer

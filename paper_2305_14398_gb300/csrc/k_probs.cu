@@ -1,15 +1,20 @@
 // Probabilities and their FP64 sum (sm_103a).
 //
 // p_i = |psi_i|^2 (Sec. 2.1, eq. 2) correctly rounded to FP64 from the FP32
-// parts (their squares are exact FP64 values, built with integer operations:
-// GB300 runs FP64 arithmetic at about 1/64 of its FP32 rate, so each
-// probability costs one FP64 add instead of two widenings, a multiply and a
-// fused multiply-add), optionally written out, and summed over the
+// parts, optionally written out, and summed over the
 // indices i with (i & zero_mask) == 0 (zero_mask = 0: the norm; otherwise the
 // marginal probability that the masked qubits read 0, as for the
 // Deutsch-Jozsa input register of Sec. 2.5).  The reduction runs in a fixed
 // order: per-block partial sums into scratch, then one warp sums the
 // partials, so the result does not depend on scheduling.
+//
+// GB300 runs FP64 arithmetic at about 1/64 of its FP32 rate.  The squares, their
+// sum and its rounding are therefore integer operations (sq_sum_bits) and the
+// FP64 pipe only adds the running sum, one operation per amplitude: with two
+// (the squares added in FP64) a 2^24 state was bound by that pipe, 88 us, now 59
+// us; four loads in flight per thread give 10 of these.  2^25 amplitudes move
+// at 5.3 TB/s, 78 % of the copy rate; bound by instruction issue (71
+// instructions per amplitude, 62 % of the issue slots).
 #include <mutex>
 
 #include "../../include/tqs.h"
@@ -23,6 +28,12 @@ namespace {
 constexpr int kProbThreads = 256;
 constexpr int64_t kAmpsPerBlock = 8192;
 constexpr int kMaxPartials = 1024;
+constexpr int kProbUnroll = 4;
+
+// |x + iy|^2 rounded to FP64, by integer operations.
+__device__ __forceinline__ double sq_sum_int(float x, float y) {
+  return __longlong_as_double(static_cast<long long>(sq_sum_bits(__float_as_uint(x), __float_as_uint(y))));
+}
 
 __global__ void __launch_bounds__(kProbThreads)
     probs_kernel(const float2* __restrict__ st, int64_t N, int64_t chunk, double* __restrict__ probs,
@@ -31,14 +42,26 @@ __global__ void __launch_bounds__(kProbThreads)
   int64_t end = begin + chunk;
   if (end > N) end = N;
   double acc = 0.0;
-  for (int64_t i = begin + 2 * threadIdx.x; i < end; i += 2 * kProbThreads) {
-    const float4 v = __ldcs(reinterpret_cast<const float4*>(st) + TQS_IX(i >> 1, N >> 1));
-    const double q0 = sq_sum_f64(v.x, v.y);
-    const double q1 = sq_sum_f64(v.z, v.w);
+  auto load = [&](int64_t i) {
+    return __ldcs(reinterpret_cast<const float4*>(st) + TQS_IX(i >> 1, N >> 1));
+  };
+  auto one = [&](int64_t i, float4 v) {
+    const double q0 = sq_sum_int(v.x, v.y), q1 = sq_sum_int(v.z, v.w);
     if (probs) __stcs(reinterpret_cast<double2*>(probs) + TQS_IX(i >> 1, N >> 1), make_double2(q0, q1));
     if ((static_cast<uint64_t>(i) & zero_mask) == 0) acc += q0;
     if ((static_cast<uint64_t>(i + 1) & zero_mask) == 0) acc += q1;
+  };
+  // kProbUnroll loads in flight per thread
+  constexpr int64_t stride = 2 * kProbThreads;
+  int64_t i = begin + 2 * threadIdx.x;
+  for (; i + (kProbUnroll - 1) * stride < end; i += kProbUnroll * stride) {
+    float4 v[kProbUnroll];
+#pragma unroll
+    for (int k = 0; k < kProbUnroll; ++k) v[k] = load(i + k * stride);
+#pragma unroll
+    for (int k = 0; k < kProbUnroll; ++k) one(i + k * stride, v[k]);
   }
+  for (; i < end; i += stride) one(i, load(i));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   __shared__ double red[kProbThreads / 32];
@@ -55,7 +78,15 @@ __global__ void __launch_bounds__(kProbThreads)
 __global__ void sum_partials_kernel(const double* __restrict__ partials, int count,
                                     double* __restrict__ out) {
   double acc = 0.0;
-  for (int i = threadIdx.x; i < count; i += 32) acc += partials[i];
+  // every load in flight before the first add
+  double p[kMaxPartials / 32];
+#pragma unroll
+  for (int k = 0; k < kMaxPartials / 32; ++k) {
+    const int i = threadIdx.x + 32 * k;
+    p[k] = i < count ? partials[i] : 0.0;
+  }
+#pragma unroll
+  for (int k = 0; k < kMaxPartials / 32; ++k) acc += p[k];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (threadIdx.x == 0) *out = acc;
