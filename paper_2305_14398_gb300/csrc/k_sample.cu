@@ -27,10 +27,10 @@
 // absolute), and a shot is one multiply, binary searches that compare the FP64
 // bit patterns as integers (the order of non-negative doubles), and at most 8
 // adds; the shared-memory path needs one FP64 multiply per shot and nothing else.
-// Two paths share that arithmetic: segments of up to 2^13 entries are staged
-// in shared memory by one CTA each, which builds the tables there and runs
-// every shot of the segment; larger segments use three kernels over global
-// memory (block tables, block prefix, shots).
+// Two paths: segments of up to 2^13 entries are read by one CTA each, which
+// builds exact tables in shared memory and runs every shot of the segment
+// there; larger segments use three kernels over global memory (block tables,
+// block prefix, shots).
 #include "checked.h"
 #include "tqs_internal.h"
 
@@ -42,15 +42,11 @@ constexpr int kThreads = 256;
 constexpr int kChunks = kSampleBlk / kSampleChunk;  // 32: one per lane
 static_assert(kChunks == 32, "one chunk per lane");
 
-// Values of the cumulative sums: FP64 (the global path) or unsigned 64-bit
-// fixed point (the shared-memory path); le: a <= b (for non-negative FP64, the
-// order of the bit patterns); pos: the value is above 0.
+// Non-negative FP64 values compared by their bit patterns (the same order).
 __device__ __forceinline__ bool le_val(double a, double b) {
   return __double_as_longlong(a) <= __double_as_longlong(b);
 }
-__device__ __forceinline__ bool le_val(unsigned long long a, unsigned long long b) { return a <= b; }
 __device__ __forceinline__ bool pos_val(double a) { return __double_as_longlong(a) > 0; }
-__device__ __forceinline__ bool pos_val(unsigned long long a) { return a > 0; }
 
 template <class V>
 __device__ __forceinline__ V warp_incl_scan(V x, int lane) {
@@ -239,35 +235,80 @@ __device__ __forceinline__ unsigned long long to_fixed(unsigned long long bits, 
   return m >> (-sh);
 }
 
+//
+// A thread owns K consecutive chunks in registers: it loads them (64 bytes a
+// chunk), converts them once S is known, and the chunk bases come from one
+// scan over the threads, so the entries cross shared memory once (written,
+// 9 words to a chunk of 8 so that neither the 64-bit stores nor a shot's
+// reads collide) and the block meets at three barriers.  With the entries
+// staged first, converted in place and summed in strides of 8 (16-way bank
+// conflicts), 16384 states of 2^11 entries and 64 shots took 158 us; now
+// 96 us (2.8 TB/s read), 16000 states of 2^5 and 10 shots 47 us, now 14 us.
+constexpr int kChunkPad = kSampleChunk + 1;
+
+// The last chunk whose base is at most the target, then the entry in it.
+__device__ __forceinline__ int64_t sample_shot_smem(const unsigned long long* e, int len,
+                                                    const unsigned long long* cb, int nc, unsigned long long T,
+                                                    unsigned long long target) {
+  auto entry = [&](int i) {
+    return e[TQS_IX((i >> 3) * kChunkPad + (i & 7), nc * kChunkPad)];
+  };
+  int i = len - 1;  // target >= T: the last entry above 0
+  if (target < T) {
+    int lo = 0, hi = nc - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (cb[TQS_IX(mid, nc)] <= target) lo = mid; else hi = mid - 1;
+    }
+    unsigned long long c = cb[lo];
+    const int i0 = lo * kSampleChunk;
+#pragma unroll
+    for (int j = 0; j < kSampleChunk; ++j) {
+      const unsigned long long x = entry(i0 + j);  // 0 past len
+      c += x;
+      if (x > 0 && c > target) return i0 + j;
+    }
+    i = min(i0 + kSampleChunk, len) - 1;
+  }
+  for (; i >= 0; --i)
+    if (entry(i) > 0) return i;
+  return -1;
+}
+
+template <int K>
 __global__ void __launch_bounds__(kThreads)
     segment_smem_kernel(const SampleLaunch L) {
   using U = unsigned long long;
   extern __shared__ U sm[];
-  __shared__ U wtot[kThreads / 32], wpre[kThreads / 32];
-  __shared__ U s_tot;
+  __shared__ U wtot[kThreads / 32];
   __shared__ int s_emax[kThreads / 32];
   __shared__ float s_fsum[kThreads / 32];
-  constexpr int kMaxBlocks = 1 << (kSampleSmemMaxQ - 8);
-  __shared__ U sbs[kMaxBlocks], sbp[kMaxBlocks];
   const SampleSeg sg = L.ssegs[TQS_IX(blockIdx.x, L.n_sseg)];
-  const int64_t len = int64_t(1) << sg.n;
-  const int64_t nb = sample_blocks(sg.n);
-  U* sp = sm;
-  U* scp = sm + (size_t(1) << L.smem_q);
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int64_t qlen = int64_t(1) << L.smem_q;
-  const int64_t nchunks = (qlen < kSampleBlk ? kSampleBlk : qlen) / kSampleChunk;
+  const int len = 1 << sg.n;
+  const int nc = (len + kSampleChunk - 1) / kSampleChunk;  // chunks of this segment
+  U* e = sm;
+  U* cb = sm + nc * kChunkPad;
+  const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, nw = T >> 5;
+  const int c0 = t * K;  // this thread's chunks: c0 .. c0 + K - 1
   (void)TQS_IX(sg.p_off + len - 1, L.probs_len);
-  // the probabilities' bits into shared memory, and their largest exponent
+  const double* ub = L.u + sg.index * L.shots;
+  double u = t < L.shots ? __ldcs(ub + t) : 0.0;
+  // the probabilities' bits, their largest exponent and an estimate of their sum
   const ulonglong2* gp = reinterpret_cast<const ulonglong2*>(L.probs + sg.p_off);
+  U v[K * kSampleChunk];
   int emax = 0;
   float fsum = 0.f;
-  for (int64_t i = t; i < len / 2; i += kThreads) {
-    const ulonglong2 v = __ldcs(gp + i);
-    sp[TQS_IX(2 * i, qlen)] = v.x;
-    sp[TQS_IX(2 * i + 1, qlen)] = v.y;
-    emax = max(emax, max(static_cast<int>((v.x >> 52) & 0x7FF), static_cast<int>((v.y >> 52) & 0x7FF)));
-    fsum += approx_f32(v.x) + approx_f32(v.y);
+#pragma unroll
+  for (int j = 0; j < K * kSampleChunk / 2; ++j) {
+    const int i = c0 * kSampleChunk + 2 * j;
+    const ulonglong2 x = i < len ? __ldg(gp + (i >> 1)) : make_ulonglong2(0, 0);
+    v[2 * j] = x.x;
+    v[2 * j + 1] = x.y;
+  }
+#pragma unroll
+  for (int j = 0; j < K * kSampleChunk; ++j) {
+    emax = max(emax, static_cast<int>((v[j] >> 52) & 0x7FF));
+    fsum += approx_f32(v[j]);
   }
   emax = __reduce_max_sync(kFull, emax);
 #pragma unroll
@@ -279,8 +320,7 @@ __global__ void __launch_bounds__(kThreads)
   __syncthreads();
   emax = 0;
   fsum = 0.f;
-#pragma unroll
-  for (int w = 0; w < kThreads / 32; ++w) {
+  for (int w = 0; w < nw; ++w) {
     emax = max(emax, s_emax[w]);
     fsum += s_fsum[w];
   }
@@ -289,26 +329,40 @@ __global__ void __launch_bounds__(kThreads)
   // exponent instead: every p < 2^(emax - 1022), 2^n of them below 2^62
   const int ET = (__float_as_int(fsum) >> 23) - 127;
   const int S = (fsum > 0.f && fsum < 3.0e38f) ? 60 - ET : 62 - sg.n - (max(emax, 1) - 1022);
-  for (int64_t i = t; i < len; i += kThreads) sp[TQS_IX(i, qlen)] = to_fixed(sp[TQS_IX(i, qlen)], S);
+  U own = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+#pragma unroll
+    for (int j = 0; j < kSampleChunk; ++j) {
+      const U x = to_fixed(v[k * kSampleChunk + j], S);
+      own += x;
+      v[k * kSampleChunk + j] = x;
+      if (c0 + k < nc) e[TQS_IX((c0 + k) * kChunkPad + j, nc * kChunkPad)] = x;
+    }
+  // chunk bases: exclusive scan of the threads' sums (exact, so in any order)
+  const U incl = warp_incl_scan(own, lane);
+  if (lane == 31) wtot[warp] = incl;
   __syncthreads();
-  for (int64_t b = warp; b < nb; b += kThreads / 32) {
-    const U bt = block_tables(sp, len, b, lane, scp + TQS_IX(b * kChunks + lane, nchunks) - lane);
-    if (lane == 0) sbs[TQS_IX(b, kMaxBlocks)] = bt;
+  U base = incl - own, total = 0;
+  for (int w = 0; w < nw; ++w) {
+    if (w < warp) base += wtot[w];
+    total += wtot[w];
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    if (c0 + k < nc) cb[TQS_IX(c0 + k, nc)] = base;
+#pragma unroll
+    for (int j = 0; j < kSampleChunk; ++j) base += v[k * kSampleChunk + j];
   }
   __syncthreads();
-  (void)TQS_IX(nb - 1, kMaxBlocks);
-  block_prefix_cta(sbs, sbp, nb, &s_tot, wtot, wpre);
-  __syncthreads();
-  absolute_chunks(sbp, scp, nb);
-  __syncthreads();
-  const U T = s_tot;
-  const double Tf = static_cast<double>(T);
-  for (int64_t k = t; k < L.shots; k += kThreads) {
+  const double Tf = static_cast<double>(total);
+  for (int64_t k = t; k < L.shots; k += T) {
+    if (k != t) u = __ldcs(ub + k);
     const int64_t kk = TQS_IX(sg.index * L.shots + k, L.n_segs * L.shots);
     // floor(u T); u < 1 keeps it below T up to the rounding of the product
-    const double x = __ldcs(L.u + kk) * Tf;
-    const U target = x >= Tf ? T : static_cast<U>(x);
-    L.out[kk] = sample_shot(sp, len, sbp, scp, nb, T, target);
+    const double x = u * Tf;
+    const U target = x >= Tf ? total : static_cast<U>(x);
+    L.out[kk] = sample_shot_smem(e, len, cb, nc, total, target);
   }
 }
 
@@ -341,13 +395,21 @@ cudaError_t launch_sample(const SampleLaunch& L, cudaStream_t s) {
     }
   }
   if (L.n_sseg > 0 && L.shots > 0) {
-    const size_t q = size_t(1) << L.smem_q;
-    const size_t chunks = (q < kSampleBlk ? kSampleBlk : q) / kSampleChunk;
-    const int smem = static_cast<int>((q + chunks) * sizeof(double));
-    cudaError_t e = cudaFuncSetAttribute(segment_smem_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // a thread per chunk of the largest segment, or per shot where there are
+    // more, up to kThreads; from 2^12 entries on two or four chunks a thread
+    const int nc = L.smem_q > 3 ? 1 << (L.smem_q - 3) : 1;
+    int threads = 32;
+    while (threads < kThreads && (threads < nc || threads < L.shots)) threads *= 2;
+    const int smem = nc * (kChunkPad + 1) * static_cast<int>(sizeof(double));
+    auto launch = [&](auto kernel) -> cudaError_t {
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e == cudaSuccess) kernel<<<L.n_sseg, threads, smem, s>>>(L);
+      return e;
+    };
+    const cudaError_t e = nc <= threads       ? launch(segment_smem_kernel<1>)
+                          : nc <= 2 * threads ? launch(segment_smem_kernel<2>)
+                                              : launch(segment_smem_kernel<4>);
     if (e != cudaSuccess) return e;
-    segment_smem_kernel<<<L.n_sseg, kThreads, smem, s>>>(L);
     ++k;
   }
   count_launches(k);
