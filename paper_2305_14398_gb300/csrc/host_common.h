@@ -697,14 +697,7 @@ struct tqs_circuit {
   Program prog;       // for the input |0...0> (leading X gates folded)
   bool prog_init_valid = false;
   Program prog_init;  // for a given input state (nothing folded)
-  DevBuf d_prog;      // FusedCirc + passes + ops
-  // what d_prog holds: the program (prog or prog_init) and the initial-state
-  // pointer it was uploaded with (valid while `uploaded`)
-  bool uploaded = false;
-  const void* uploaded_prog = nullptr;
-  const void* uploaded_init = nullptr;
-  cudaEvent_t upload_done = nullptr;  // recorded after the upload, on upload_stream
-  cudaStream_t upload_stream = nullptr;
+  ProgramUpload run_prog;  // `prog`, or `prog_init` with its initial-state pointer
   DevBuf d_counter;   // job counter
   DevBuf d_gscratch;  // TEAM_GLOBAL slot
   // cached plain-form step table
@@ -726,9 +719,6 @@ struct tqs_circuit {
   // chain scratch
   DevBuf d_chain;
   DevBuf d_err;
-  ~tqs_circuit() {
-    if (upload_done) cudaEventDestroy(upload_done);
-  }
 };
 
 // ---------------------------------------------- shared helpers of the entry points

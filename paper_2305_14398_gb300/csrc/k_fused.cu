@@ -729,7 +729,7 @@ __device__ __noinline__ void wide_pass(const FusedLaunch& L, int nint, int k, ui
 template <int TEAM>
 __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, int size,
                             double* s_red, int& next_job, int& next_ci, int* s_slot,
-                            GridBar* bar = nullptr) {
+                            GridBar* bar = nullptr, float* blk_sum = nullptr) {
   const FusedCirc cd = L.circs[ci];
   const int nint = cd.nint;
   const int n = cd.n;
@@ -827,6 +827,15 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
   }
   if (TEAM == TEAM_WARP || TEAM == TEAM_PAIR)
     next_ci = next_job < L.n_jobs ? __ldg(L.order + next_job) : 0;
+  // TEAM_SOLO: the CTA's threads as norm_width lanes times several workers, each
+  // with its own blocks of a lane's pairs.
+  int blk0 = 0, blk_step = 8;
+  if (TEAM == TEAM_SOLO) {
+    blk0 = rank / L.norm_width * 8;
+    blk_step = size / L.norm_width * 8;
+    rank &= L.norm_width - 1;
+    size = L.norm_width;
+  }
   // Output: logical index i holds the amplitude at physical index P(i) =
   // col_off ^ lin(i) (the output map), whose shared-memory slot is A(i) =
   // swz(P(i)).  lin and swz are linear over GF(2), so A(i) is swz(col_off)
@@ -855,7 +864,7 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
       const int iters = N > (1 << sh) ? (N >> sh) : 1;  // pairs per thread
       const int NI = 1 << nint;
 #pragma unroll 1
-      for (int blk = 0; blk < iters; blk += 8) {
+      for (int blk = TEAM == TEAM_SOLO ? blk0 : 0; blk < iters; blk += TEAM == TEAM_SOLO ? blk_step : 8) {
         // A at the block's first pair: the block index's bits sh + 3 ...
         int ab = a_i0;
         for (int q = 3; (blk >> q) != 0; ++q)
@@ -887,15 +896,24 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
           }
         }
         // the block's 16 values summed as a tree in FP32, then added in FP64
-        acc += static_cast<double>(((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7])));
+        const float bs = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+        if (TEAM == TEAM_SOLO) blk_sum[(blk >> 3) * size + rank] = bs;
+        else acc += static_cast<double>(bs);
       }
     }
+  }
+  if (TEAM == TEAM_SOLO) {
+    // lane by lane, the blocks in order; the first norm_width threads go on
+    __syncthreads();
+    if (static_cast<int>(threadIdx.x) < size && 2 * rank < N)
+      for (int b = 0; 8 * b < max(1, N / (2 * size)); ++b) acc += static_cast<double>(blk_sum[b * size + rank]);
+    rank = threadIdx.x;
   }
   // Fixed-order reduction (deterministic): per-thread FP64 partials, warp
   // butterfly, then the warps of the team in order.
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (TEAM == TEAM_WARP) {
+  if (TEAM == TEAM_WARP || (TEAM == TEAM_SOLO && size == 32)) {
     if (rank == 0 && L.norms) L.norms[ci] = acc;
   } else {
     const int warp = rank >> 5, lane = rank & 31;
@@ -914,8 +932,12 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
   team_sync<TEAM>();
 }
 
+// TEAM_SOLO: sums of 8 pairs of amplitudes, 2^kWarpMaxQ amplitudes at most
+// (and at least one per lane of the 64).
+constexpr int kSoloSums = (1 << kWarpMaxQ) / 16;
+
 template <int TEAM>
-__global__ void __launch_bounds__(TEAM == TEAM_CTA ? kCtaThreads : 512)
+__global__ void __launch_bounds__(TEAM == TEAM_SOLO ? kSoloThreads : TEAM == TEAM_CTA ? kCtaThreads : 512)
     fused_kernel(const __grid_constant__ FusedLaunch L) {
   extern __shared__ float4 smem_raw[];
   float2* smem = reinterpret_cast<float2*>(smem_raw);
@@ -952,6 +974,12 @@ __global__ void __launch_bounds__(TEAM == TEAM_CTA ? kCtaThreads : 512)
       job = next_job;
       ci = next_ci;
     }
+  } else if (TEAM == TEAM_SOLO) {
+    __shared__ double s_red[32];
+    __shared__ float blk_sum[kSoloSums];
+    int unused_job = 0, unused_ci = 0;
+    run_circuit<TEAM_SOLO>(L, 0, smem, threadIdx.x, blockDim.x, s_red, unused_job, unused_ci, nullptr, nullptr,
+                           blk_sum);
   } else if (TEAM == TEAM_MULTI) {
     __shared__ double s_red[32];
     const int K = L.ctas_per_job;
@@ -1084,12 +1112,12 @@ __global__ void __launch_bounds__(kFsvThreads)
 size_t fused_smem_bytes(int team, int warps_per_cta, int slice_q) {
   if (team == TEAM_WARP) return (static_cast<size_t>(warps_per_cta) << slice_q) * sizeof(float2);
   if (team == TEAM_PAIR) return (static_cast<size_t>(warps_per_cta / 2) << slice_q) * sizeof(float2);
-  if (team == TEAM_CTA) return (static_cast<size_t>(1) << slice_q) * sizeof(float2);
+  if (team == TEAM_CTA || team == TEAM_SOLO) return (static_cast<size_t>(1) << slice_q) * sizeof(float2);
   return 0;
 }
 
 int fused_threads(int team, int warps_per_cta) {
-  if (team == TEAM_WARP || team == TEAM_PAIR) return 32 * warps_per_cta;
+  if (team == TEAM_WARP || team == TEAM_PAIR || team == TEAM_SOLO) return 32 * warps_per_cta;
   if (team == TEAM_CTA) return warps_per_cta > 0 ? 32 * warps_per_cta : kCtaThreads;
   return kGlobalThreads;
 }
@@ -1168,6 +1196,8 @@ cudaError_t launch_fused(const FusedLaunch& L, cudaStream_t s) {
                              static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     fused_kernel<TEAM_CTA><<<L.grid, threads, smem, s>>>(L);
+  } else if (L.team == TEAM_SOLO) {
+    fused_kernel<TEAM_SOLO><<<1, threads, smem, s>>>(L);
   } else if (L.team == TEAM_MULTI) {
     // cooperative: the CTAs wait on one another at the grid barriers
     FusedLaunch arg = L;

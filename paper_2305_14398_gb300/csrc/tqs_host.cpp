@@ -82,7 +82,7 @@ tqs_status tqs_add_gate(tqs_circuit* c, int gate, const int* qubits, int nq, con
   c->prog_valid = false;
   c->cols_prog.valid = false;
   c->prog_init_valid = false;
-  c->uploaded = false;
+  c->run_prog.valid = false;
   c->steps_valid = false;
   c->fsv_valid = false;
   return TQS_OK;
@@ -160,7 +160,7 @@ tqs_status tqs_add_custom(tqs_circuit* c, const char* name, const int* qubits, i
   c->prog_valid = false;
   c->cols_prog.valid = false;
   c->prog_init_valid = false;
-  c->uploaded = false;
+  c->run_prog.valid = false;
   c->steps_valid = false;
   c->fsv_valid = false;
   return TQS_OK;
@@ -226,47 +226,32 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const Program& P = ensure_program(c, d_init != nullptr);
   const int team = team_for(P.nint);
-  Image img;
-  img.add(P, 0);
-  img.circs[0].init = reinterpret_cast<const float2*>(d_init);
-  const size_t order_off = (img.bytes() + 255) & ~size_t(255);
   // The device program is uploaded once per (program, initial-state pointer)
   // and reused by later calls on the circuit.
-  if (!c->uploaded || c->uploaded_prog != &P || c->uploaded_init != d_init) {
-    c->uploaded = false;
-    TQS_CUDA(c->d_prog.ensure(order_off + 256), "tqs_simulate: cudaMalloc program");
-    TQS_CUDA(img.upload(c->d_prog.p, s), "tqs_simulate: upload program");
-    // order[0] = 0 lives right after the image
-    static const int32_t zero_order[1] = {0};
-    TQS_CUDA(cudaMemcpyAsync(c->d_prog.as<char>() + order_off, zero_order, sizeof(int32_t),
-                             cudaMemcpyHostToDevice, s),
-             "tqs_simulate: upload order");
-    if (!c->upload_done)
-      TQS_CUDA(cudaEventCreateWithFlags(&c->upload_done, cudaEventDisableTiming),
-               "tqs_simulate: event");
-    TQS_CUDA(cudaEventRecord(c->upload_done, s), "tqs_simulate: event");
-    c->upload_stream = s;
-    c->uploaded = true;
-    c->uploaded_prog = &P;
-    c->uploaded_init = d_init;
-  } else if (s != c->upload_stream) {
-    // another stream reuses the program: its kernels wait for the upload
-    TQS_CUDA(cudaStreamWaitEvent(s, c->upload_done, 0), "tqs_simulate: wait upload");
-  }
-  TQS_CUDA(c->d_counter.ensure(2 * sizeof(int32_t)), "tqs_simulate: cudaMalloc counter");
-  char* base = c->d_prog.as<char>();
-  TQS_CUDA(cudaMemsetAsync(c->d_counter.p, 0, 2 * sizeof(int32_t), s), "tqs_simulate: memset");
   FusedLaunch L{};
-  img.point(L, base);
-  L.order = reinterpret_cast<const int32_t*>(base + order_off);
+  tqs_status st = c->run_prog.ensure(P, reinterpret_cast<const float2*>(d_init), L, s,
+                                     "tqs_simulate: upload program");
+  if (st != TQS_OK) return st;
   L.n_jobs = 1;
-  L.counter = c->d_counter.as<int32_t>();
   L.out = reinterpret_cast<float2*>(d_out);
   L.probs = d_probs;
   L.exact_probs = g_exact_probs.load();
   L.norms = d_norm;
   L.uniforms = d_u;
   L.outcomes = d_outcomes;
+  L.grid = 1;
+  if (team == TEAM_WARP && P.n_instr == 0 && P.coef.empty()) {
+    // alone on the GPU: a thread per group instead of a warp for all
+    L.team = TEAM_SOLO;
+    L.slice_q = P.nint;
+    L.norm_width = 32 * g_team_warps_for_q[P.nint].load();
+    L.warps_per_cta = std::max(L.norm_width, std::min(kSoloThreads, 1 << (P.nint - 4))) / 32;
+    TQS_CUDA(launch_fused(L, s), "tqs_simulate: launch");
+    return TQS_OK;
+  }
+  TQS_CUDA(c->d_counter.ensure(2 * sizeof(int32_t)), "tqs_simulate: cudaMalloc counter");
+  TQS_CUDA(cudaMemsetAsync(c->d_counter.p, 0, 2 * sizeof(int32_t), s), "tqs_simulate: memset");
+  L.counter = c->d_counter.as<int32_t>();
   LaunchPlan lp = plan_for(team, P.nint, 1, 1);
   if (team == TEAM_GLOBAL) {
     TQS_CUDA(c->d_gscratch.ensure((size_t(1) << kGlobalSlotQ) * sizeof(float2)),
@@ -276,7 +261,6 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
   L.team = lp.team;
   L.warps_per_cta = lp.warps;
   L.slice_q = lp.slice_q;
-  L.grid = 1;
   // A single circuit of the global class runs on several CTAs (TEAM_MULTI,
   // bitwise the same results) when it has no instructions or custom unitaries.
   const int multi = multi_ctas_for(P);

@@ -134,7 +134,13 @@ static_assert(sizeof(FusedPass) == 16, "FusedPass layout");
 // the outputs with exactly the TEAM_GLOBAL output phase, so results are
 // bitwise those of TEAM_GLOBAL.  Circuits without instructions or custom
 // unitaries, few enough that all their CTAs are resident at once.
-enum TeamKind : int32_t { TEAM_WARP = 0, TEAM_CTA = 1, TEAM_GLOBAL = 2, TEAM_PAIR = 3, TEAM_MULTI = 4 };
+// TEAM_SOLO: one circuit of the warp class alone on the GPU, a CTA with a
+// thread per group of a pass (up to 128).  It writes the outputs block by block
+// as the warps of a warp team (or pair) would, so they and the norm are
+// bitwise the same.  Circuits without instructions or custom unitaries.
+enum TeamKind : int32_t {
+  TEAM_WARP = 0, TEAM_CTA = 1, TEAM_GLOBAL = 2, TEAM_PAIR = 3, TEAM_MULTI = 4, TEAM_SOLO = 5
+};
 
 // Grid barrier of TEAM_MULTI: spins at most this many SM cycles (about 1 s),
 // then records a time-out in FusedLaunch::err and stops waiting.
@@ -168,6 +174,7 @@ static_assert(sizeof(FusedCirc) == 80, "FusedCirc layout");
 constexpr int kWarpMaxQ = 11;
 constexpr int kCtaMaxQ = 14;
 constexpr int kCtaThreads = 512;
+constexpr int kSoloThreads = 128;
 constexpr int kGlobalThreads = 512;
 constexpr int kGlobalSlotQ = 16;   // log2 amplitudes per TEAM_GLOBAL scratch slot
 
@@ -190,6 +197,7 @@ struct FusedLaunch {
   int32_t ctas_per_job;     // TEAM_MULTI: CTAs per circuit; job j runs on CTAs
                             // [j K, (j + 1) K), its barrier counter is counter[j],
                             // its scratch slot gscratch + j 2^kGlobalSlotQ
+  int32_t norm_width;       // TEAM_SOLO: threads of the team whose norm it forms (32 or 64)
   int32_t team;             // TeamKind of this launch
   int32_t warps_per_cta;    // TEAM_WARP
   int32_t slice_q;          // TEAM_WARP: log2 amplitudes per warp slice; TEAM_CTA: log2 per CTA
