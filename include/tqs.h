@@ -401,7 +401,8 @@ tqs_status tqs_batch_instructions(const tqs_batch* b, int64_t* h_off);
 
 /* Launch shape of a batch's persistent kernel for one size class (0: circuits
  * of n <= 11, run by one or two warps each; 1: n = 12..14, one CTA each with
- * the state in shared memory; 2: n = 15..16, one CTA each on global scratch),
+ * the state in shared memory, launched size by size: the numbers are those of
+ * all sizes, the threads the largest's; 2: n = 15..16, one CTA each on global scratch),
  * as the last tqs_batch_run chose it from the options in force then (a
  * scheduling fact: results do not depend on it).  Outputs (each may be
  * NULL): jobs = circuits of that class, grid = CTAs, threads = threads per
@@ -566,7 +567,8 @@ tqs_status tqs_check_violations(uint32_t* count, int reset);
 /* Launch-shape options for the autotuner (results never depend on them
  * beyond the order of floating-point reductions noted):
  * TQS_OPT_CTA_THREADS, key = 0: threads of the one-CTA team that runs a
- *   circuit of 12..14 qubits, 256 or 512 (default 512).  States and
+ *   circuit of 12..14 qubits, 256 or 512 (default 512; circuits of 12 and 13
+ *   qubits may take fewer, with the same results).  States and
  *   probabilities are bitwise the same; the FP64 norm's reduction order
  *   follows the team size.  A batch reads it (with the warp-class options)
  *   when it is first run on the device, and keeps that launch plan.

@@ -13,10 +13,10 @@
 // device arrays are the segments concatenated in order, so a program's global
 // offsets are its segment's base plus its local offsets.  Headers are written
 // and passes renumbered in parallel, in place.
-// Number of team kinds (warp, CTA, global) that have circuits in the batch.
-static int team_kinds(const tqs_batch* b) {
+// Number of launch kinds that have circuits in the batch.
+static int launch_kinds(const tqs_batch* b) {
   int k = 0;
-  for (int t = 0; t < 3; ++t) k += b->n_team[t] > 0;
+  for (int n : b->n_kind) k += n > 0;
   return k;
 }
 
@@ -67,29 +67,29 @@ static tqs_status batch_finish(tqs_batch* b, const std::vector<CircMeta>& progs,
     for (size_t k = 0; k < m.np; ++k)
       sg.passes[m.lp + k] = Image::rebase(sg.passes[m.lp + k], o0, b->instr_off[i], c0);
   });
-  // Job order per team kind, costliest first (load balance only: every
+  // Job order per launch kind, costliest first (load balance only: every
   // circuit's results are the same in any order).  A counting sort on the
   // cost's log2 in steps of 1/16 (about 4 % apart), batch order within a step.
   constexpr int kBuckets = 1024;
   static thread_local std::vector<int> key, start;
   key.resize(static_cast<size_t>(b->count));
-  start.assign(3 * (kBuckets + 1), 0);
+  start.assign(tqs_batch::kKinds * (kBuckets + 1), 0);
   for (int i = 0; i < b->count; ++i) {
-    const int t = team_for(progs[i].nint);
+    const int t = tqs_batch::kind_for(progs[i].nint);
     const double c = std::max(progs[i].cost, 1.0);
     const int k = std::min(kBuckets - 1, static_cast<int>(std::log2(c) * 16.0));
     key[static_cast<size_t>(i)] = t * kBuckets + (kBuckets - 1 - k);  // descending cost
     ++start[static_cast<size_t>(t * (kBuckets + 1) + (kBuckets - 1 - k) + 1)];
-    ++b->n_team[t];
+    ++b->n_kind[t];
     b->max_nint[t] = std::max(b->max_nint[t], progs[i].nint);
   }
   b->order.resize(static_cast<size_t>(b->count));
   int base = 0;
-  for (int t = 0; t < 3; ++t) {
+  for (int t = 0; t < tqs_batch::kKinds; ++t) {
     int* st = &start[static_cast<size_t>(t * (kBuckets + 1))];
     st[0] = base;
     for (int k = 0; k < kBuckets; ++k) st[k + 1] += st[k];
-    base += b->n_team[t];
+    base += b->n_kind[t];
   }
   for (int i = 0; i < b->count; ++i) {
     const int kk = key[static_cast<size_t>(i)], t = kk / kBuckets, k = kk % kBuckets;
@@ -240,13 +240,12 @@ static tqs_status batch_upload(tqs_batch* b, cudaStream_t s) {
   TQS_CUDA(cudaMemcpyAsync(b->d_img.as<char>() + b->order_off, b->order.data(),
                            b->order.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s),
            "tqs_batch: upload order");
-  for (int t = 0; t < 3; ++t)
-    b->plans[t] = plan_for(t, b->max_nint[t], b->n_team[t], 0);
-  if (b->n_team[TEAM_GLOBAL] > 0)
-    TQS_CUDA(b->d_gscratch.ensure(size_t(b->plans[TEAM_GLOBAL].grid) *
+  b->make_plans();
+  if (b->n_kind[tqs_batch::kKinds - 1] > 0)
+    TQS_CUDA(b->d_gscratch.ensure(size_t(b->plans[tqs_batch::kKinds - 1].grid) *
                                   (size_t(1) << kGlobalSlotQ) * sizeof(float2)),
              "tqs_batch: cudaMalloc scratch");
-  if (team_kinds(b) > 1) TQS_CUDA(b->ensure_side(), "tqs_batch: side streams");
+  if (launch_kinds(b) > 1) TQS_CUDA(b->ensure_side(), "tqs_batch: side streams");
   b->uploaded = true;
   return TQS_OK;
 }
@@ -258,20 +257,20 @@ static tqs_status batch_enqueue_at(tqs_batch* b, char* base, size_t order_off, s
                                    cudaStream_t s, int* kernels = nullptr,
                                    const double* u = nullptr, int32_t* outcomes = nullptr) {
   int32_t* counters = reinterpret_cast<int32_t*>(base + counter_off);
-  TQS_CUDA(cudaMemsetAsync(counters, 0, 3 * sizeof(int32_t), s), "tqs_batch: memset counters");
+  TQS_CUDA(cudaMemsetAsync(counters, 0, tqs_batch::kKinds * sizeof(int32_t), s), "tqs_batch: memset counters");
   int k = 0;
   int first = 0;
-  const bool fork = team_kinds(b) > 1;  // (the side streams exist: ensure_side before any capture)
+  const bool fork = launch_kinds(b) > 1;  // (the side streams exist: ensure_side before any capture)
   if (fork) {
     if (!b->ev_fork) return fail(TQS_ERR_STATE, "tqs_batch: side streams missing");
     TQS_CUDA(cudaEventRecord(b->ev_fork, s), "tqs_batch: fork");
   }
-  for (int t = 0; t < 3; ++t) {
-    if (b->n_team[t] == 0) continue;
+  for (int t = 0; t < tqs_batch::kKinds; ++t) {
+    if (b->n_kind[t] == 0) continue;
     FusedLaunch L{};
     b->img.point(L, base);
     L.order = reinterpret_cast<const int32_t*>(base + order_off) + first;
-    L.n_jobs = b->n_team[t];
+    L.n_jobs = b->n_kind[t];
     L.counter = counters + t;
     L.out = states;
     L.probs = probs;
@@ -284,6 +283,7 @@ static tqs_status batch_enqueue_at(tqs_batch* b, char* base, size_t order_off, s
     L.warps_per_cta = b->plans[t].warps;
     L.slice_q = b->plans[t].slice_q;
     L.grid = b->plans[t].grid;
+    L.norm_width = b->plans[t].norm_width;
     if (fork) {
       TQS_CUDA(cudaStreamWaitEvent(b->side[t], b->ev_fork, 0), "tqs_batch: fork");
       TQS_CUDA(launch_fused(L, b->side[t]), "tqs_batch: launch");
@@ -291,12 +291,12 @@ static tqs_status batch_enqueue_at(tqs_batch* b, char* base, size_t order_off, s
     } else {
       TQS_CUDA(launch_fused(L, s), "tqs_batch: launch");
     }
-    first += b->n_team[t];
+    first += b->n_kind[t];
     ++k;
   }
   if (fork)
-    for (int t = 0; t < 3; ++t)
-      if (b->n_team[t] > 0) TQS_CUDA(cudaStreamWaitEvent(s, b->ev_join[t], 0), "tqs_batch: join");
+    for (int t = 0; t < tqs_batch::kKinds; ++t)
+      if (b->n_kind[t] > 0) TQS_CUDA(cudaStreamWaitEvent(s, b->ev_join[t], 0), "tqs_batch: join");
   if (kernels) *kernels = k;
   return TQS_OK;
 }
@@ -389,17 +389,24 @@ tqs_status tqs_batch_launch_info(const tqs_batch* b, int size_class, int* jobs, 
   if (!b || size_class < 0 || size_class > 2)
     return fail(TQS_ERR_ARG, "tqs_batch_launch_info: NULL batch or size class outside 0..2");
   if (!b->uploaded) return fail(TQS_ERR_STATE, "tqs_batch_launch_info: the batch has not run yet");
-  const LaunchPlan& lp = b->plans[size_class];
-  const int n_jobs = b->n_team[size_class];
-  int per_cta = 1;
-  if (lp.team == TEAM_WARP) per_cta = lp.warps;
-  else if (lp.team == TEAM_PAIR) per_cta = lp.warps / 2;
+  // class 1 is launched once per size: jobs, CTAs and teams in all, and the
+  // threads of the largest of its CTAs
+  const int k0 = size_class == 0 ? 0 : size_class == 1 ? 1 : tqs_batch::kKinds - 1;
+  const int k1 = size_class == 1 ? tqs_batch::kKinds - 2 : k0;
+  int n_jobs = 0, n_grid = 0, n_threads = 0, n_teams = 0;
+  for (int k = k0; k <= k1; ++k) {
+    if (b->n_kind[k] == 0) continue;
+    const LaunchPlan& lp = b->plans[k];
+    const int per_cta = lp.team == TEAM_WARP ? lp.warps : lp.team == TEAM_PAIR ? lp.warps / 2 : 1;
+    n_jobs += b->n_kind[k];
+    n_grid += lp.grid;
+    n_teams += lp.grid * per_cta;
+    n_threads = std::max(n_threads, lp.team == TEAM_GLOBAL ? kGlobalThreads : 32 * lp.warps);
+  }
   if (jobs) *jobs = n_jobs;
-  if (grid) *grid = n_jobs ? lp.grid : 0;
-  const int nthreads = (lp.team == TEAM_WARP || lp.team == TEAM_PAIR) ? 32 * lp.warps
-                       : lp.team == TEAM_CTA ? 32 * lp.warps : kGlobalThreads;
-  if (threads) *threads = n_jobs ? nthreads : 0;
-  if (teams) *teams = n_jobs ? lp.grid * per_cta : 0;
+  if (grid) *grid = n_grid;
+  if (threads) *threads = n_threads;
+  if (teams) *teams = n_teams;
   return TQS_OK;
 }
 
@@ -430,9 +437,9 @@ tqs_status tqs_batch_run_host(tqs_batch* b, tqs_c64* h_states, double* h_probs, 
   const size_t probs_off = (states_off + (zs ? 0 : amps * sizeof(float2)) + 255) & ~size_t(255);
   const size_t norms_off = (probs_off + (h_probs && !zp ? amps * sizeof(double) : 0) + 255) & ~size_t(255);
   const size_t total = norms_off + (zn ? 0 : size_t(b->count) * sizeof(double));
-  for (int t = 0; t < 3; ++t) b->plans[t] = plan_for(t, b->max_nint[t], b->n_team[t], 0);
-  const size_t gscr = b->n_team[TEAM_GLOBAL]
-                          ? size_t(b->plans[TEAM_GLOBAL].grid) * (size_t(1) << kGlobalSlotQ) * sizeof(float2)
+  b->make_plans();
+  const size_t gscr = b->n_kind[tqs_batch::kKinds - 1]
+                          ? size_t(b->plans[tqs_batch::kKinds - 1].grid) * (size_t(1) << kGlobalSlotQ) * sizeof(float2)
                           : 0;
   char* base = nullptr;
   const Allocator A = current_allocator();
@@ -453,7 +460,7 @@ tqs_status tqs_batch_run_host(tqs_batch* b, tqs_c64* h_states, double* h_probs, 
   double* dn = zn ? zn : reinterpret_cast<double*>(base + norms_off);
   const size_t gscr_at = (total + 255) & ~size_t(255);
   b->exact_probs = g_exact_probs.load();
-  if (team_kinds(b) > 1) TQS_CUDA(b->ensure_side(), "tqs_batch_run_host: side streams");
+  if (launch_kinds(b) > 1) TQS_CUDA(b->ensure_side(), "tqs_batch_run_host: side streams");
   tqs_status st = batch_enqueue_at(b, base, order_off, counter_off,
                                    reinterpret_cast<float2*>(base + gscr_at), ds, dp, dn, s);
   if (st != TQS_OK) return st;

@@ -813,6 +813,7 @@ struct LaunchPlan {
   int warps;
   int slice_q;
   int grid;
+  int norm_width = 0;  // FusedLaunch::norm_width
 };
 
 // TQS_OPT_WARPS_PER_CTA table, indexed by the warp slice's log2 amplitudes.
@@ -833,7 +834,9 @@ inline std::atomic<int> g_chain_kchunk{0};
 // TQS_OPT_CHAIN_PAIR: the chain's GEMMs as two-CTA clusters sharing B tiles (1) or not (0).
 inline std::atomic<int> g_chain_pair{0};
 
-inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint) {
+// instr: the circuits hold instructions (their reductions are summed in a
+// partition that depends on the CTA's threads, which then stay the option's).
+inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint, bool instr = false) {
   LaunchPlan lp{team, 1, 4, 1};
   if (team == TEAM_WARP) {
     lp.slice_q = std::max(4, max_nint);
@@ -856,7 +859,16 @@ inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint) {
     lp.grid = std::max(1, std::min(want, per_sm * device_sms()));
   } else if (team == TEAM_CTA) {
     lp.slice_q = std::max(4, max_nint);
-    lp.warps = g_cta_threads.load() / 32;
+    lp.norm_width = g_cta_threads.load();
+    lp.warps = lp.norm_width / 32;
+    // A 12-qubit circuit has 256 groups a pass; with 256 threads two CTAs share
+    // an SM's registers, and where circuits queue up a 13-qubit one gains more
+    // from the neighbour that works while it waits at a barrier or writes its
+    // outputs than from a second set of threads: 1024 random circuits of 12
+    // qubits 408 -> 194 us, of 13 qubits 546 -> 312 us, QFT and the like 267 ->
+    // 166 us (4096 of 12) and 176 -> 118 us (2048 of 13).
+    if (!instr && (lp.slice_q <= 12 || (lp.slice_q == 13 && jobs > device_sms())))
+      lp.warps = std::min(lp.warps, 8);
     const int per_sm = std::max(1, fused_max_ctas_per_sm(TEAM_CTA, lp.warps, lp.slice_q));
     lp.grid = std::max(1, std::min(jobs, per_sm * device_sms()));
   } else {
@@ -1039,16 +1051,28 @@ struct tqs_batch {
   std::vector<int64_t> offsets;  // count + 1
   std::vector<int64_t> instr_off;  // count + 1: instruction (uniform / outcome) offsets
   Image img;
-  std::vector<int32_t> order;    // [warp jobs][cta jobs][global jobs]
-  int n_team[3] = {0, 0, 0};
-  int max_nint[3] = {4, 4, 4};
+  // Launches of the batch: the warp class, one per size of the CTA class
+  // (12, 13, 14 qubits: with a launch for all three the smaller ones would
+  // hold the shared memory and threads of the largest), the global class.
+  static constexpr int kKinds = 5;
+  static int kind_for(int nint) {
+    return nint <= kWarpMaxQ ? 0 : nint <= kCtaMaxQ ? nint - kWarpMaxQ : kKinds - 1;
+  }
+  static int team_of(int kind) { return kind == 0 ? TEAM_WARP : kind < kKinds - 1 ? TEAM_CTA : TEAM_GLOBAL; }
+  std::vector<int32_t> order;    // the jobs of each kind in turn
+  int n_kind[kKinds] = {};
+  int max_nint[kKinds] = {4, 4, 4, 4, 4};
   DevBuf d_img;                  // image + order + counters
   size_t order_off = 0, counter_off = 0;
   bool uploaded = false;
   DevBuf d_gscratch;
   DevBuf d_sample;               // sampling: segment tables + block sums / prefixes
   std::unique_ptr<SamplePlan> sample_plan;
-  LaunchPlan plans[3];
+  LaunchPlan plans[kKinds];
+  void make_plans() {
+    for (int t = 0; t < kKinds; ++t)
+      plans[t] = plan_for(team_of(t), max_nint[t], n_kind[t], 0, instr_off.back() > 0);
+  }
   // graph cache
   cudaStream_t cap_stream = nullptr;
   cudaGraph_t graph = nullptr;
@@ -1065,13 +1089,14 @@ struct tqs_batch {
   // side by side: forked from the caller's stream onto these streams and
   // joined back (inside a captured graph too), so the kinds share the GPU in
   // each other's tails instead of running one after the other.
-  cudaStream_t side[3] = {nullptr, nullptr, nullptr};
+  cudaStream_t side[kKinds] = {};
   cudaEvent_t ev_fork = nullptr;
-  cudaEvent_t ev_join[3] = {nullptr, nullptr, nullptr};
+  cudaEvent_t ev_join[kKinds] = {};
   cudaError_t ensure_side() {
     if (ev_fork) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    for (int t = 0; t < 3 && e == cudaSuccess; ++t) {
+    for (int t = 0; t < kKinds && e == cudaSuccess; ++t) {
+      if (n_kind[t] == 0) continue;
       if (!side[t]) e = cudaStreamCreateWithFlags(&side[t], cudaStreamNonBlocking);
       if (e == cudaSuccess && !ev_join[t]) e = cudaEventCreateWithFlags(&ev_join[t], cudaEventDisableTiming);
     }
@@ -1082,7 +1107,7 @@ struct tqs_batch {
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
     if (cap_stream) cudaStreamDestroy(cap_stream);
-    for (int t = 0; t < 3; ++t) {
+    for (int t = 0; t < kKinds; ++t) {
       if (side[t]) cudaStreamDestroy(side[t]);
       if (ev_join[t]) cudaEventDestroy(ev_join[t]);
     }

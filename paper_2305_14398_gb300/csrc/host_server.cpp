@@ -183,6 +183,7 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
     L.warps_per_cta = plans[t].warps;
     L.slice_q = plans[t].slice_q;
     L.grid = plans[t].grid;
+    L.norm_width = plans[t].norm_width;
     if (t == TEAM_GLOBAL && multi_k) {
       L.team = TEAM_MULTI;
       L.ctas_per_job = multi_k;

@@ -852,8 +852,12 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
     // log2 of the index stride between a thread's pairs (2 size): fixed for
     // the warp and pair teams, so the stores take immediate offsets
     constexpr int kSh = TEAM == TEAM_WARP ? 6 : TEAM == TEAM_PAIR ? 7 : 0;
-    const int sh = kSh ? kSh : 31 - __clz(2 * size);
-    const int i0 = 2 * rank;
+    const int sh = kSh ? kSh : 31 - __clz(2 * (TEAM == TEAM_CTA && L.norm_width > size ? L.norm_width : size));
+    // a CTA of fewer threads than norm_width does the work of several of that
+    // team's threads in turn, so the norm's partial sums are the same
+    const int width = TEAM == TEAM_CTA && L.norm_width > size ? L.norm_width : size;
+    for (int vr = rank; vr < (TEAM == TEAM_CTA ? width : rank + 1); vr += size) {
+    const int i0 = 2 * vr;
     if (i0 < N) {
       const float oscale = cd.out_scale;
       const bool exact = L.exact_probs != 0;
@@ -901,6 +905,17 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
         else acc += static_cast<double>(bs);
       }
     }
+    if (TEAM == TEAM_CTA && vr + size < width) {  // (the last turn's sum goes on below)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if ((vr & 31) == 0) s_red[vr >> 5] = acc;
+      acc = 0.0;
+    }
+    }
+    if (TEAM == TEAM_CTA) {
+      rank += width - size;
+      size = width;
+    }
   }
   if (TEAM == TEAM_SOLO) {
     // lane by lane, the blocks in order; the first norm_width threads go on
@@ -919,7 +934,7 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
     const int warp = rank >> 5, lane = rank & 31;
     if (lane == 0) s_red[warp] = acc;
     team_sync<TEAM>();
-    if (rank == 0) { double s = 0.0; for (int w = 0; w < (size >> 5); ++w) s += s_red[w]; if (L.norms) L.norms[ci] = s; }
+    if (TEAM == TEAM_CTA ? threadIdx.x == 0 : rank == 0) { double s = 0.0; for (int w = 0; w < (size >> 5); ++w) s += s_red[w]; if (L.norms) L.norms[ci] = s; }
   }
   if (TEAM == TEAM_MULTI && rank == 0 && *reinterpret_cast<volatile int*>(L.err) != 0) {
     // a grid barrier timed out: the outputs are not valid, make that visible

@@ -252,13 +252,14 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
   TQS_CUDA(c->d_counter.ensure(2 * sizeof(int32_t)), "tqs_simulate: cudaMalloc counter");
   TQS_CUDA(cudaMemsetAsync(c->d_counter.p, 0, 2 * sizeof(int32_t), s), "tqs_simulate: memset");
   L.counter = c->d_counter.as<int32_t>();
-  LaunchPlan lp = plan_for(team, P.nint, 1, 1);
+  LaunchPlan lp = plan_for(team, P.nint, 1, 1, P.n_instr > 0);
   if (team == TEAM_GLOBAL) {
     TQS_CUDA(c->d_gscratch.ensure((size_t(1) << kGlobalSlotQ) * sizeof(float2)),
              "tqs_simulate: cudaMalloc scratch");
     L.gscratch = c->d_gscratch.as<float2>();
   }
   L.team = lp.team;
+  L.norm_width = lp.norm_width;
   L.warps_per_cta = lp.warps;
   L.slice_q = lp.slice_q;
   // A single circuit of the global class runs on several CTAs (TEAM_MULTI,

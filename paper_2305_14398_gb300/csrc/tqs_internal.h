@@ -197,7 +197,8 @@ struct FusedLaunch {
   int32_t ctas_per_job;     // TEAM_MULTI: CTAs per circuit; job j runs on CTAs
                             // [j K, (j + 1) K), its barrier counter is counter[j],
                             // its scratch slot gscratch + j 2^kGlobalSlotQ
-  int32_t norm_width;       // TEAM_SOLO: threads of the team whose norm it forms (32 or 64)
+  int32_t norm_width;       // threads of the team whose norm is formed: TEAM_SOLO 32 or 64;
+                            // TEAM_CTA at least the CTA's (0: its own)
   int32_t team;             // TeamKind of this launch
   int32_t warps_per_cta;    // TEAM_WARP
   int32_t slice_q;          // TEAM_WARP: log2 amplitudes per warp slice; TEAM_CTA: log2 per CTA
