@@ -74,8 +74,10 @@ static tqs_status batch_finish(tqs_batch* b, const std::vector<CircMeta>& progs,
   static thread_local std::vector<int> key, start;
   key.resize(static_cast<size_t>(b->count));
   start.assign(tqs_batch::kKinds * (kBuckets + 1), 0);
+  int warp_class = 0;
+  for (const CircMeta& m : progs) warp_class += m.nint <= kWarpMaxQ;
   for (int i = 0; i < b->count; ++i) {
-    const int t = tqs_batch::kind_for(progs[i].nint);
+    const int t = tqs_batch::kind_for(progs[i].nint, tqs_batch::solo(progs[i], warp_class));
     const double c = std::max(progs[i].cost, 1.0);
     const int k = std::min(kBuckets - 1, static_cast<int>(std::log2(c) * 16.0));
     key[static_cast<size_t>(i)] = t * kBuckets + (kBuckets - 1 - k);  // descending cost
@@ -257,7 +259,10 @@ static tqs_status batch_enqueue_at(tqs_batch* b, char* base, size_t order_off, s
                                    cudaStream_t s, int* kernels = nullptr,
                                    const double* u = nullptr, int32_t* outcomes = nullptr) {
   int32_t* counters = reinterpret_cast<int32_t*>(base + counter_off);
-  TQS_CUDA(cudaMemsetAsync(counters, 0, tqs_batch::kKinds * sizeof(int32_t), s), "tqs_batch: memset counters");
+  bool counted = false;
+  for (int t = 0; t < tqs_batch::kKinds; ++t) counted = counted || (b->n_kind[t] > 0 && !b->one_each(t));
+  if (counted)
+    TQS_CUDA(cudaMemsetAsync(counters, 0, tqs_batch::kKinds * sizeof(int32_t), s), "tqs_batch: memset counters");
   int k = 0;
   int first = 0;
   const bool fork = launch_kinds(b) > 1;  // (the side streams exist: ensure_side before any capture)
@@ -271,7 +276,7 @@ static tqs_status batch_enqueue_at(tqs_batch* b, char* base, size_t order_off, s
     b->img.point(L, base);
     L.order = reinterpret_cast<const int32_t*>(base + order_off) + first;
     L.n_jobs = b->n_kind[t];
-    L.counter = counters + t;
+    L.counter = b->one_each(t) ? nullptr : counters + t;
     L.out = states;
     L.probs = probs;
     L.exact_probs = b->exact_probs;
@@ -389,10 +394,10 @@ tqs_status tqs_batch_launch_info(const tqs_batch* b, int size_class, int* jobs, 
   if (!b || size_class < 0 || size_class > 2)
     return fail(TQS_ERR_ARG, "tqs_batch_launch_info: NULL batch or size class outside 0..2");
   if (!b->uploaded) return fail(TQS_ERR_STATE, "tqs_batch_launch_info: the batch has not run yet");
-  // class 1 is launched once per size: jobs, CTAs and teams in all, and the
-  // threads of the largest of its CTAs
-  const int k0 = size_class == 0 ? 0 : size_class == 1 ? 1 : tqs_batch::kKinds - 1;
-  const int k1 = size_class == 1 ? tqs_batch::kKinds - 2 : k0;
+  // classes 0 and 1 may take several launches: jobs, CTAs and teams in all, and
+  // the threads of the largest CTAs
+  const int k0 = size_class == 0 ? 0 : size_class == 1 ? tqs_batch::kCtaKind : tqs_batch::kKinds - 1;
+  const int k1 = size_class == 0 ? tqs_batch::kCtaKind - 1 : size_class == 1 ? tqs_batch::kKinds - 2 : k0;
   int n_jobs = 0, n_grid = 0, n_threads = 0, n_teams = 0;
   for (int k = k0; k <= k1; ++k) {
     if (b->n_kind[k] == 0) continue;

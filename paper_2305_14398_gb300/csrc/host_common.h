@@ -284,6 +284,7 @@ struct Program {
   // left here for the program that follows (else it is applied, and 1).
   cd carry = 1.0;
   bool defer = false;
+  bool rotations = false;  // holds general gates (as rotations)
   double cost = 0.0;
   // Empty the program for reuse (keeps the vectors' capacity).
   void reset() {
@@ -298,6 +299,7 @@ struct Program {
     n_instr = 0;
     carry = 1.0;
     defer = false;
+    rotations = false;
     cost = 0.0;
   }
 };
@@ -444,6 +446,7 @@ struct ImageSeg {
 // segment `seg` (passes still numbered program-locally).
 struct CircMeta {
   int n = 0, nint = 4, n_instr = 0, gen_index = 0;
+  bool rotations = false;
   float out_scale = 1.0f;
   double cost = 0.0;
   uint16_t col[16] = {};
@@ -459,6 +462,7 @@ inline CircMeta append_program(const Program& P, ImageSeg& sg, int seg) {
   m.n = P.n;
   m.nint = P.nint;
   m.n_instr = P.n_instr;
+  m.rotations = P.rotations;
   m.col_off = P.col_off;
   m.gen_index = P.gen_index;
   m.out_scale = P.out_scale;
@@ -857,6 +861,12 @@ inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint, boo
     const int circuits_per_cta = lp.team == TEAM_PAIR ? w / 2 : w;
     const int want = (jobs + circuits_per_cta - 1) / circuits_per_cta;
     lp.grid = std::max(1, std::min(want, per_sm * device_sms()));
+  } else if (team == TEAM_SOLO) {
+    lp.slice_q = std::max(4, max_nint);
+    lp.norm_width = 32 * g_team_warps_for_q[lp.slice_q].load();
+    lp.warps = std::max(lp.norm_width, std::min(kSoloThreads, 1 << (lp.slice_q - 4))) / 32;
+    const int per_sm = std::max(1, fused_max_ctas_per_sm(TEAM_SOLO, lp.warps, lp.slice_q));
+    lp.grid = std::max(1, std::min(jobs, per_sm * device_sms()));
   } else if (team == TEAM_CTA) {
     lp.slice_q = std::max(4, max_nint);
     lp.norm_width = g_cta_threads.load();
@@ -1051,17 +1061,42 @@ struct tqs_batch {
   std::vector<int64_t> offsets;  // count + 1
   std::vector<int64_t> instr_off;  // count + 1: instruction (uniform / outcome) offsets
   Image img;
-  // Launches of the batch: the warp class, one per size of the CTA class
-  // (12, 13, 14 qubits: with a launch for all three the smaller ones would
-  // hold the shared memory and threads of the largest), the global class.
-  static constexpr int kKinds = 5;
-  static int kind_for(int nint) {
-    return nint <= kWarpMaxQ ? 0 : nint <= kCtaMaxQ ? nint - kWarpMaxQ : kKinds - 1;
+  // Launches of the batch: the warp class, those of its circuits that take a
+  // CTA each (by threads: up to 9 qubits, 10, 11), one per size of the CTA
+  // class (12, 13, 14 qubits: with a launch for all three the smaller ones
+  // would hold the shared memory and threads of the largest), the global class.
+  static constexpr int kSoloKind = 1, kCtaKind = 4, kKinds = 8;
+  static int kind_for(int nint, bool solo) {
+    if (nint > kCtaMaxQ) return kKinds - 1;
+    if (nint > kWarpMaxQ) return kCtaKind + nint - kWarpMaxQ - 1;
+    return solo ? kSoloKind + std::max(0, nint - (kWarpMaxQ - 2)) : 0;
   }
-  static int team_of(int kind) { return kind == 0 ? TEAM_WARP : kind < kKinds - 1 ? TEAM_CTA : TEAM_GLOBAL; }
+  // Which circuits of the warp class take a CTA each (without instructions or
+  // custom unitaries).
+  //   * From 10 qubits on, those with general gates: every amplitude is worked
+  //     from the second pass on, and the warps of a CTA share the program's
+  //     instructions and records (2000 random circuits of 11 qubits 366 -> 189
+  //     us, of 10 qubits 203 -> 132 us; of 9 qubits 117 against 122 us).
+  //   * In a batch of kSoloFew or fewer, all: they all run at once, and a
+  //     circuit's own time counts (1000 of the paper's programs of 11 qubits
+  //     35.7 -> 22.7 us, of 8 qubits 16.2 -> 12.3 us).
+  //   * Up to twice as many (16 CTAs of 32 threads to an SM), those without
+  //     general gates (2000 of 9 qubits 23.3 -> 14.7 us, of 11 qubits 44.5 ->
+  //     40.4 us; random ones of 8 qubits 93 against 109 us).
+  // Beyond, the paper's programs work few groups until their last passes and
+  // are bound by their outputs (16384 of 11 qubits: 146 us on warps, 274 us on CTAs).
+  static constexpr int kSoloFew = 1216;
+  static bool solo(const CircMeta& m, int warp_class) {
+    if (m.nint > kWarpMaxQ || m.n_instr > 0 || m.nc > 0) return false;
+    if (m.rotations) return warp_class <= kSoloFew || m.nint >= kWarpMaxQ - 1;
+    return warp_class <= 2 * kSoloFew;
+  }
+  static int team_of(int kind) {
+    return kind == 0 ? TEAM_WARP : kind < kCtaKind ? TEAM_SOLO : kind < kKinds - 1 ? TEAM_CTA : TEAM_GLOBAL;
+  }
   std::vector<int32_t> order;    // the jobs of each kind in turn
   int n_kind[kKinds] = {};
-  int max_nint[kKinds] = {4, 4, 4, 4, 4};
+  int max_nint[kKinds] = {4, 4, 4, 4, 4, 4, 4, 4};
   DevBuf d_img;                  // image + order + counters
   size_t order_off = 0, counter_off = 0;
   bool uploaded = false;
@@ -1069,6 +1104,8 @@ struct tqs_batch {
   DevBuf d_sample;               // sampling: segment tables + block sums / prefixes
   std::unique_ptr<SamplePlan> sample_plan;
   LaunchPlan plans[kKinds];
+  // every CTA of the launch has one job: no job counter
+  bool one_each(int kind) const { return team_of(kind) == TEAM_SOLO && plans[kind].grid == n_kind[kind]; }
   void make_plans() {
     for (int t = 0; t < kKinds; ++t)
       plans[t] = plan_for(team_of(t), max_nint[t], n_kind[t], 0, instr_off.back() > 0);

@@ -1008,6 +1008,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
   if (!prepared) {
     fused_tls.clear();
     split = prepare_gates(n, gs, fused_tls, P.carry, absorb ? &flips : nullptr);
+    P.rotations = split;
   }
 
   std::vector<uint32_t>& qmask = qmask_tls;

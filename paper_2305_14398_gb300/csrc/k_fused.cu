@@ -992,9 +992,20 @@ __global__ void __launch_bounds__(TEAM == TEAM_SOLO ? kSoloThreads : TEAM == TEA
   } else if (TEAM == TEAM_SOLO) {
     __shared__ double s_red[32];
     __shared__ float blk_sum[kSoloSums];
+    __shared__ int s_job;
     int unused_job = 0, unused_ci = 0;
-    run_circuit<TEAM_SOLO>(L, 0, smem, threadIdx.x, blockDim.x, s_red, unused_job, unused_ci, nullptr, nullptr,
-                           blk_sum);
+    for (;;) {
+      int job = blockIdx.x;  // without a counter: one job per CTA
+      if (L.counter != nullptr) {
+        if (threadIdx.x == 0) s_job = atomicAdd(L.counter, 1);
+        __syncthreads();
+        job = s_job;
+        if (job >= L.n_jobs) break;
+      }
+      run_circuit<TEAM_SOLO>(L, L.order[job], smem, threadIdx.x, blockDim.x, s_red, unused_job, unused_ci, nullptr,
+                             nullptr, blk_sum);
+      if (L.counter == nullptr) break;
+    }
   } else if (TEAM == TEAM_MULTI) {
     __shared__ double s_red[32];
     const int K = L.ctas_per_job;
@@ -1159,6 +1170,8 @@ int fused_max_ctas_per_sm(int team, int warps_per_cta, int slice_q) {
                          static_cast<int>(smem));
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fused_kernel<TEAM_CTA>, threads,
                                                       smem);
+  } else if (team == TEAM_SOLO) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fused_kernel<TEAM_SOLO>, threads, smem);
   } else {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fused_kernel<TEAM_GLOBAL>, threads,
                                                       smem);
@@ -1212,7 +1225,7 @@ cudaError_t launch_fused(const FusedLaunch& L, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     fused_kernel<TEAM_CTA><<<L.grid, threads, smem, s>>>(L);
   } else if (L.team == TEAM_SOLO) {
-    fused_kernel<TEAM_SOLO><<<1, threads, smem, s>>>(L);
+    fused_kernel<TEAM_SOLO><<<L.grid, threads, smem, s>>>(L);
   } else if (L.team == TEAM_MULTI) {
     // cooperative: the CTAs wait on one another at the grid barriers
     FusedLaunch arg = L;

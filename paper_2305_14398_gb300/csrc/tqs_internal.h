@@ -134,8 +134,8 @@ static_assert(sizeof(FusedPass) == 16, "FusedPass layout");
 // the outputs with exactly the TEAM_GLOBAL output phase, so results are
 // bitwise those of TEAM_GLOBAL.  Circuits without instructions or custom
 // unitaries, few enough that all their CTAs are resident at once.
-// TEAM_SOLO: one circuit of the warp class alone on the GPU, a CTA with a
-// thread per group of a pass (up to 128).  It writes the outputs block by block
+// TEAM_SOLO: a circuit of the warp class on a CTA with a thread per group of a
+// pass (up to 128): alone on the GPU, or the jobs of a batch in turn.  It writes the outputs block by block
 // as the warps of a warp team (or pair) would, so they and the norm are
 // bitwise the same.  Circuits without instructions or custom unitaries.
 enum TeamKind : int32_t {
@@ -184,7 +184,8 @@ struct FusedLaunch {
   const FusedOp* ops;       // device
   const int32_t* order;     // device: circuit indices of this team kind, costliest first
   int32_t n_jobs;
-  int32_t* counter;         // device: job counter, zeroed before the launch
+  int32_t* counter;         // device: job counter, zeroed before the launch (nullptr where every
+                            // CTA of TEAM_SOLO has one job: grid = n_jobs)
   float2* out;              // device outputs (logical order)
   double* probs;            // nullable
   double* norms;            // nullable

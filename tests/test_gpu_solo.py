@@ -42,3 +42,47 @@ def test_single_equals_batch(n, team_warps):
                 B.tqs_circuit_destroy(c)
     finally:
         B.tqs_set_option(B.OPT_TEAM_WARPS, q, old)
+
+
+@pytest.mark.parametrize("count", [3, 1300, 2500])
+def test_batches_on_either_team_equal_singles(count):
+    """Batches on both sides of the rules that give circuits of the warp class a
+    CTA each: with and without general gates, 8 to 11 qubits, more circuits
+    than CTAs, instructions and custom unitaries (which stay on warps) between
+    them; every copy bitwise the single call's."""
+    from test_host_program import with_customs
+    g = W.rng(97)
+    kinds = [(n, ops) for n in (5, 9, 10, 11) for ops in (W.qft_on_basis(n, 3), W.random_mixed(n, 5, (97, n)))]
+    extra = [(10, [("h", (0,), ()), ("measure", (0,), ()), ("rx", (1,), (0.3,))]), (9, with_customs(9, 7)[0])]
+    circs = extra + [kinds[int(g.integers(0, len(kinds)))] for _ in range(count)]
+    handles = {}
+    for n, ops in circs:
+        if id(ops) not in handles:
+            handles[id(ops)] = B.circuit_from_ops(n, ops)
+    try:
+        b = B.tqs_batch_create([handles[id(ops)] for _, ops in circs])
+        try:
+            _, total, offs = B.tqs_batch_info(b)
+            st = torch.empty(total, dtype=torch.complex64, device="cuda")
+            pr = torch.empty(total, dtype=torch.float64, device="cuda")
+            nm = torch.empty(len(circs), dtype=torch.float64, device="cuda")
+            u = torch.full((1,), 0.25, dtype=torch.float64, device="cuda")
+            B.tqs_batch_run_measured(b, st, u, probs=pr, norms=nm)
+            assert B.tqs_batch_launch_info(b, 0)["jobs"] == len(circs)
+        finally:
+            B.tqs_batch_destroy(b)
+        single = {}
+        for n, ops in circs:
+            if id(ops) in single:
+                continue
+            o = [torch.empty(1 << n, dtype=d, device="cuda") for d in (torch.complex64, torch.float64)]
+            o.append(torch.empty(1, dtype=torch.float64, device="cuda"))
+            B.tqs_simulate_measured(handles[id(ops)], o[0], u=u, probs=o[1], norm=o[2])
+            single[id(ops)] = o
+        for i, (n, ops) in enumerate(circs):
+            s, p, m = single[id(ops)]
+            assert torch.equal(st[offs[i]:offs[i + 1]], s) and torch.equal(pr[offs[i]:offs[i + 1]], p)
+            assert float(nm[i]) == float(m)
+    finally:
+        for c in handles.values():
+            B.tqs_circuit_destroy(c)
