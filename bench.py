@@ -898,6 +898,12 @@ def bench_chain(B, W, torch, peaks, mpeaks):
         sec = s.elapsed_time(e) / 1e3 / reps
         N = 1 << n
         gemms = B.tqs_circuit_info(c)[2] - 1
+        if prec != B.PREC_FP32_SIMT:
+            # products formed (steps are multiplied together first): a call launches
+            # a generator for the first matrix, then a generator and a GEMM each
+            before = B.tqs_launch_count()
+            B.tqs_circuit_unitary(c, prec, U)
+            gemms = (B.tqs_launch_count() - before - 1) // 2
         key = f"n{n}_{names[prec]}"
         rec = {"ms": 1e3 * sec, "gemms": gemms,
                "useful_complex_gflops": 8.0 * N ** 3 * gemms / sec / 1e9}
@@ -1145,7 +1151,11 @@ def bench_chain_sharded(B, W, torch, dist, rank, world, peaks, n=13, reps=2):
         e.record()
         torch.cuda.synchronize()
         sec = s.elapsed_time(e) / 1e3 / reps
-        gemms = B.tqs_circuit_info(c)[2] - 1
+        before = B.tqs_launch_count()
+        if ncols > 0:
+            B.tqs_circuit_unitary_cols(c, B.PREC_TC_BF16X3, col0, ncols, blk)
+            torch.cuda.synchronize()
+        gemms = (B.tqs_launch_count() - before - 1) // 2 if ncols > 0 else 0  # products formed
     finally:
         B.tqs_circuit_destroy(c)
     slowest = max_over_ranks(sec, dist, "cuda")

@@ -223,7 +223,9 @@ tqs_status tqs_materialize_step(tqs_circuit* c, int step, tqs_c64* d_S, void* st
 /* ----------------------------------------------------------------- unitary
  * Algorithm 1: the circuit unitary U = S_m ... S_1 as a chain of complex
  * matrix products U <- S_k U (the product with the initial identity is
- * skipped), in the arithmetic `prec` (tqs_prec).
+ * skipped), in the arithmetic `prec` (tqs_prec).  The tensor-core forms first
+ * multiply, in FP64, consecutive steps whose gates fall into blocks of at most
+ * 5 qubits: such a run enters the chain as one step.
  *   d_U : 2^n x 2^n tqs_c64, row-major, d_U[r * 2^n + c] = <r|U|c>.
  * n <= TQS_MAX_DENSE_QUBITS; tensor-core precisions need n >= 7.
  * Scratch (cached on the circuit): 36 * 4^n bytes for TQS_PREC_TC_BF16X3

@@ -529,19 +529,24 @@ static tqs_status unitary_block(tqs_circuit* c, int prec, int col0, int ncols, t
              "tqs_circuit_unitary: columns");
     return TQS_OK;
   }
-  tqs_status st = upload_factors(c, s);
+  // the tensor-core chain's table: steps multiplied together where they allow
+  StepTable& T = prec == TQS_PREC_FP32_SIMT ? c->table : c->chain_table;
+  if (prec == TQS_PREC_FP32_SIMT) ensure_steps(c);
+  else ensure_chain_steps(c);
+  tqs_status st = upload_table(T, s);
   if (st != TQS_OK) return st;
-  if (c->nsteps <= 1) {
+  const int nsteps = static_cast<int>(T.steps.size());
+  if (nsteps <= 1) {
     // Algorithm 1 with at most one step: U = S_1 (or the identity).
-    StepDesc d = c->nsteps == 1 ? c->steps[0] : StepDesc{0, 0, (1u << c->n) - 1u, 0};
+    StepDesc d = nsteps == 1 ? T.steps[0] : StepDesc{0, 0, (1u << c->n) - 1u, 0};
     if (col0 == 0 && ncols == N && ldu == N) {
-      TQS_CUDA(launch_materialize(c->d_factors.as<StepFactor>(), d, c->n, U, s),
+      TQS_CUDA(launch_materialize(T.dev.as<StepFactor>(), d, c->n, U, s),
                "tqs_circuit_unitary: materialize");
       return TQS_OK;
     }
     TQS_CUDA(c->d_chain.ensure(size_t(N) * N * sizeof(float2)), "tqs_circuit_unitary: cudaMalloc");
     float2* S = c->d_chain.as<float2>();
-    TQS_CUDA(launch_materialize(c->d_factors.as<StepFactor>(), d, c->n, S, s),
+    TQS_CUDA(launch_materialize(T.dev.as<StepFactor>(), d, c->n, S, s),
              "tqs_circuit_unitary: materialize");
     TQS_CUDA(cudaMemcpy2DAsync(U, size_t(ldu) * sizeof(float2), S + col0, size_t(N) * sizeof(float2),
                                size_t(ncols) * sizeof(float2), size_t(N), cudaMemcpyDeviceToDevice, s),
@@ -551,7 +556,7 @@ static tqs_status unitary_block(tqs_circuit* c, int prec, int col0, int ncols, t
   TQS_CUDA(c->d_chain.ensure(chain_tc_scratch_bytes(c->n, prec, ncols)), "tqs_circuit_unitary: cudaMalloc");
   TQS_CUDA(c->d_err.ensure(sizeof(int)), "tqs_circuit_unitary: cudaMalloc");
   TQS_CUDA(cudaMemsetAsync(c->d_err.p, 0, sizeof(int), s), "tqs_circuit_unitary: memset");
-  TQS_CUDA(chain_tc(c->d_factors.as<StepFactor>(), c->steps.data(), c->nsteps, c->n, prec, col0, ncols,
+  TQS_CUDA(chain_tc(T.dev.as<StepFactor>(), T.steps.data(), nsteps, c->n, prec, col0, ncols,
                     U, ldu, c->d_chain.p, c->d_err.as<int>(), g_chain_group.load(),
                     g_chain_kchunk.load(), g_chain_pair.load(), s),
            "tqs_circuit_unitary: tensor-core chain");

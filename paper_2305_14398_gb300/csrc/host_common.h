@@ -690,6 +690,22 @@ struct ProgramUpload {
   }
 };
 
+// Steps as Kronecker factors, and their device copy.
+struct StepTable {
+  bool valid = false;
+  std::vector<StepFactor> factors;
+  std::vector<int64_t> factor_coef;  // per factor: offset in coef_pool, -1 if none
+  std::vector<float2> coef_pool;     // custom factors' entries (row-major, FP32)
+  std::vector<StepDesc> steps;
+  DevBuf dev;
+  void clear() {
+    factors.clear();
+    factor_coef.clear();
+    coef_pool.clear();
+    steps.clear();
+  }
+};
+
 struct tqs_circuit {
   int n = 0;
   int n_instr = 0;  // measure / reset instructions
@@ -704,13 +720,8 @@ struct tqs_circuit {
   ProgramUpload run_prog;  // `prog`, or `prog_init` with its initial-state pointer
   DevBuf d_counter;   // job counter
   DevBuf d_gscratch;  // TEAM_GLOBAL slot
-  // cached plain-form step table
-  bool steps_valid = false;
-  std::vector<StepFactor> factors;
-  std::vector<int64_t> factor_coef;  // per factor: offset in coef_pool, -1 if none
-  std::vector<float2> coef_pool;     // custom factors' entries (row-major, FP32)
-  std::vector<StepDesc> steps;
-  DevBuf d_factors;
+  StepTable table;        // a factor per gate (plain form)
+  StepTable chain_table;  // steps multiplied together (tensor-core chain)
   DevBuf d_plain;     // S scratch + two state vectors
   DevBuf d_partials;  // probability partials
   DevBuf d_collapse;  // simulateAndCollapse: state + probabilities
@@ -913,84 +924,201 @@ inline int multi_ctas_for(const Program& P) {
   return std::max(1, std::min(limit, groups / kGlobalThreads));
 }
 
+// The gates [first, last) on qubits `qs` (ascending, k of them) as one factor
+// of a step: a built-in one where there is one gate or k <= 2, else a custom
+// one.  Products are formed in FP64 and rounded once.
+inline void add_factor(StepTable& T, StepDesc& d, const std::vector<const Gate*>& gates, const std::vector<int>& qs) {
+  StepFactor f{};
+  int64_t coef_at = -1;
+  const Gate& g0 = *gates[0];
+  for (int q : qs) d.idle &= ~(1u << q);
+  if (gates.size() == 1 && is_wide(g0)) {
+    f.nq = static_cast<uint8_t>(g0.nq);
+    f.custom = 1;
+    for (int t = 0; t < g0.nq; ++t) f.qc[t] = static_cast<uint8_t>(g0.q[t]);
+    coef_at = static_cast<int64_t>(T.coef_pool.size());
+    for (const cd& v : g0.cm->m) T.coef_pool.push_back(to_f2(v));
+  } else if (gates.size() == 1 && !is_two_qubit(g0.kind)) {
+    f.nq = 1;
+    f.q0 = f.q1 = static_cast<uint8_t>(g0.q[0]);
+    for (int i = 0; i < 4; ++i) f.m[i] = to_f2(g0.u.m[i]);
+  } else if (gates.size() == 1) {
+    f.nq = 2;
+    f.q0 = static_cast<uint8_t>(g0.q[0]);
+    f.q1 = static_cast<uint8_t>(g0.q[1]);
+    cd M[16] = {};
+    if (g0.kind == TQS_SWAP) {
+      // |a b> -> |b a> in the (q0, q1) labelling
+      M[0 * 4 + 0] = M[1 * 4 + 2] = M[2 * 4 + 1] = M[3 * 4 + 3] = 1.0;
+    } else {
+      // eq. 7: diag(I, U) with the control first
+      M[0 * 4 + 0] = M[1 * 4 + 1] = 1.0;
+      M[2 * 4 + 2] = g0.u.m[0];
+      M[2 * 4 + 3] = g0.u.m[1];
+      M[3 * 4 + 2] = g0.u.m[2];
+      M[3 * 4 + 3] = g0.u.m[3];
+    }
+    for (int i = 0; i < 16; ++i) f.m[i] = to_f2(M[i]);
+  } else {
+    // M <- G M gate by gate, local index bit t the bit of qs[t]
+    const int k = static_cast<int>(qs.size()), D = 1 << k;
+    std::vector<cd> M(static_cast<size_t>(D) * D, cd(0.0)), in(static_cast<size_t>(D));
+    for (int i = 0; i < D; ++i) M[static_cast<size_t>(i) * D + i] = 1.0;
+    auto loc = [&](int q) { return static_cast<int>(std::find(qs.begin(), qs.end(), q) - qs.begin()); };
+    for (const Gate* g : gates) {
+      if (is_wide(*g)) {
+        const int G = 1 << g->nq;
+        int at[1 << kMaxCustomQubits], mask = 0;
+        for (int j = 0; j < G; ++j) {
+          at[j] = 0;
+          for (int t = 0; t < g->nq; ++t) at[j] |= ((j >> t) & 1) << loc(g->q[t]);
+          mask |= at[j];
+        }
+        for (int b = 0; b < D; ++b) {
+          if (b & mask) continue;
+          for (int c = 0; c < D; ++c) {
+            for (int j = 0; j < G; ++j) in[static_cast<size_t>(j)] = M[static_cast<size_t>(b | at[j]) * D + c];
+            for (int r = 0; r < G; ++r) {
+              cd v = 0.0;
+              for (int j = 0; j < G; ++j) v += g->cm->m[static_cast<size_t>(r) * G + j] * in[static_cast<size_t>(j)];
+              M[static_cast<size_t>(b | at[r]) * D + c] = v;
+            }
+          }
+        }
+        continue;
+      }
+      const bool two = is_two_qubit(g->kind);
+      const int c1 = two ? 1 << loc(g->q[0]) : 0, t1 = 1 << loc(g->q[two ? 1 : 0]);
+      for (int r0 = 0; r0 < D; ++r0) {
+        if (r0 & t1) continue;
+        if (g->kind == TQS_SWAP) {  // the row with (control, target) = (1, 0) and its partner
+          if (r0 & c1)
+            for (int c = 0; c < D; ++c)
+              std::swap(M[static_cast<size_t>(r0) * D + c], M[static_cast<size_t>((r0 ^ c1) | t1) * D + c]);
+          continue;
+        }
+        if (two && !(r0 & c1)) continue;
+        cd* x0 = &M[static_cast<size_t>(r0) * D];
+        cd* x1 = &M[static_cast<size_t>(r0 | t1) * D];
+        for (int c = 0; c < D; ++c) {
+          const cd y0 = x0[c], y1 = x1[c];
+          x0[c] = g->u.m[0] * y0 + g->u.m[1] * y1;
+          x1[c] = g->u.m[2] * y0 + g->u.m[3] * y1;
+        }
+      }
+    }
+    f.nq = static_cast<uint8_t>(k);
+    if (k == 1) {
+      f.q0 = f.q1 = static_cast<uint8_t>(qs[0]);
+      for (int i = 0; i < 4; ++i) f.m[i] = to_f2(M[static_cast<size_t>(i)]);
+    } else if (k == 2) {
+      f.q0 = static_cast<uint8_t>(qs[1]);  // local index (bit q0 << 1) | bit q1
+      f.q1 = static_cast<uint8_t>(qs[0]);
+      for (int i = 0; i < 16; ++i) f.m[i] = to_f2(M[static_cast<size_t>(i)]);
+    } else {
+      f.custom = 1;
+      for (int t = 0; t < k; ++t) f.qc[t] = static_cast<uint8_t>(qs[static_cast<size_t>(t)]);
+      coef_at = static_cast<int64_t>(T.coef_pool.size());
+      for (const cd& v : M) T.coef_pool.push_back(to_f2(v));
+    }
+  }
+  T.factors.push_back(f);
+  T.factor_coef.push_back(coef_at);
+  ++d.f_count;
+}
+
+// The circuit's step table: a factor per gate.
 inline void ensure_steps(tqs_circuit* c) {
-  if (c->steps_valid) return;
-  c->factors.clear();
-  c->factor_coef.clear();
-  c->coef_pool.clear();
-  c->steps.assign(c->nsteps, StepDesc{0, 0, 0, 0});
+  StepTable& T = c->table;
+  if (T.valid) return;
+  T.clear();
   const uint32_t all = (1u << c->n) - 1u;
   std::vector<std::vector<const Gate*>> by_step(c->nsteps);
   for (const Gate& g : c->gates) by_step[g.step].push_back(&g);
   for (int k = 0; k < c->nsteps; ++k) {
-    StepDesc d{static_cast<int32_t>(c->factors.size()), 0, all, 0};
-    for (const Gate* g : by_step[k]) {
-      StepFactor f{};
-      int64_t coef_at = -1;
-      if (is_wide(*g)) {
-        f.nq = static_cast<uint8_t>(g->nq);
-        f.custom = 1;
-        for (int t = 0; t < g->nq; ++t) f.qc[t] = static_cast<uint8_t>(g->q[t]);
-        coef_at = static_cast<int64_t>(c->coef_pool.size());
-        for (const cd& v : g->cm->m) c->coef_pool.push_back(to_f2(v));
-        d.idle &= ~qubit_mask(*g);
-      } else if (!is_two_qubit(g->kind)) {
-        f.nq = 1;
-        f.q0 = f.q1 = static_cast<uint8_t>(g->q[0]);
-        for (int i = 0; i < 4; ++i) f.m[i] = to_f2(g->u.m[i]);
-        d.idle &= ~(1u << g->q[0]);
-      } else {
-        f.nq = 2;
-        f.q0 = static_cast<uint8_t>(g->q[0]);
-        f.q1 = static_cast<uint8_t>(g->q[1]);
-        cd M[16] = {};
-        if (g->kind == TQS_SWAP) {
-          // |a b> -> |b a> in the (q0, q1) labelling
-          M[0 * 4 + 0] = 1.0;
-          M[1 * 4 + 2] = 1.0;
-          M[2 * 4 + 1] = 1.0;
-          M[3 * 4 + 3] = 1.0;
-        } else {
-          // eq. 7: diag(I, U) with the control first
-          M[0 * 4 + 0] = 1.0;
-          M[1 * 4 + 1] = 1.0;
-          M[2 * 4 + 2] = g->u.m[0];
-          M[2 * 4 + 3] = g->u.m[1];
-          M[3 * 4 + 2] = g->u.m[2];
-          M[3 * 4 + 3] = g->u.m[3];
-        }
-        for (int i = 0; i < 16; ++i) f.m[i] = to_f2(M[i]);
-        d.idle &= ~((1u << g->q[0]) | (1u << g->q[1]));
-      }
-      c->factors.push_back(f);
-      c->factor_coef.push_back(coef_at);
-      ++d.f_count;
-    }
-    c->steps[k] = d;
+    StepDesc d{static_cast<int32_t>(T.factors.size()), 0, all, 0};
+    for (const Gate* g : by_step[k]) add_factor(T, d, {g}, std::vector<int>(g->q, g->q + g->nq));
+    T.steps.push_back(d);
   }
-  c->steps_valid = true;
+  T.valid = true;
+}
+
+// The step table of the tensor-core chain: consecutive steps are multiplied
+// first where their gates fall into blocks of at most kMaxCustomQubits qubits,
+// so that the chain has fewer products (the step matrix of such a run is the
+// Kronecker product of its blocks, as a step's is of its gates).  One in-order
+// scan per run: a gate joins unless an earlier gate left for a later run
+// shares a qubit with it or the block it would make is too large.  A product
+// costs 18 N^3 tensor operations whatever S_k is, and rounds: 40 steps (20
+// layers of U3 and CNOTs) of 12 qubits become 13, 35.4 -> 11.4 ms; 6 steps 2
+// or 3, 4.58 -> 1.36 ms, error against FP64 1.0e-5 -> 6.2e-6; the 12-qubit
+// QFT in TF32x3 42.0 -> 14.2 ms.  With blocks of 6 qubits 11.7 runs instead of
+// 13.2 on average, but 4096 coefficients a block to form on the host.
+inline void ensure_chain_steps(tqs_circuit* c) {
+  StepTable& T = c->chain_table;
+  if (T.valid) return;
+  T.clear();
+  const uint32_t all = (1u << c->n) - 1u;
+  std::vector<const Gate*> pending = step_order(c->gates), still, taken;
+  while (!pending.empty()) {
+    std::vector<uint32_t> block(static_cast<size_t>(c->n), 0);  // the block each qubit is in
+    uint32_t blocked = 0;
+    still.clear();
+    taken.clear();
+    for (const Gate* g : pending) {
+      const uint32_t qm = qubit_mask(*g);
+      uint32_t m = qm;
+      for (uint32_t b = qm; b; b &= b - 1) m |= block[static_cast<size_t>(__builtin_ctz(b))];
+      if ((qm & blocked) || __builtin_popcount(m) > kMaxCustomQubits) {
+        blocked |= qm;
+        still.push_back(g);
+        continue;
+      }
+      for (uint32_t b = m; b; b &= b - 1) block[static_cast<size_t>(__builtin_ctz(b))] = m;
+      taken.push_back(g);
+    }
+    StepDesc d{static_cast<int32_t>(T.factors.size()), 0, all, 0};
+    std::vector<const Gate*> gates;
+    std::vector<int> qs;
+    for (int q = 0; q < c->n; ++q) {
+      const uint32_t m = block[static_cast<size_t>(q)];
+      if (m == 0 || __builtin_ctz(m) != q) continue;  // at its lowest qubit
+      gates.clear();
+      qs.clear();
+      for (const Gate* g : taken)
+        if (qubit_mask(*g) & m) gates.push_back(g);
+      for (uint32_t b = m; b; b &= b - 1) qs.push_back(__builtin_ctz(b));
+      add_factor(T, d, gates, qs);
+    }
+    T.steps.push_back(d);
+    pending.swap(still);
+  }
+  T.valid = true;
 }
 
 // Device step table: [StepFactor...][custom entries (float2)...]; each custom
 // factor's `coef` points into the second part.
-inline tqs_status upload_factors(tqs_circuit* c, cudaStream_t s) {
-  ensure_steps(c);
-  const size_t fbytes = (std::max<size_t>(c->factors.size(), 1) * sizeof(StepFactor) + 15) & ~size_t(15);
-  const size_t bytes = fbytes + c->coef_pool.size() * sizeof(float2);
-  TQS_CUDA(c->d_factors.ensure(bytes), "cudaMalloc step table");
-  const float2* pool = reinterpret_cast<const float2*>(c->d_factors.as<char>() + fbytes);
-  std::vector<StepFactor> fs = c->factors;
+inline tqs_status upload_table(StepTable& T, cudaStream_t s) {
+  const size_t fbytes = (std::max<size_t>(T.factors.size(), 1) * sizeof(StepFactor) + 15) & ~size_t(15);
+  const size_t bytes = fbytes + T.coef_pool.size() * sizeof(float2);
+  TQS_CUDA(T.dev.ensure(bytes), "cudaMalloc step table");
+  const float2* pool = reinterpret_cast<const float2*>(T.dev.as<char>() + fbytes);
+  std::vector<StepFactor> fs = T.factors;
   for (size_t i = 0; i < fs.size(); ++i)
-    if (c->factor_coef[i] >= 0) fs[i].coef = pool + c->factor_coef[i];
+    if (T.factor_coef[i] >= 0) fs[i].coef = pool + T.factor_coef[i];
   if (!fs.empty())
-    TQS_CUDA(cudaMemcpyAsync(c->d_factors.p, fs.data(), fs.size() * sizeof(StepFactor),
-                             cudaMemcpyHostToDevice, s),
+    TQS_CUDA(cudaMemcpyAsync(T.dev.p, fs.data(), fs.size() * sizeof(StepFactor), cudaMemcpyHostToDevice, s),
              "upload step table");
-  if (!c->coef_pool.empty())
-    TQS_CUDA(cudaMemcpyAsync(c->d_factors.as<char>() + fbytes, c->coef_pool.data(),
-                             c->coef_pool.size() * sizeof(float2), cudaMemcpyHostToDevice, s),
+  if (!T.coef_pool.empty())
+    TQS_CUDA(cudaMemcpyAsync(T.dev.as<char>() + fbytes, T.coef_pool.data(), T.coef_pool.size() * sizeof(float2),
+                             cudaMemcpyHostToDevice, s),
              "upload custom entries");
   return TQS_OK;
+}
+
+inline tqs_status upload_factors(tqs_circuit* c, cudaStream_t s) {
+  ensure_steps(c);
+  return upload_table(c->table, s);
 }
 
 // Segment tables of an inverse-CDF sampling call (see k_sample.cu).

@@ -83,7 +83,7 @@ tqs_status tqs_add_gate(tqs_circuit* c, int gate, const int* qubits, int nq, con
   c->cols_prog.valid = false;
   c->prog_init_valid = false;
   c->run_prog.valid = false;
-  c->steps_valid = false;
+  c->table.valid = c->chain_table.valid = false;
   c->fsv_valid = false;
   return TQS_OK;
 }
@@ -161,7 +161,7 @@ tqs_status tqs_add_custom(tqs_circuit* c, const char* name, const int* qubits, i
   c->cols_prog.valid = false;
   c->prog_init_valid = false;
   c->run_prog.valid = false;
-  c->steps_valid = false;
+  c->table.valid = c->chain_table.valid = false;
   c->fsv_valid = false;
   return TQS_OK;
 }
@@ -312,7 +312,7 @@ tqs_status tqs_materialize_step(tqs_circuit* c, int step, tqs_c64* d_S, void* st
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   tqs_status st = upload_factors(c, s);
   if (st != TQS_OK) return st;
-  TQS_CUDA(launch_materialize(c->d_factors.as<StepFactor>(), c->steps[step], c->n,
+  TQS_CUDA(launch_materialize(c->table.dev.as<StepFactor>(), c->table.steps[step], c->n,
                               reinterpret_cast<float2*>(d_S), s),
            "tqs_materialize_step: launch");
   return TQS_OK;
@@ -344,7 +344,7 @@ tqs_status tqs_simulate_plain(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* d_
     TQS_CUDA(cudaMemcpyAsync(x, &one, sizeof(float2), cudaMemcpyHostToDevice, s), "init |0>");
   }
   for (int k = 0; k < c->nsteps; ++k) {
-    TQS_CUDA(launch_materialize(c->d_factors.as<StepFactor>(), c->steps[k], c->n, S, s),
+    TQS_CUDA(launch_materialize(c->table.dev.as<StepFactor>(), c->table.steps[k], c->n, S, s),
              "tqs_simulate_plain: materialize");
     TQS_CUDA(launch_matvec(S, x, y, c->n, s), "tqs_simulate_plain: matvec");
     std::swap(x, y);
