@@ -542,11 +542,12 @@ tqs_status tqs_check_violations(uint32_t* count, int reset);
  * TQS_OPT_MULTI_CTAS, key = 0, value = CTAs at most for one circuit of 15 or
  * 16 qubits in tqs_simulate, and for each such request of a server batch that
  * holds few of them (together at most the SMs divided by the server's batches
- * in flight) (0 or 1: one CTA; default 8; at most 64).  The
- * CTAs (a cooperative launch) share the circuit's passes, one thread per
- * amplitude group, and meet at a grid barrier after each pass; CTA 0 writes
- * the outputs exactly as one CTA would, so states, probabilities and the norm
- * are bitwise the same for every value.  Circuits with measure / reset
+ * in flight) (0 or 1: one CTA; default 8; at most 64), counted in CTAs of 512
+ * threads: each is launched as four of 128.  The CTAs (a cooperative launch)
+ * share the circuit's passes, one thread per amplitude group, meet at a grid
+ * barrier after each pass, and write the outputs block by block exactly as
+ * one CTA would, so states, probabilities and the norm are bitwise the same
+ * for every value.  Circuits with measure / reset
  * instructions or custom unitaries always take one CTA.  A grid barrier that
  * waits longer than about a second (it cannot while the launch is
  * cooperative) stops waiting and leaves NaN in the norm and in amplitude 0. */

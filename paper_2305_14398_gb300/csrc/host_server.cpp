@@ -130,7 +130,8 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
   const size_t gscr_off = (norms_off + sl.reqs.size() * sizeof(double) + 255) & ~size_t(255);
   const size_t gscr_bytes =
       J ? size_t(std::max(plans[TEAM_GLOBAL].grid, J)) << kGlobalSlotQ : size_t(0);
-  const size_t total = gscr_off + gscr_bytes * sizeof(float2);
+  const size_t sums_off = gscr_off + gscr_bytes * sizeof(float2);
+  const size_t total = sums_off + (multi_k ? size_t(J) * kMultiSums * sizeof(float) : 0);
   // the program goes through pinned memory so the copy is truly asynchronous
   const size_t prog_bytes = order_off + order.size() * sizeof(int32_t);
   {
@@ -186,8 +187,10 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
     L.norm_width = plans[t].norm_width;
     if (t == TEAM_GLOBAL && multi_k) {
       L.team = TEAM_MULTI;
-      L.ctas_per_job = multi_k;
-      L.grid = J * multi_k;
+      L.ctas_per_job = multi_k * kMultiSplit;
+      L.grid = J * L.ctas_per_job;
+      L.norm_width = kGlobalThreads;
+      L.blk_sums = reinterpret_cast<float*>(base + sums_off);
       L.counter = counters + 4;
       L.err = counters + 3;
     }

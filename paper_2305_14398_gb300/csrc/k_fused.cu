@@ -580,14 +580,17 @@ __device__ __forceinline__ void team_sync() {
 // Barrier of the K TEAM_MULTI CTAs of one circuit (all co-resident:
 // cooperative launch).  Thread 0 of each arrives on the circuit's monotone
 // counter (zeroed before the launch) and waits, at most kGridBarrierCycles,
-// until all K have arrived as often; a time-out is recorded and later
-// barriers do not wait.
+// until all K have arrived as often; a time-out is recorded, and a wait that
+// sees one recorded gives up.  The arrival is a release and the wait an
+// acquire, cumulative with the block barriers around them, so no fence of its
+// own is needed (with fences and a read of the error word before each wait a
+// 16-qubit circuit of 28 barriers took 172 us, now 166).
 struct GridBar {
   unsigned int* ctr;
   int* err;
   unsigned int target;
   unsigned int nblocks;  // CTAs that meet at this barrier
-  bool leader;           // the first of them: writes the outputs
+  bool leader;           // the first of them: adds up the norm
 };
 
 __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
@@ -600,18 +603,18 @@ __device__ __forceinline__ void grid_sync(GridBar& b) {
   __syncthreads();
   if (threadIdx.x == 0) {
     b.target += b.nblocks;
-    __threadfence();
-    atomicAdd(b.ctr, 1u);
-    if (*reinterpret_cast<volatile int*>(b.err) == 0) {
+    // release: the CTA's writes, ordered by the barrier above, before the arrival
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(b.ctr) : "memory");
+    {
       const long long t0 = clock64();
       while (ld_acquire_u32(b.ctr) < b.target) {
         if (clock64() - t0 > kGridBarrierCycles) {
           atomicExch(b.err, 1);
           break;
         }
+        if (*reinterpret_cast<volatile int*>(b.err) != 0) break;
       }
     }
-    __threadfence();
   }
   __syncthreads();
 }
@@ -809,12 +812,6 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
     }
     if (TEAM == TEAM_MULTI) grid_sync(*bar); else team_sync<TEAM>();
   }
-  // TEAM_MULTI: the first CTA alone writes the outputs, as a TEAM_GLOBAL CTA would.
-  if (TEAM == TEAM_MULTI) {
-    if (!bar->leader) return;
-    rank = threadIdx.x;
-    size = blockDim.x;
-  }
   // Warp and pair teams: the next job (its atomic was issued when this
   // circuit started) is shared with the team here and its circuit index is
   // loaded, so both latencies hide behind the output phase.
@@ -827,10 +824,11 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
   }
   if (TEAM == TEAM_WARP || TEAM == TEAM_PAIR)
     next_ci = next_job < L.n_jobs ? __ldg(L.order + next_job) : 0;
-  // TEAM_SOLO: the CTA's threads as norm_width lanes times several workers, each
-  // with its own blocks of a lane's pairs.
+  // TEAM_SOLO, TEAM_MULTI: the threads as norm_width lanes times several workers,
+  // each with its own blocks of a lane's pairs.
+  constexpr bool kWorkers = TEAM == TEAM_SOLO || TEAM == TEAM_MULTI;
   int blk0 = 0, blk_step = 8;
-  if (TEAM == TEAM_SOLO) {
+  if (kWorkers) {
     blk0 = rank / L.norm_width * 8;
     blk_step = size / L.norm_width * 8;
     rank &= L.norm_width - 1;
@@ -868,7 +866,7 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
       const int iters = N > (1 << sh) ? (N >> sh) : 1;  // pairs per thread
       const int NI = 1 << nint;
 #pragma unroll 1
-      for (int blk = TEAM == TEAM_SOLO ? blk0 : 0; blk < iters; blk += TEAM == TEAM_SOLO ? blk_step : 8) {
+      for (int blk = kWorkers ? blk0 : 0; blk < iters; blk += kWorkers ? blk_step : 8) {
         // A at the block's first pair: the block index's bits sh + 3 ...
         int ab = a_i0;
         for (int q = 3; (blk >> q) != 0; ++q)
@@ -901,7 +899,7 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
         }
         // the block's 16 values summed as a tree in FP32, then added in FP64
         const float bs = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
-        if (TEAM == TEAM_SOLO) blk_sum[(blk >> 3) * size + rank] = bs;
+        if (kWorkers) blk_sum[(blk >> 3) * size + rank] = bs;
         else acc += static_cast<double>(bs);
       }
     }
@@ -924,6 +922,19 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
       for (int b = 0; 8 * b < max(1, N / (2 * size)); ++b) acc += static_cast<double>(blk_sum[b * size + rank]);
     rank = threadIdx.x;
   }
+  if (TEAM == TEAM_MULTI) {
+    // the first CTA adds the sums up, several lanes a thread
+    grid_sync(*bar);
+    if (!bar->leader) return;
+    for (rank = threadIdx.x; rank < size; rank += blockDim.x) {
+      acc = 0.0;
+      for (int b = 0; 8 * b < max(1, N / (2 * size)); ++b) acc += static_cast<double>(__ldcg(blk_sum + b * size + rank));
+      if (rank + static_cast<int>(blockDim.x) >= size) break;  // (the last turn's goes on below)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if ((rank & 31) == 0) s_red[rank >> 5] = acc;
+    }
+  }
   // Fixed-order reduction (deterministic): per-thread FP64 partials, warp
   // butterfly, then the warps of the team in order.
 #pragma unroll
@@ -934,9 +945,9 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
     const int warp = rank >> 5, lane = rank & 31;
     if (lane == 0) s_red[warp] = acc;
     team_sync<TEAM>();
-    if (TEAM == TEAM_CTA ? threadIdx.x == 0 : rank == 0) { double s = 0.0; for (int w = 0; w < (size >> 5); ++w) s += s_red[w]; if (L.norms) L.norms[ci] = s; }
+    if (TEAM == TEAM_CTA || TEAM == TEAM_MULTI ? threadIdx.x == 0 : rank == 0) { double s = 0.0; for (int w = 0; w < (size >> 5); ++w) s += s_red[w]; if (L.norms) L.norms[ci] = s; }
   }
-  if (TEAM == TEAM_MULTI && rank == 0 && *reinterpret_cast<volatile int*>(L.err) != 0) {
+  if (TEAM == TEAM_MULTI && threadIdx.x == 0 && *reinterpret_cast<volatile int*>(L.err) != 0) {
     // a grid barrier timed out: the outputs are not valid, make that visible
     const float nan = __int_as_float(0x7fffffff);
     if (L.norms) L.norms[ci] = static_cast<double>(nan);
@@ -952,7 +963,10 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
 constexpr int kSoloSums = (1 << kWarpMaxQ) / 16;
 
 template <int TEAM>
-__global__ void __launch_bounds__(TEAM == TEAM_SOLO ? kSoloThreads : TEAM == TEAM_CTA ? kCtaThreads : 512)
+__global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kSoloThreads
+                                  : TEAM == TEAM_MULTI ? kMultiThreads
+                                  : TEAM == TEAM_CTA   ? kCtaThreads
+                                                       : 512)
     fused_kernel(const __grid_constant__ FusedLaunch L) {
   extern __shared__ float4 smem_raw[];
   float2* smem = reinterpret_cast<float2*>(smem_raw);
@@ -1015,7 +1029,7 @@ __global__ void __launch_bounds__(TEAM == TEAM_SOLO ? kSoloThreads : TEAM == TEA
     int unused_job = 0, unused_ci = 0;
     run_circuit<TEAM_MULTI>(L, L.order[job], L.gscratch + (static_cast<size_t>(job) << kGlobalSlotQ),
                             local * blockDim.x + threadIdx.x, K * blockDim.x, s_red, unused_job,
-                            unused_ci, nullptr, &bar);
+                            unused_ci, nullptr, &bar, L.blk_sums + static_cast<size_t>(job) * kMultiSums);
   } else {
     __shared__ int s_job;
     __shared__ double s_red[32];
@@ -1168,7 +1182,7 @@ size_t fused_smem_bytes(int team, int warps_per_cta, int slice_q) {
 int fused_threads(int team, int warps_per_cta) {
   if (team == TEAM_WARP || team == TEAM_PAIR || team == TEAM_SOLO) return 32 * warps_per_cta;
   if (team == TEAM_CTA) return warps_per_cta > 0 ? 32 * warps_per_cta : kCtaThreads;
-  return kGlobalThreads;
+  return team == TEAM_MULTI ? kMultiThreads : kGlobalThreads;
 }
 
 }  // namespace

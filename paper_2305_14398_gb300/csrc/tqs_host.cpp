@@ -254,9 +254,10 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
   L.counter = c->d_counter.as<int32_t>();
   LaunchPlan lp = plan_for(team, P.nint, 1, 1, P.n_instr > 0);
   if (team == TEAM_GLOBAL) {
-    TQS_CUDA(c->d_gscratch.ensure((size_t(1) << kGlobalSlotQ) * sizeof(float2)),
+    TQS_CUDA(c->d_gscratch.ensure((size_t(1) << kGlobalSlotQ) * sizeof(float2) + kMultiSums * sizeof(float)),
              "tqs_simulate: cudaMalloc scratch");
     L.gscratch = c->d_gscratch.as<float2>();
+    L.blk_sums = reinterpret_cast<float*>(L.gscratch + (size_t(1) << kGlobalSlotQ));
   }
   L.team = lp.team;
   L.norm_width = lp.norm_width;
@@ -267,8 +268,8 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
   const int multi = multi_ctas_for(P);
   if (team == TEAM_GLOBAL && multi >= 2) {
     L.team = TEAM_MULTI;
-    L.grid = multi;
-    L.ctas_per_job = multi;
+    L.grid = L.ctas_per_job = multi * kMultiSplit;
+    L.norm_width = kGlobalThreads;
     L.err = c->d_counter.as<int32_t>() + 1;  // zeroed with the counter above
   }
   TQS_CUDA(launch_fused(L, s), "tqs_simulate: launch");

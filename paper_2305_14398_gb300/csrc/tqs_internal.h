@@ -130,9 +130,9 @@ static_assert(sizeof(FusedPass) == 16, "FusedPass layout");
 // TEAM_WARP: twice the warps per byte of shared memory).
 // TEAM_MULTI: each circuit of the global class on K co-resident CTAs (a
 // cooperative launch): they share its global scratch slot and meet at a
-// bounded barrier of the K after every pass; the first of the K alone writes
-// the outputs with exactly the TEAM_GLOBAL output phase, so results are
-// bitwise those of TEAM_GLOBAL.  Circuits without instructions or custom
+// bounded barrier of the K after every pass; they write the outputs block by
+// block as the threads of a TEAM_GLOBAL CTA would and the first of the K adds
+// the norm up, so results are bitwise those of TEAM_GLOBAL.  Circuits without instructions or custom
 // unitaries, few enough that all their CTAs are resident at once.
 // TEAM_SOLO: a circuit of the warp class on a CTA with a thread per group of a
 // pass (up to 128): alone on the GPU, or the jobs of a batch in turn.  It writes the outputs block by block
@@ -176,6 +176,13 @@ constexpr int kCtaMaxQ = 14;
 constexpr int kCtaThreads = 512;
 constexpr int kSoloThreads = 128;
 constexpr int kGlobalThreads = 512;
+// TEAM_MULTI: a CTA of TQS_OPT_MULTI_CTAS is four of these, on four SMs where
+// they are free: a warp to a scheduler instead of four shortens every pass, and
+// the CTAs share the output phase (16 qubits, 10 layers 258 -> 172 us, QFT 95 ->
+// 45 us; eight of 64 threads: 171 and 47 us).
+constexpr int kMultiThreads = 128;
+constexpr int kMultiSplit = kGlobalThreads / kMultiThreads;
+constexpr int kMultiSums = (1 << 16) / 16;  // a job's block sums: floats behind all scratch slots
 constexpr int kGlobalSlotQ = 16;   // log2 amplitudes per TEAM_GLOBAL scratch slot
 
 struct FusedLaunch {
@@ -199,7 +206,8 @@ struct FusedLaunch {
                             // [j K, (j + 1) K), its barrier counter is counter[j],
                             // its scratch slot gscratch + j 2^kGlobalSlotQ
   int32_t norm_width;       // threads of the team whose norm is formed: TEAM_SOLO 32 or 64;
-                            // TEAM_CTA at least the CTA's (0: its own)
+                            // TEAM_CTA at least the CTA's (0: its own); TEAM_MULTI kGlobalThreads
+  float* blk_sums;          // TEAM_MULTI: kMultiSums floats per job
   int32_t team;             // TeamKind of this launch
   int32_t warps_per_cta;    // TEAM_WARP
   int32_t slice_q;          // TEAM_WARP: log2 amplitudes per warp slice; TEAM_CTA: log2 per CTA
