@@ -284,7 +284,7 @@ struct Program {
   // left here for the program that follows (else it is applied, and 1).
   cd carry = 1.0;
   bool defer = false;
-  bool rotations = false;  // holds general gates (as rotations)
+  bool rotations = false;  // holds rotations (general gates) or their phases
   double cost = 0.0;
   // Empty the program for reuse (keeps the vectors' capacity).
   void reset() {
@@ -1224,6 +1224,7 @@ struct tqs_batch {
   }
   std::vector<int32_t> order;    // the jobs of each kind in turn
   int n_kind[kKinds] = {};
+  bool rotations[kKinds] = {};   // some circuit of the kind holds rotations
   int max_nint[kKinds] = {4, 4, 4, 4, 4, 4, 4, 4};
   DevBuf d_img;                  // image + order + counters
   size_t order_off = 0, counter_off = 0;

@@ -1008,7 +1008,6 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
   if (!prepared) {
     fused_tls.clear();
     split = prepare_gates(n, gs, fused_tls, P.carry, absorb ? &flips : nullptr);
-    P.rotations = split;
   }
 
   std::vector<uint32_t>& qmask = qmask_tls;
@@ -1080,6 +1079,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     // the phase diag(1, alpha) that a rotation leaves on its own target
     auto emit_phase = [&](cd alpha, int tl) {
       FusedOp op{};
+      P.rotations = true;
       op.c = 1;  // hi + lo, multiplied in at once
       op.code = static_cast<uint8_t>(OPC_DLN + tl);
       op.fbit = op.tbit = 0xFF;
@@ -1122,6 +1122,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
         } else if (r.c < 0) {  // dense, or anti-diagonal other than X: a rotation
           const RotSplit rs = split_rotation(u, false);
           carry *= rs.gamma * rs.scale;
+          P.rotations = true;
           op.code = static_cast<uint8_t>(OPC_DENSE + tl);
           op.hc = make_float2(rs.tau, 0.f);
           const float2 b = to_f2(rs.beta), bl = to_f2(rs.beta - cd(b.x, b.y));

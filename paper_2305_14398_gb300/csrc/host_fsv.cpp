@@ -245,6 +245,7 @@ tqs_status tqs_simulate_fsv(tqs_circuit* c, tqs_c64* d_state, void* stream) {
     F.nfar = info.nfar;
     std::memcpy(F.far, info.far, sizeof(F.far));
     L.circs = circs + k;
+    L.no_rot = !c->fsv.progs[k].rotations;
     TQS_CUDA(launch_fsv_tile(L, F, s), "tqs_simulate_fsv: launch");
   }
   return TQS_OK;

@@ -280,7 +280,9 @@ __device__ __forceinline__ float2 f2(unsigned x, unsigned y) {
 // one place each 314 us).  SMALL keeps also the hi + lo phase in one place;
 // the other teams' warps run the same ops at about the same time and take one
 // branch less instead (n = 14 batch 702 -> 694 us).
-template <bool SMALL>
+// ROT: the programs may hold rotations.  Those that hold none (the paper's) take
+// kernels without their code.
+template <bool SMALL, bool ROT>
 __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restrict__ ops,
                                         uint32_t count, int base, float scale) {
   Pending pd;
@@ -298,14 +300,14 @@ __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restri
     const int fbit = (q0.y >> 8) & 0xff;
     if (fbit != 0xff && !((base >> fbit) & 1)) continue;  // a far control is 0 here
     // a phase that a rotation left on its target: hi + lo, at once
-    const bool phase_op = code >= OPC_DLN && code < OPC_DFL && ((q0.x >> 16) & 0xff);
+    const bool phase_op = ROT && code >= OPC_DLN && code < OPC_DFL && ((q0.x >> 16) & 0xff);
     if (code < OPC_DLN || phase_op) {
       // target local position t, or the mask hm of a Hadamard's positions;
       // exchanges act on the pairs in `act`
       int t = code & 3;
       unsigned act = q0.y >> 16;
       const bool had = code < OPC_X || code == OPC_HMASK;
-      const bool rot = code >= OPC_DENSE && code < OPC_CDENSE;
+      const bool rot = ROT && code >= OPC_DENSE && code < OPC_CDENSE;
       unsigned hm = 1u << t;
       if (code == OPC_HMASK) hm = (q0.x >> 8) & 15;
       if (code >= OPC_XL && code < OPC_ANTI) {
@@ -729,7 +731,7 @@ __device__ __noinline__ void wide_pass(const FusedLaunch& L, int nint, int k, ui
   team_sync<TEAM>();
 }
 
-template <int TEAM>
+template <int TEAM, bool ROT>
 __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, int size,
                             double* s_red, int& next_job, int& next_ci, int* s_slot,
                             GridBar* bar = nullptr, float* blk_sum = nullptr) {
@@ -805,7 +807,7 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
           a[j] = ld_state<TEAM>(&st[TQS_IX(sb ^ ((j & 1) ? w0 : 0) ^ ((j & 2) ? w1 : 0) ^ ((j & 4) ? w2 : 0) ^ ((j & 8) ? w3 : 0), 1 << nint)]);
         }
       }
-      run_ops<TEAM == TEAM_WARP || TEAM == TEAM_PAIR>(a, ops, count, base, scale);
+      run_ops<TEAM == TEAM_WARP || TEAM == TEAM_PAIR, ROT>(a, ops, count, base, scale);
 #pragma unroll
       for (int j = 0; j < 16; ++j)
         st[TQS_IX(sb ^ ((j & 1) ? w0 : 0) ^ ((j & 2) ? w1 : 0) ^ ((j & 4) ? w2 : 0) ^ ((j & 8) ? w3 : 0), 1 << nint)] = a[j];
@@ -962,7 +964,7 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
 // (and at least one per lane of the 64).
 constexpr int kSoloSums = (1 << kWarpMaxQ) / 16;
 
-template <int TEAM>
+template <int TEAM, bool ROT>
 __global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kSoloThreads
                                   : TEAM == TEAM_MULTI ? kMultiThreads
                                   : TEAM == TEAM_CTA   ? kCtaThreads
@@ -986,7 +988,7 @@ __global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kSoloThreads
     while (job < L.n_jobs) {
       int next_job = rank == 0 ? atomicAdd(L.counter, 1) : 0;
       int next_ci = 0;
-      run_circuit<TEAM_PAIR>(L, ci, st, rank, 64, s_red[pair], next_job, next_ci, &s_job[pair]);
+      run_circuit<TEAM_PAIR, ROT>(L, ci, st, rank, 64, s_red[pair], next_job, next_ci, &s_job[pair]);
       job = next_job;
       ci = next_ci;
     }
@@ -999,7 +1001,7 @@ __global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kSoloThreads
     while (job < L.n_jobs) {
       int next_job = lane == 0 ? atomicAdd(L.counter, 1) : 0;
       int next_ci = 0;
-      run_circuit<TEAM_WARP>(L, ci, st, lane, 32, nullptr, next_job, next_ci, nullptr);
+      run_circuit<TEAM_WARP, ROT>(L, ci, st, lane, 32, nullptr, next_job, next_ci, nullptr);
       job = next_job;
       ci = next_ci;
     }
@@ -1016,7 +1018,7 @@ __global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kSoloThreads
         job = s_job;
         if (job >= L.n_jobs) break;
       }
-      run_circuit<TEAM_SOLO>(L, L.order[job], smem, threadIdx.x, blockDim.x, s_red, unused_job, unused_ci, nullptr,
+      run_circuit<TEAM_SOLO, ROT>(L, L.order[job], smem, threadIdx.x, blockDim.x, s_red, unused_job, unused_ci, nullptr,
                              nullptr, blk_sum);
       if (L.counter == nullptr) break;
     }
@@ -1027,7 +1029,7 @@ __global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kSoloThreads
     GridBar bar{reinterpret_cast<unsigned int*>(L.counter) + job, L.err, 0u,
                 static_cast<unsigned int>(K), local == 0};
     int unused_job = 0, unused_ci = 0;
-    run_circuit<TEAM_MULTI>(L, L.order[job], L.gscratch + (static_cast<size_t>(job) << kGlobalSlotQ),
+    run_circuit<TEAM_MULTI, ROT>(L, L.order[job], L.gscratch + (static_cast<size_t>(job) << kGlobalSlotQ),
                             local * blockDim.x + threadIdx.x, K * blockDim.x, s_red, unused_job,
                             unused_ci, nullptr, &bar, L.blk_sums + static_cast<size_t>(job) * kMultiSums);
   } else {
@@ -1043,7 +1045,7 @@ __global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kSoloThreads
       __syncthreads();
       if (job >= L.n_jobs) break;
       int unused_job = 0, unused_ci = 0;
-      run_circuit<TEAM>(L, L.order[job], st, threadIdx.x, blockDim.x, s_red, unused_job, unused_ci,
+      run_circuit<TEAM, ROT>(L, L.order[job], st, threadIdx.x, blockDim.x, s_red, unused_job, unused_ci,
                         nullptr);
     }
   }
@@ -1078,6 +1080,7 @@ constexpr int kFsvHighQ = kFsvTileQ - kFsvLowQ;
 // instruction; 26 qubits, 10 layers 21.4 ms, now 18.9 ms; with 8 in flight, 19.8).
 constexpr int kFsvBatch = 4;
 
+template <bool ROT>
 __global__ void __launch_bounds__(kFsvThreads, 2)
     fsv_tile_kernel(const __grid_constant__ FusedLaunch L, const __grid_constant__ FsvTile F) {
   extern __shared__ float4 smem_raw[];
@@ -1149,7 +1152,7 @@ __global__ void __launch_bounds__(kFsvThreads, 2)
 #pragma unroll
         for (int q = 0; q < 16; ++q)
           a[q] = st[TQS_IX(sb ^ ((q & 1) ? w0 : 0) ^ ((q & 2) ? w1 : 0) ^ ((q & 4) ? w2 : 0) ^ ((q & 8) ? w3 : 0), NT)];
-        run_ops<false>(a, ops, count, base | ext, scale);
+        run_ops<false, ROT>(a, ops, count, base | ext, scale);
 #pragma unroll
         for (int q = 0; q < 16; ++q)
           st[TQS_IX(sb ^ ((q & 1) ? w0 : 0) ^ ((q & 2) ? w1 : 0) ^ ((q & 4) ? w2 : 0) ^ ((q & 8) ? w3 : 0), NT)] = a[q];
@@ -1185,58 +1188,63 @@ int fused_threads(int team, int warps_per_cta) {
   return team == TEAM_MULTI ? kMultiThreads : kGlobalThreads;
 }
 
+template <bool ROT>
+const void* fused_kernel_of(int team) {
+  switch (team) {
+    case TEAM_WARP: return reinterpret_cast<const void*>(fused_kernel<TEAM_WARP, ROT>);
+    case TEAM_PAIR: return reinterpret_cast<const void*>(fused_kernel<TEAM_PAIR, ROT>);
+    case TEAM_CTA: return reinterpret_cast<const void*>(fused_kernel<TEAM_CTA, ROT>);
+    case TEAM_SOLO: return reinterpret_cast<const void*>(fused_kernel<TEAM_SOLO, ROT>);
+    case TEAM_MULTI: return reinterpret_cast<const void*>(fused_kernel<TEAM_MULTI, ROT>);
+    default: return reinterpret_cast<const void*>(fused_kernel<TEAM_GLOBAL, ROT>);
+  }
+}
+
+// The kernel of a launch, ready for `smem` bytes of dynamic shared memory.
+cudaError_t fused_kernel_for(int team, bool no_rot, size_t smem, const void** fn) {
+  *fn = no_rot ? fused_kernel_of<false>(team) : fused_kernel_of<true>(team);
+  if (smem <= 48 * 1024 - 1024) return cudaSuccess;  // (the kernels' static arrays: below 1 KiB)
+  return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+}
+
 }  // namespace
 
 int fused_max_ctas_per_sm(int team, int warps_per_cta, int slice_q) {
   const size_t smem = fused_smem_bytes(team, warps_per_cta, slice_q);
-  const int threads = fused_threads(team, warps_per_cta);
+  const void* fn = nullptr;
   int blocks = 0;
-  cudaError_t e;
-  if (team == TEAM_WARP) {
-    cudaFuncSetAttribute(fused_kernel<TEAM_WARP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fused_kernel<TEAM_WARP>, threads,
-                                                      smem);
-  } else if (team == TEAM_PAIR) {
-    cudaFuncSetAttribute(fused_kernel<TEAM_PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fused_kernel<TEAM_PAIR>, threads,
-                                                      smem);
-  } else if (team == TEAM_CTA) {
-    cudaFuncSetAttribute(fused_kernel<TEAM_CTA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem));
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fused_kernel<TEAM_CTA>, threads,
-                                                      smem);
-  } else if (team == TEAM_SOLO) {
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fused_kernel<TEAM_SOLO>, threads, smem);
-  } else {
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fused_kernel<TEAM_GLOBAL>, threads,
-                                                      smem);
-  }
-  if (e != cudaSuccess) return 0;
+  if (fused_kernel_for(team, false, smem, &fn) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, fused_threads(team, warps_per_cta), smem) !=
+          cudaSuccess)
+    return 0;
   return blocks;
 }
 
-cudaError_t launch_fsv_tile(const FusedLaunch& L, const FsvTile& F, cudaStream_t s) {
+template <bool ROT>
+static cudaError_t launch_fsv(const FusedLaunch& L, const FsvTile& F, cudaStream_t s) {
   static int per_sm = 0, sms = 0;
   const int smem_max = static_cast<int>((size_t(1) << kFsvTileQ) * sizeof(float2));
   if (per_sm == 0) {
-    cudaError_t e = cudaFuncSetAttribute(fsv_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(fsv_tile_kernel<ROT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          smem_max);
     if (e != cudaSuccess) return e;
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fsv_tile_kernel, kFsvThreads, smem_max);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fsv_tile_kernel<ROT>, kFsvThreads, smem_max);
     if (per_sm < 1) per_sm = 1;
   }
   const uint64_t ntiles = 1ull << (F.n - F.T);
   const uint64_t cap = static_cast<uint64_t>(per_sm) * static_cast<uint64_t>(sms > 0 ? sms : 152);
   const int grid = static_cast<int>(ntiles < cap ? ntiles : cap);
   const size_t smem = (size_t(1) << F.T) * sizeof(float2);
-  fsv_tile_kernel<<<grid, kFsvThreads, smem, s>>>(L, F);
+  fsv_tile_kernel<ROT><<<grid, kFsvThreads, smem, s>>>(L, F);
   count_launches(1);
   return cudaGetLastError();
+}
+
+cudaError_t launch_fsv_tile(const FusedLaunch& L, const FsvTile& F, cudaStream_t s) {
+  return L.no_rot ? launch_fsv<false>(L, F, s) : launch_fsv<true>(L, F, s);
 }
 
 TQS_DEFINE_VIOLATIONS(violations_fused)
@@ -1245,34 +1253,15 @@ cudaError_t launch_fused(const FusedLaunch& L, cudaStream_t s) {
   if (L.n_jobs <= 0) return cudaSuccess;
   const size_t smem = fused_smem_bytes(L.team, L.warps_per_cta, L.slice_q);
   const int threads = fused_threads(L.team, L.warps_per_cta);
-  cudaError_t e = cudaSuccess;
-  if (L.team == TEAM_WARP) {
-    e = cudaFuncSetAttribute(fused_kernel<TEAM_WARP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    fused_kernel<TEAM_WARP><<<L.grid, threads, smem, s>>>(L);
-  } else if (L.team == TEAM_PAIR) {
-    e = cudaFuncSetAttribute(fused_kernel<TEAM_PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    fused_kernel<TEAM_PAIR><<<L.grid, threads, smem, s>>>(L);
-  } else if (L.team == TEAM_CTA) {
-    e = cudaFuncSetAttribute(fused_kernel<TEAM_CTA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    fused_kernel<TEAM_CTA><<<L.grid, threads, smem, s>>>(L);
-  } else if (L.team == TEAM_SOLO) {
-    fused_kernel<TEAM_SOLO><<<L.grid, threads, smem, s>>>(L);
-  } else if (L.team == TEAM_MULTI) {
-    // cooperative: the CTAs wait on one another at the grid barriers
-    FusedLaunch arg = L;
-    void* args[] = {&arg};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fused_kernel<TEAM_MULTI>),
-                                    dim3(L.grid), dim3(threads), args, 0, s);
-    if (e != cudaSuccess) return e;
-  } else {
-    fused_kernel<TEAM_GLOBAL><<<L.grid, threads, 0, s>>>(L);
-  }
+  const void* fn = nullptr;
+  cudaError_t e = fused_kernel_for(L.team, L.no_rot != 0, smem, &fn);
+  if (e != cudaSuccess) return e;
+  FusedLaunch arg = L;
+  void* args[] = {&arg};
+  // TEAM_MULTI is cooperative: the CTAs wait on one another at the grid barriers
+  e = L.team == TEAM_MULTI ? cudaLaunchCooperativeKernel(fn, dim3(L.grid), dim3(threads), args, smem, s)
+                           : cudaLaunchKernel(fn, dim3(L.grid), dim3(threads), args, smem, s);
+  if (e != cudaSuccess) return e;
   count_launches(1);
   return cudaGetLastError();
 }

@@ -233,6 +233,7 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
                                      "tqs_simulate: upload program");
   if (st != TQS_OK) return st;
   L.n_jobs = 1;
+  L.no_rot = !P.rotations;
   L.out = reinterpret_cast<float2*>(d_out);
   L.probs = d_probs;
   L.exact_probs = g_exact_probs.load();
