@@ -540,7 +540,7 @@ tqs_status tqs_check_violations(uint32_t* count, int reset);
  * in HBM per gate.  Read by tqs_simulate_fsv and tqs_fsv_passes (a circuit's
  * cached passes are rebuilt when it changed).
  * TQS_OPT_MULTI_CTAS, key = 0, value = CTAs at most for one circuit of 15 or
- * 16 qubits in tqs_simulate, and for each such request of a server batch that
+ * 16 qubits (or 14, with general gates) in tqs_simulate, and for each request of 15 or 16 qubits of a server batch that
  * holds few of them (together at most the SMs divided by the server's batches
  * in flight) (0 or 1: one CTA; default 8; at most 64), counted in CTAs of 512
  * threads: each is launched as four of 128.  The CTAs (a cooperative launch)

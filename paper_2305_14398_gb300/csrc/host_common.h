@@ -888,7 +888,8 @@ inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint, boo
     // outputs than from a second set of threads: 1024 random circuits of 12
     // qubits 408 -> 194 us, of 13 qubits 546 -> 312 us, QFT and the like 267 ->
     // 166 us (4096 of 12) and 176 -> 118 us (2048 of 13).
-    if (!instr && (lp.slice_q <= 12 || (lp.slice_q == 13 && jobs > device_sms())))
+    // (One circuit alone writes its outputs faster with all.)
+    if (!instr && jobs > 1 && (lp.slice_q <= 12 || (lp.slice_q == 13 && jobs > device_sms())))
       lp.warps = std::min(lp.warps, 8);
     const int per_sm = std::max(1, fused_max_ctas_per_sm(TEAM_CTA, lp.warps, lp.slice_q));
     lp.grid = std::max(1, std::min(jobs, per_sm * device_sms()));
@@ -899,8 +900,8 @@ inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint, boo
   return lp;
 }
 
-// CTAs for a single global-class circuit: one per 512 groups of a pass (a
-// thread per group), at most TQS_OPT_MULTI_CTAS; 1 when the program holds
+// CTAs of 512 threads for one circuit of 14 qubits or more: one per 512 groups
+// of a pass (a thread per group), at most TQS_OPT_MULTI_CTAS; 1 when the program holds
 // instructions or custom unitaries, or the device has no cooperative launch.
 inline std::atomic<int> g_multi_ctas{8};
 // TQS_OPT_EXACT_PROBS: the fused kernels' |psi_i|^2 in FP32 arithmetic (0,
@@ -909,7 +910,7 @@ inline std::atomic<int> g_exact_probs{0};
 constexpr int kMaxMultiJobs = 60;  // barrier counters that fit the server's counter block
 inline int multi_ctas_for(const Program& P) {
   const int limit = g_multi_ctas.load();
-  if (limit < 2 || P.nint <= kCtaMaxQ) return 1;
+  if (limit < 2 || P.nint < kCtaMaxQ) return 1;
   for (const FusedPass& ps : P.passes)
     if (ps.L[0] == kInstrPass || ps.L[0] == kWidePass) return 1;
   static int coop = -1;

@@ -960,12 +960,11 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
   team_sync<TEAM>();
 }
 
-// TEAM_SOLO: sums of 8 pairs of amplitudes, 2^kWarpMaxQ amplitudes at most
-// (and at least one per lane of the 64).
-constexpr int kSoloSums = (1 << kWarpMaxQ) / 16;
+// TEAM_SOLO: sums of 8 pairs of amplitudes, 2^kCtaMaxQ amplitudes at most.
+constexpr int kSoloSums = (1 << kCtaMaxQ) / 16;
 
 template <int TEAM, bool ROT>
-__global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kSoloThreads
+__global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kCtaThreads
                                   : TEAM == TEAM_MULTI ? kMultiThreads
                                   : TEAM == TEAM_CTA   ? kCtaThreads
                                                        : 512)
@@ -1203,7 +1202,7 @@ const void* fused_kernel_of(int team) {
 // The kernel of a launch, ready for `smem` bytes of dynamic shared memory.
 cudaError_t fused_kernel_for(int team, bool no_rot, size_t smem, const void** fn) {
   *fn = no_rot ? fused_kernel_of<false>(team) : fused_kernel_of<true>(team);
-  if (smem <= 48 * 1024 - 1024) return cudaSuccess;  // (the kernels' static arrays: below 1 KiB)
+  if (smem <= 40 * 1024) return cudaSuccess;  // (48 KiB with the kernels' static arrays, 5 KiB at most)
   return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
 }
 

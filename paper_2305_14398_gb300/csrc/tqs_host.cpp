@@ -241,38 +241,48 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
   L.uniforms = d_u;
   L.outcomes = d_outcomes;
   L.grid = 1;
-  if (team == TEAM_WARP && P.n_instr == 0 && P.coef.empty()) {
-    // alone on the GPU: a thread per group instead of a warp for all
+  // A circuit of the global class runs on several CTAs (TEAM_MULTI, bitwise the
+  // same results) when it has no instructions or custom unitaries, and so does
+  // one of 14 qubits with general gates and kCoopPasses passes or more (10
+  // layers 241 -> 131 us, 1 layer 26 -> 34 us; without general gates the
+  // barriers cost more than they bring, QFT 35 -> 37 us, and at 13 qubits the
+  // two are even, 123 and 120 us).
+  constexpr size_t kCoopPasses = 8;
+  const int multi = multi_ctas_for(P);
+  const bool coop = multi >= 2 && (team == TEAM_GLOBAL ||
+                                   (P.nint == kCtaMaxQ && P.rotations && P.passes.size() >= kCoopPasses));
+  if (!coop && team != TEAM_GLOBAL && P.n_instr == 0 && P.coef.empty()) {
+    // alone on the GPU: a thread per group instead of a warp for all, no job counter
     L.team = TEAM_SOLO;
     L.slice_q = P.nint;
-    L.norm_width = 32 * g_team_warps_for_q[P.nint].load();
-    L.warps_per_cta = std::max(L.norm_width, std::min(kSoloThreads, 1 << (P.nint - 4))) / 32;
+    L.norm_width = team == TEAM_CTA ? g_cta_threads.load() : 32 * g_team_warps_for_q[P.nint].load();
+    L.warps_per_cta =
+        std::max(L.norm_width, std::min(team == TEAM_CTA ? L.norm_width : kSoloThreads, 1 << (P.nint - 4))) / 32;
     TQS_CUDA(launch_fused(L, s), "tqs_simulate: launch");
     return TQS_OK;
   }
   TQS_CUDA(c->d_counter.ensure(2 * sizeof(int32_t)), "tqs_simulate: cudaMalloc counter");
   TQS_CUDA(cudaMemsetAsync(c->d_counter.p, 0, 2 * sizeof(int32_t), s), "tqs_simulate: memset");
   L.counter = c->d_counter.as<int32_t>();
-  LaunchPlan lp = plan_for(team, P.nint, 1, 1, P.n_instr > 0);
-  if (team == TEAM_GLOBAL) {
+  if (team == TEAM_GLOBAL || coop) {
     TQS_CUDA(c->d_gscratch.ensure((size_t(1) << kGlobalSlotQ) * sizeof(float2) + kMultiSums * sizeof(float)),
              "tqs_simulate: cudaMalloc scratch");
     L.gscratch = c->d_gscratch.as<float2>();
     L.blk_sums = reinterpret_cast<float*>(L.gscratch + (size_t(1) << kGlobalSlotQ));
   }
+  if (coop) {
+    L.team = TEAM_MULTI;
+    L.grid = L.ctas_per_job = multi * kMultiSplit;
+    L.norm_width = team == TEAM_CTA ? g_cta_threads.load() : kGlobalThreads;
+    L.err = c->d_counter.as<int32_t>() + 1;  // zeroed with the counter above
+    TQS_CUDA(launch_fused(L, s), "tqs_simulate: launch");
+    return TQS_OK;
+  }
+  const LaunchPlan lp = plan_for(team, P.nint, 1, 1, P.n_instr > 0);
   L.team = lp.team;
   L.norm_width = lp.norm_width;
   L.warps_per_cta = lp.warps;
   L.slice_q = lp.slice_q;
-  // A single circuit of the global class runs on several CTAs (TEAM_MULTI,
-  // bitwise the same results) when it has no instructions or custom unitaries.
-  const int multi = multi_ctas_for(P);
-  if (team == TEAM_GLOBAL && multi >= 2) {
-    L.team = TEAM_MULTI;
-    L.grid = L.ctas_per_job = multi * kMultiSplit;
-    L.norm_width = kGlobalThreads;
-    L.err = c->d_counter.as<int32_t>() + 1;  // zeroed with the counter above
-  }
   TQS_CUDA(launch_fused(L, s), "tqs_simulate: launch");
   return TQS_OK;
 }

@@ -135,7 +135,8 @@ static_assert(sizeof(FusedPass) == 16, "FusedPass layout");
 // the norm up, so results are bitwise those of TEAM_GLOBAL.  Circuits without instructions or custom
 // unitaries, few enough that all their CTAs are resident at once.
 // TEAM_SOLO: a circuit of the warp class on a CTA with a thread per group of a
-// pass (up to 128): alone on the GPU, or the jobs of a batch in turn.  It writes the outputs block by block
+// pass (up to 128), alone on the GPU or the jobs of a batch in turn; or one of
+// the CTA class alone on the GPU.  It writes the outputs block by block
 // as the warps of a warp team (or pair) would, so they and the norm are
 // bitwise the same.  Circuits without instructions or custom unitaries.
 enum TeamKind : int32_t {

@@ -86,3 +86,29 @@ def test_batches_on_either_team_equal_singles(count):
     finally:
         for c in handles.values():
             B.tqs_circuit_destroy(c)
+
+
+@pytest.mark.parametrize("threads", [256, 512])
+@pytest.mark.parametrize("name", ["qft", "layered"])
+def test_one_circuit_of_14_qubits_on_either_team(name, threads):
+    """A lone 14-qubit circuit with general gates runs on cooperating CTAs, any
+    other (and every one with the option at 1) on one: the same bits."""
+    n = 14
+    c = B.circuit_from_ops(n, W.qft_on_basis(n, 77) if name == "qft" else W.random_layered(n, 3, (98, n)))
+    got = []
+    old = B.tqs_get_option(B.OPT_CTA_THREADS, 0)
+    B.tqs_set_option(B.OPT_CTA_THREADS, 0, threads)
+    try:
+        for k in (8, 3, 1):
+            B.tqs_set_option(B.OPT_MULTI_CTAS, 0, k)
+            out = torch.empty(1 << n, dtype=torch.complex64, device="cuda")
+            pr = torch.empty(1 << n, dtype=torch.float64, device="cuda")
+            nm = torch.empty(1, dtype=torch.float64, device="cuda")
+            B.tqs_simulate(c, out, probs=pr, norm=nm)
+            got.append((out, pr, nm))
+        for other in got[1:]:
+            assert all(torch.equal(x, y) for x, y in zip(got[0], other))
+    finally:
+        B.tqs_set_option(B.OPT_MULTI_CTAS, 0, 8)
+        B.tqs_set_option(B.OPT_CTA_THREADS, 0, old)
+        B.tqs_circuit_destroy(c)
