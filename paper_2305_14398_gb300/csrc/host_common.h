@@ -639,6 +639,15 @@ struct Image {
     }
     return e;
   }
+  // The same for an image that goes before the copy is known to have run: its
+  // buffers may be page-locked ones of the pool, and the pool's next user would
+  // overwrite what a queued copy still has to read.  The copy is made from
+  // pageable memory, which the call has taken over when it returns.
+  cudaError_t upload_staged(void* dst, cudaStream_t s) const {
+    std::vector<char> h(bytes());
+    copy_to(h.data());
+    return cudaMemcpyAsync(dst, h.data(), h.size(), cudaMemcpyHostToDevice, s);
+  }
 };
 
 // Device copy of one program: its FusedCirc, passes, ops and coefficients, then
@@ -666,7 +675,7 @@ struct ProgramUpload {
       img.circs[0].init = d_init;
       static const int32_t zero_order[1] = {0};
       TQS_CUDA(buf.ensure(order_off + 256), who);
-      TQS_CUDA(img.upload(buf.p, s), who);
+      TQS_CUDA(img.upload_staged(buf.p, s), who);
       TQS_CUDA(cudaMemcpyAsync(buf.as<char>() + order_off, zero_order, sizeof(int32_t), cudaMemcpyHostToDevice, s),
                who);
       if (!done) TQS_CUDA(cudaEventCreateWithFlags(&done, cudaEventDisableTiming), who);

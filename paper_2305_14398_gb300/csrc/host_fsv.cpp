@@ -229,7 +229,7 @@ tqs_status tqs_simulate_fsv(tqs_circuit* c, tqs_c64* d_state, void* stream) {
     c->fsv_img = Image();
     for (const Program& tp : c->fsv.progs) c->fsv_img.add(tp, 0);
     TQS_CUDA(c->d_fsv.ensure(c->fsv_img.bytes()), "tqs_simulate_fsv: cudaMalloc");
-    TQS_CUDA(c->fsv_img.upload(c->d_fsv.p, s), "tqs_simulate_fsv: upload");
+    TQS_CUDA(c->fsv_img.upload_staged(c->d_fsv.p, s), "tqs_simulate_fsv: upload");
     c->fsv_valid = true;
   }
   FusedLaunch L{};
