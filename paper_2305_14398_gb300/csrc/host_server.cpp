@@ -112,9 +112,12 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
   for (int t = 0; t < 3; ++t) plans[t] = plan_for(t, max_nint[t], n_team[t], 0);
   // Few global-class requests: K cooperating CTAs each (TEAM_MULTI),
   // bitwise the same results as one CTA each.  The J K CTAs take at most an
-  // equal share of the SMs per slot in flight, so the cooperative grids of all
-  // slots fit the GPU together (one such CTA per SM) and none waits at a
-  // barrier for SMs held by another waiting grid.
+  // equal share of the SMs per slot in flight, counted in CTAs of kGlobalThreads
+  // (kMultiSplit CTAs of kMultiThreads threads each: at the kernel's 128
+  // registers an SM holds that many), so the cooperative grids of all slots fit the GPU
+  // together and none waits at a barrier for SMs held by another waiting grid.
+  // Their block sums count against the budget; where only they do not fit, one
+  // CTA works each request.
   int multi_k = 0;
   const int J = n_team[TEAM_GLOBAL];
   if (J > 0 && J <= kMaxMultiJobs) {
@@ -122,6 +125,13 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
     for (int32_t i : idx[TEAM_GLOBAL]) k = std::min(k, multi_ctas_for(sl.reqs[i].prog));
     const int share = device_sms() / std::max<int>(1, static_cast<int>(sv->slots.size()));
     if (k >= 2 && J * k <= share) multi_k = k;
+  }
+  const size_t sums_bytes = size_t(J) * kMultiSums * sizeof(float);
+  if (sv->in_use + sums_bytes > sv->budget) multi_k = 0;
+  if (multi_k) {
+    sl.bytes += sums_bytes;
+    sv->in_use += sums_bytes;
+    sv->peak_in_use = std::max(sv->peak_in_use, sv->in_use);
   }
   const size_t order_off = (img.bytes() + 255) & ~size_t(255);
   const size_t counter_off = (order_off + order.size() * sizeof(int32_t) + 255) & ~size_t(255);
@@ -131,7 +141,7 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
   const size_t gscr_bytes =
       J ? size_t(std::max(plans[TEAM_GLOBAL].grid, J)) << kGlobalSlotQ : size_t(0);
   const size_t sums_off = gscr_off + gscr_bytes * sizeof(float2);
-  const size_t total = sums_off + (multi_k ? size_t(J) * kMultiSums * sizeof(float) : 0);
+  const size_t total = sums_off + (multi_k ? sums_bytes : 0);
   // the program goes through pinned memory so the copy is truly asynchronous
   const size_t prog_bytes = order_off + order.size() * sizeof(int32_t);
   {
