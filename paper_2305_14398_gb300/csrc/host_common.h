@@ -1061,8 +1061,9 @@ inline void ensure_steps(tqs_circuit* c) {
 // shares a qubit with it or the block it would make is too large.  A product
 // costs 18 N^3 tensor operations whatever S_k is, and rounds: 40 steps (20
 // layers of U3 and CNOTs) of 12 qubits become 13, 35.4 -> 11.4 ms; 6 steps 2
-// or 3, 4.58 -> 1.36 ms, error against FP64 1.0e-5 -> 6.2e-6; the 12-qubit
-// QFT in TF32x3 42.0 -> 14.2 ms.  With blocks of 6 qubits 11.7 runs instead of
+// or 3 by the CNOT pairs: of 12 drawn circuits, 4.52..4.64 ms before, 7 take
+// 1.05..1.10 ms and 5 take 1.90..2.03 ms, error against FP64 1.0e-5 -> 6.2e-6
+// and 7.2e-6 on two such; the 12-qubit QFT in TF32x3 42.0 -> 14.2 ms.  With blocks of 6 qubits 11.7 runs instead of
 // 13.2 on average, but 4096 coefficients a block to form on the host.
 inline void ensure_chain_steps(tqs_circuit* c) {
   StepTable& T = c->chain_table;

@@ -4,7 +4,7 @@
 
 chain: the 40-step random layered circuit-unitary chain at n = COUNT
        (tensor-core BF16x3); chain_tf32, chain_simt: the same in TF32x3 /
-       FP32 SIMT;
+       FP32 (the columns as a batch);
 probs: tqs_probabilities on a random 2^COUNT state;
 sample: 64 inverse-CDF shots per circuit of COUNT paper-shaped 11-qubit
        circuits (tqs_batch_sample);
