@@ -208,8 +208,11 @@ cd snap_phase(cd z) {
   return std::abs(z - cd(re, im)) <= 1e-14 ? cd(re, im) : z / std::abs(z);
 }
 
-// real_column: the first column's ratio is known to be real (its computed phase
-// is then rounding, large beside a small entry), so alpha is a sign.
+// real_column: the first column's ratio is known to be real, so the small
+// entry's phase is the large one's up to a sign and alpha is that sign.  Its
+// computed phase is rounding, 1e-16 over the entry; without a real column
+// alpha and beta hold that rounding with opposite signs and it cancels, so
+// here beta may not hold it either.
 RotSplit split_rotation(const Mat2& u, bool real_column) {
   RotSplit r;
   double c = std::abs(u.m[0]), s = std::abs(u.m[2]);
@@ -219,21 +222,21 @@ RotSplit split_rotation(const Mat2& u, bool real_column) {
   // u = gamma diag(p0, p1) [[c, -s beta], [s, c beta]]; with s > c the bracket
   // is X [[s, c beta], [c, -s beta]] = X [[s, -c beta'], [c, s beta']], beta' = -beta
   cd p0, p1;  // the phases of the first column, row 0 and row 1
+  const bool minus = real_column && (u.m[2] * std::conj(u.m[0])).real() < 0.0;
   if (!r.flip) {
     p0 = u.m[0] / c;
-    p1 = s > 0.0 ? u.m[2] / s : p0;
+    p1 = s == 0.0 ? p0 : !real_column ? u.m[2] / s : minus ? -p0 : p0;
     r.tau = static_cast<float>(s / c);
     r.beta = u.m[3] / (p1 * std::abs(u.m[3]));
   } else {
     p1 = u.m[2] / s;
-    p0 = c > 0.0 ? u.m[0] / c : p1;
+    p0 = c == 0.0 ? p1 : !real_column ? u.m[0] / c : minus ? -p1 : p1;
     r.tau = static_cast<float>(c / s);
     r.beta = u.m[1] / (p0 * std::abs(u.m[1]));
   }
   r.beta = snap_phase(r.beta);
   r.gamma = snap_phase(p0);
   r.alpha = snap_phase(p1 / p0);
-  if (real_column) r.alpha = r.alpha.real() < 0.0 ? -1.0 : 1.0;
   if (r.alpha == cd(-1.0)) {  // a sign: the rotation the other way
     r.alpha = 1.0;
     r.tau = -r.tau;
