@@ -83,7 +83,7 @@ static tqs_status batch_finish(tqs_batch* b, const std::vector<CircMeta>& progs,
     key[static_cast<size_t>(i)] = t * kBuckets + (kBuckets - 1 - k);  // descending cost
     ++start[static_cast<size_t>(t * (kBuckets + 1) + (kBuckets - 1 - k) + 1)];
     ++b->n_kind[t];
-    b->rotations[t] = b->rotations[t] || progs[i].rotations;
+    b->rot[t] = std::max(b->rot[t], progs[i].rot);
     b->max_nint[t] = std::max(b->max_nint[t], progs[i].nint);
   }
   b->order.resize(static_cast<size_t>(b->count));
@@ -290,7 +290,7 @@ static tqs_status batch_enqueue_at(tqs_batch* b, char* base, size_t order_off, s
     L.slice_q = b->plans[t].slice_q;
     L.grid = b->plans[t].grid;
     L.norm_width = b->plans[t].norm_width;
-    L.no_rot = !b->rotations[t];
+    L.rot = b->rot[t];
     if (fork) {
       TQS_CUDA(cudaStreamWaitEvent(b->side[t], b->ev_fork, 0), "tqs_batch: fork");
       TQS_CUDA(launch_fused(L, b->side[t]), "tqs_batch: launch");
@@ -526,7 +526,7 @@ static tqs_status unitary_block(tqs_circuit* c, int prec, int col0, int ncols, t
     FusedLaunch L{};
     tqs_status st = c->cols_prog.ensure(P, nullptr, L, s, "tqs_circuit_unitary: upload program");
     if (st != TQS_OK) return st;
-    L.no_rot = !P.rotations;
+    L.rot = P.rot;
     TQS_CUDA(c->d_chain.ensure(columns_scratch_bytes(c->n, ncols)), "tqs_circuit_unitary: cudaMalloc");
     TQS_CUDA(launch_columns(L, c->n, P.nint, col0, ncols, U, ldu, c->d_chain.p, device_sms(), s),
              "tqs_circuit_unitary: columns");

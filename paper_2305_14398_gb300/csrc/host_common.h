@@ -284,7 +284,7 @@ struct Program {
   // left here for the program that follows (else it is applied, and 1).
   cd carry = 1.0;
   bool defer = false;
-  bool rotations = false;  // holds rotations (general gates) or their phases
+  int rot = 0;  // FusedLaunch::rot
   double cost = 0.0;
   // Empty the program for reuse (keeps the vectors' capacity).
   void reset() {
@@ -299,7 +299,7 @@ struct Program {
     n_instr = 0;
     carry = 1.0;
     defer = false;
-    rotations = false;
+    rot = 0;
     cost = 0.0;
   }
 };
@@ -351,7 +351,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
 // Fusion of a circuit's single-qubit factors and the move of its phases past
 // one another, in place of gs (new gates live in `store`); see host_compile.cpp.
 bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store, cd& global,
-                   uint32_t* flips);
+                   uint32_t* flips, bool from_basis);
 
 inline int team_for(int nint) {
   if (nint <= kWarpMaxQ) return TEAM_WARP;
@@ -446,7 +446,7 @@ struct ImageSeg {
 // segment `seg` (passes still numbered program-locally).
 struct CircMeta {
   int n = 0, nint = 4, n_instr = 0, gen_index = 0;
-  bool rotations = false;
+  int rot = 0;
   float out_scale = 1.0f;
   double cost = 0.0;
   uint16_t col[16] = {};
@@ -462,7 +462,7 @@ inline CircMeta append_program(const Program& P, ImageSeg& sg, int seg) {
   m.n = P.n;
   m.nint = P.nint;
   m.n_instr = P.n_instr;
-  m.rotations = P.rotations;
+  m.rot = P.rot;
   m.col_off = P.col_off;
   m.gen_index = P.gen_index;
   m.out_scale = P.out_scale;
@@ -1227,7 +1227,7 @@ struct tqs_batch {
   static constexpr int kSoloFew = 1216;
   static bool solo(const CircMeta& m, int warp_class) {
     if (m.nint > kWarpMaxQ || m.n_instr > 0 || m.nc > 0) return false;
-    if (m.rotations) return warp_class <= kSoloFew || m.nint >= kWarpMaxQ - 1;
+    if (m.rot != 0) return warp_class <= kSoloFew || m.nint >= kWarpMaxQ - 1;
     return warp_class <= 2 * kSoloFew;
   }
   static int team_of(int kind) {
@@ -1235,7 +1235,7 @@ struct tqs_batch {
   }
   std::vector<int32_t> order;    // the jobs of each kind in turn
   int n_kind[kKinds] = {};
-  bool rotations[kKinds] = {};   // some circuit of the kind holds rotations
+  int rot[kKinds] = {};          // per kind: FusedLaunch::rot
   int max_nint[kKinds] = {4, 4, 4, 4, 4, 4, 4, 4};
   DevBuf d_img;                  // image + order + counters
   size_t order_off = 0, counter_off = 0;

@@ -191,13 +191,12 @@ double single_cost(const Mat2& u, bool is_h) {
 // An uncontrolled single-qubit unitary as the kernel runs it:
 //   u = gamma diag(1, alpha) X^flip scale R diag(1, beta),  R = [[1, -tau], [tau, 1]],
 // with phases alpha, beta, gamma and |tau| the ratio of the small to the large
-// entry, at most 1.  R costs one multiply-add per real part (the dense product
+// entry, at most 1.  R costs two multiply-adds per real part (the dense product
 // with hi + lo coefficients: eight), and scale = (1 + tau^2)^-1/2 is taken
-// from tau as FP32 holds it, so scale R is a rotation exactly: rounding tau
-// turns it by less than 1.5e-8 and leaves the norm alone.
+// from tau as the record holds it (TauParts), so scale R is a rotation exactly.
 struct RotSplit {
   bool flip;
-  float tau;
+  double tau;
   double scale;
   cd alpha, beta, gamma;
 };
@@ -208,12 +207,77 @@ cd snap_phase(cd z) {
   return std::abs(z - cd(re, im)) <= 1e-14 ? cd(re, im) : z / std::abs(z);
 }
 
+// tau as the record holds it, a + b in FP32.  One FP32 value is off by up to
+// 2^-25, the same way for the same angle, and a circuit that repeats an angle adds
+// that up (2.4e-8 a gate).  b is 0 where one value is as good, else |b| is in
+// [2^-13, 2^-12) and a a multiple of 2^-13 above it, so that a + b is tau to 2^-37.  The
+// parts are not hi + lo: x + lo y with lo below 2^-24 is x again, each time, and
+// the same drift is left.  b y is thousands of units of x's last place, and what
+// the sum rounds off averages out.  On FP32 arithmetic, 18000 turns by 0.9274 of 6
+// qubits: one value 1.9e-5 off, hi + lo 5.2e-5, these parts 1.4e-6, the dense
+// product with hi + lo coefficients 1.1e-6.
+struct TauParts {
+  float a, b;
+};
+TauParts split_tau(double tau) {
+  const double t = std::abs(tau);
+  TauParts p{static_cast<float>(t), 0.f};
+  if (std::abs(t - double(p.a)) > 0x1p-37) {
+    p.a = static_cast<float>((std::floor(t * 0x1p13) - 1.0) * 0x1p-13);
+    p.b = static_cast<float>(t - double(p.a));
+  }
+  return tau < 0.0 ? TauParts{-p.a, -p.b} : p;
+}
+
+// The angles of a circuit met so far, each by its tau in FP32, and how far its uses
+// as one FP32 value turn off in all.  One value rounds each amplitude once
+// where two parts round it twice (a 16-qubit circuit of 10 layers of random
+// angles 4.3e-7 off, with two parts throughout 5.0e-7, dense 4.8e-7), so an angle
+// takes one as long as its uses together are off by no more than FP32 rounds
+// a value, 2^-24.
+class SeenAngles {
+ public:
+  void clear() {
+    if (++epoch_ == 0) {
+      for (Slot& s : slots_) s = Slot();
+      epoch_ = 1;
+    }
+  }
+  // Whether one FP32 value will do for this use.
+  bool one_will_do(double tau) {
+    const float t = static_cast<float>(std::abs(tau));
+    const float off = static_cast<float>(std::abs(std::abs(tau) - double(t)) / (1.0 + tau * tau));
+    uint32_t key;
+    std::memcpy(&key, &t, 4);
+    uint32_t h = (key * 0x9E3779B1u) >> 20;
+    for (int i = 0; i < 8; ++i, h = (h + 1) & (kSlots - 1)) {
+      Slot& s = slots_[h];
+      if (s.epoch != epoch_) s = {epoch_, key, 0.f};
+      if (s.key != key) continue;
+      if (s.off + off > 0x1p-24f) return false;
+      s.off += off;
+      return true;
+    }
+    return false;  // no room left to know
+  }
+
+ private:
+  static constexpr uint32_t kSlots = 4096;  // 2^(32 - 20)
+  struct Slot {
+    uint32_t epoch = 0, key = 0;
+    float off = 0.f;
+  };
+  Slot slots_[kSlots];
+  uint32_t epoch_ = 0;
+};
+
 // real_column: the first column's ratio is known to be real, so the small
 // entry's phase is the large one's up to a sign and alpha is that sign.  Its
 // computed phase is rounding, 1e-16 over the entry; without a real column
 // alpha and beta hold that rounding with opposite signs and it cancels, so
 // here beta may not hold it either.
-RotSplit split_rotation(const Mat2& u, bool real_column) {
+// seen: the circuit's angles, if one FP32 value may do for tau.
+RotSplit split_rotation(const Mat2& u, bool real_column, SeenAngles* seen = nullptr) {
   RotSplit r;
   double c = std::abs(u.m[0]), s = std::abs(u.m[2]);
   if (s <= 1e-14) s = 0.0;  // rounding of a zero: its phase means nothing
@@ -226,12 +290,12 @@ RotSplit split_rotation(const Mat2& u, bool real_column) {
   if (!r.flip) {
     p0 = u.m[0] / c;
     p1 = s == 0.0 ? p0 : !real_column ? u.m[2] / s : minus ? -p0 : p0;
-    r.tau = static_cast<float>(s / c);
+    r.tau = s / c;
     r.beta = u.m[3] / (p1 * std::abs(u.m[3]));
   } else {
     p1 = u.m[2] / s;
     p0 = c == 0.0 ? p1 : !real_column ? u.m[0] / c : minus ? -p1 : p1;
-    r.tau = static_cast<float>(c / s);
+    r.tau = c / s;
     r.beta = u.m[1] / (p0 * std::abs(u.m[1]));
   }
   r.beta = snap_phase(r.beta);
@@ -243,13 +307,19 @@ RotSplit split_rotation(const Mat2& u, bool real_column) {
     r.beta = -r.beta;
     if (r.flip) r.gamma = -r.gamma;
   }
-  r.scale = 1.0 / std::sqrt(1.0 + double(r.tau) * double(r.tau));
+  if (seen != nullptr && seen->one_will_do(r.tau)) {
+    r.tau = static_cast<float>(r.tau);
+  } else {
+    const TauParts p = split_tau(r.tau);
+    r.tau = double(p.a) + double(p.b);
+  }
+  r.scale = 1.0 / std::sqrt(1.0 + r.tau * r.tau);
   return r;
 }
 
 // scale R diag(1, beta): what is left of u with gamma, alpha and X taken out.
 Mat2 rotation_part(const RotSplit& r) {
-  const double c = r.scale, s = r.scale * double(r.tau);
+  const double c = r.scale, s = r.scale * r.tau;
   return {{c, -s * r.beta, s, c * r.beta}};
 }
 
@@ -285,6 +355,14 @@ bool needs_rotation(const Gate& g) {
   if (cls == G_ANTI) return !(exact_phase(g.u.m[1]) && exact_phase(g.u.m[2]));
   Mat2 d1, d2;
   return !hadamard_split(g.u, d2, d1);
+}
+
+// The coefficients of a dense op: FP32 hi + lo.
+void set_dense(FusedOp& op, const Mat2& u) {
+  for (int i = 0; i < 4; ++i) {
+    op.m[i] = to_f2(u.m[i]);
+    op.lo[i] = to_f2(u.m[i] - cd(op.m[i].x, op.m[i].y));
+  }
 }
 
 // Local target position of a non-diagonal op.
@@ -697,8 +775,13 @@ void group_hadamards(std::vector<FusedOp>& ops, size_t begin) {
 // receives the qubits whose X is left at the end (else it becomes a gate).
 // Circuits without such a factor (the paper's programs) are left as they are.
 // True when rotations were taken out.
+// from_basis: gs is all that acts on a basis state.  Where a caller passes a
+// state, it may be one that the same circuit returned, a thousand times over, and
+// a coefficient's error adds up as a repeated gate's would: no angle counts as
+// seldom used (SeenAngles), and the phases of a qubit's last rotation are
+// applied behind it as FP32 hi + lo, not at the end in FP32.
 bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store, cd& global,
-                   uint32_t* flips) {
+                   uint32_t* flips, bool from_basis) {
   static thread_local std::vector<const Gate*> fl_tls;
   std::vector<const Gate*>& fl = fl_tls;
   fl.clear();
@@ -746,12 +829,16 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
   fl.swap(gs);
   gs.clear();
   // after[i]: what lies between the single-qubit gate i and the next
-  // non-diagonal one on its qubit
+  // non-diagonal one on its qubit; final[i]: there is no next one
   enum : uint8_t { kAbsorbed = 0, kZOnly = 1, kXOnly = 2, kOther = 3, kEnd = 4 };
   static thread_local std::vector<uint8_t> after_tls;
   std::vector<uint8_t>& after = after_tls;
   after.assign(fl.size(), kEnd);
+  static thread_local std::vector<uint8_t> final_tls;
+  std::vector<uint8_t>& final = final_tls;
+  final.assign(fl.size(), 0);
   {
+    uint64_t met = 0;  // qubits with a non-diagonal factor further on
     uint8_t st[TQS_MAX_FSV_QUBITS];
     for (uint8_t& v : st) v = kEnd;
     auto meet = [&](int q, uint8_t b) { st[q] = (st[q] == kAbsorbed || st[q] == kEnd || st[q] == b) ? b : kOther; };
@@ -759,6 +846,7 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
       const Gate& g = *fl[i];
       if (g.kind == TQS_SWAP) {
         std::swap(st[g.q[0]], st[g.q[1]]);
+        if (((met >> g.q[0]) ^ (met >> g.q[1])) & 1) met ^= (uint64_t(1) << g.q[0]) | (uint64_t(1) << g.q[1]);
       } else if (is_controlled(g.kind)) {
         meet(g.q[0], kZOnly);
         const GClass cls = classify_mat(g.u);
@@ -767,7 +855,9 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
         for (int k = 0; k < g.nq; ++k) meet(g.q[k], kOther);
       } else {
         after[i] = st[g.q[0]];
+        final[i] = !((met >> g.q[0]) & 1);
         const GClass cls = classify_mat(g.u);
+        if (cls == G_DENSE) met |= uint64_t(1) << g.q[0];
         if (cls == G_DENSE) st[g.q[0]] = kAbsorbed;
         else if (g.kind != TQS_X) meet(g.q[0], kZOnly);
       }
@@ -777,8 +867,11 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
     cd phi = 1.0;
     bool x = false;     // kind X
     bool flip = false;  // kind Z
+    bool rot = false;   // phi comes from a rotation
   };
   Pend pend[TQS_MAX_FSV_QUBITS];
+  static thread_local SeenAngles seen;
+  seen.clear();
   const Mat2 mat_x = {{0.0, 1.0, 1.0, 0.0}};
   auto put = [&](int kind, int q, const Mat2& u) {
     store.emplace_back();
@@ -797,8 +890,16 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
     const cd a = 0.5 * (1.0 + p.phi), b = 0.5 * (1.0 - p.phi);
     return {{a, b, b, a}};
   };
-  // the rotation of u into the circuit, its left factor pending
-  auto rotate = [&](int q, Mat2 u, bool left_x) {
+  // a pending Z's phase becomes a gate: diag(1, phi) X = X phi diag(1, conj phi)
+  auto stop_phase = [&](int q) {
+    Pend& p = pend[q];
+    if (p.flip) global *= p.phi;
+    put_phase(kPhaseKind, q, p.flip ? std::conj(p.phi) : p.phi);
+    p.phi = 1.0;
+  };
+  // the rotation of u into the circuit, its left factor pending; its phase too
+  // if none is to be left at the end (`last`)
+  auto rotate = [&](int q, Mat2 u, bool left_x, bool last) {
     Pend& p = pend[q];
     p = Pend();
     if (left_x) {
@@ -808,7 +909,7 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
       p.x = true;
       u = mat_mul(pend_mat({std::conj(p.phi), true, false}), u);
     }
-    const RotSplit r = split_rotation(u, left_x);
+    const RotSplit r = split_rotation(u, left_x, from_basis ? &seen : nullptr);
     global *= r.gamma;
     if (left_x) {
       if (r.flip) p.phi = -p.phi;  // X = H diag(1, -1) H
@@ -816,7 +917,9 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
       p.phi = r.alpha;
       p.flip = r.flip;
     }
+    p.rot = true;
     put(TQS_U3, q, rotation_part(r));
+    if (last) stop_phase(q);
   };
   // make the pending factor of q one that passes what the flags name: gates
   // that Z (with its X) passes, those that X passes
@@ -824,14 +927,11 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
     Pend& p = pend[q];
     if (p.x) {
       if (p.phi == cd(1.0)) p = Pend();
-      else if (!x) rotate(q, pend_mat(p), false);
+      else if (!x) rotate(q, pend_mat(p), false, false);
     }
     if (p.x || z) return;
     if (x) {
-      // only the phase stops: diag(1, phi) X = X phi diag(1, conj phi)
-      if (p.flip) global *= p.phi;
-      put_phase(kPhaseKind, q, p.flip ? std::conj(p.phi) : p.phi);
-      p.phi = 1.0;
+      stop_phase(q);  // only the phase stops
     } else {
       if (p.flip) put(TQS_X, q, mat_x);
       put_phase(kPhaseKind, q, p.phi);
@@ -920,7 +1020,8 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
       p.x = true;
       gs.push_back(g);
     } else {
-      rotate(q, mat_mul(g->u, pend_mat(p)), after[i] == kXOnly);
+      const bool last = !from_basis && final[i];
+      rotate(q, mat_mul(g->u, pend_mat(p)), after[i] == kXOnly && !last, last);
     }
   }
   if (flips) *flips = 0;
@@ -934,7 +1035,7 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
     } else if (p.flip) {
       put(TQS_X, q, mat_x);
     }
-    put_phase(TQS_R, q, p.phi);
+    put_phase(p.rot && !from_basis ? kPhaseKind : TQS_R, q, p.phi);
   }
   return true;
 }
@@ -1006,11 +1107,12 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     gs.swap(xf);
   }
   static thread_local std::deque<Gate> fused_tls;
+  const bool from_basis = absorb && fold_x;
   bool split = prepared;  // the program runs rotations (split_rotation)
   uint32_t flips = 0;     // qubits with an X left after the program's gates
   if (!prepared) {
     fused_tls.clear();
-    split = prepare_gates(n, gs, fused_tls, P.carry, absorb ? &flips : nullptr);
+    split = prepare_gates(n, gs, fused_tls, P.carry, absorb ? &flips : nullptr, from_basis);
   }
 
   std::vector<uint32_t>& qmask = qmask_tls;
@@ -1082,7 +1184,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     // the phase diag(1, alpha) that a rotation leaves on its own target
     auto emit_phase = [&](cd alpha, int tl) {
       FusedOp op{};
-      P.rotations = true;
+      P.rot = std::max(P.rot, 1);
       op.c = 1;  // hi + lo, multiplied in at once
       op.code = static_cast<uint8_t>(OPC_DLN + tl);
       op.fbit = op.tbit = 0xFF;
@@ -1124,17 +1226,20 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
           pass_cost += 0.5;
         } else if (r.c < 0) {  // dense, or anti-diagonal other than X: a rotation
           const RotSplit rs = split_rotation(u, false);
+          const TauParts tp = split_tau(rs.tau);
+          const cd u01 = -rs.tau * rs.beta;
           carry *= rs.gamma * rs.scale;
-          P.rotations = true;
+          P.rot = std::max(P.rot, tp.b != 0.f ? 2 : 1);
           op.code = static_cast<uint8_t>(OPC_DENSE + tl);
-          op.hc = make_float2(rs.tau, 0.f);
-          const float2 b = to_f2(rs.beta), bl = to_f2(rs.beta - cd(b.x, b.y));
-          op.d0one = rs.beta == cd(1.0) ? 1 : bl.x == 0.f && bl.y == 0.f ? 2 : 0;
+          op.hc = make_float2(tp.a, tp.b);
           op.m[0] = make_float2(1.f, 0.f);
-          op.m[1] = make_float2(-rs.tau * b.x, -rs.tau * b.y);
-          op.m[2] = make_float2(rs.tau, 0.f);
-          op.m[3] = b;
-          op.lo[3] = bl;
+          op.m[1] = to_f2(u01);
+          op.lo[1] = to_f2(u01 - cd(op.m[1].x, op.m[1].y));
+          op.m[2] = to_f2(rs.tau);
+          op.lo[2] = to_f2(rs.tau - double(op.m[2].x));
+          op.m[3] = to_f2(rs.beta);
+          op.lo[3] = to_f2(rs.beta - cd(op.m[3].x, op.m[3].y));
+          op.d0one = rs.beta == cd(1.0) ? 1 : op.lo[3].x == 0.f && op.lo[3].y == 0.f ? 2 : 0;
           pass_cost += 1.0;
           P.ops.push_back(op);
           if (rs.flip) emit_raw({gate_matrix(TQS_X, nullptr), G_ANTI, false, true, r.t, -1, false}, emit_raw);
@@ -1142,11 +1247,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
           return;
         } else {  // controlled: hi + lo coefficients
           op.code = static_cast<uint8_t>(OPC_CDENSE + tl);
-          for (int i = 0; i < 4; ++i) {
-            op.m[i] = to_f2(u.m[i]);
-            const cd hi(op.m[i].x, op.m[i].y);
-            op.lo[i] = to_f2(u.m[i] - hi);
-          }
+          set_dense(op, u);
           pass_cost += 3.0;
         }
       } else {
@@ -1319,25 +1420,49 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
   }
   if (P.passes.empty()) emit_pass(0u, 0, true);
   // What is left of the rotations' phases and scales multiplies the start (or,
-  // in a full-state-vector pass that is not the last, passes on to the next).
+  // in a full-state-vector pass that is not the last, passes on to the next).  A
+  // basis state's one amplitude takes it in FP32, which it is rounded to anyway.
+  // A caller's state may have been through the same circuit many times, each off
+  // the same way (3000 steps: 2e-4), and takes it as FP32 hi + lo: in the first
+  // rotation, as a dense product, or in one of its own.
   if (carry != cd(1.0)) {
     if (h_carry) carry *= std::sqrt(0.5);
     h_carry = 0;
     if (!P.defer) {
       FusedOp op{};
-      op.code = OPC_DLIST;
-      op.t = 4;
-      op.c = 1;
       op.fbit = op.tbit = 0xFF;
       op.act = 0xFFFF;
-      std::memset(&op.hc, 0xFF, sizeof(op.hc));  // every factor always on
-      op.m[0] = to_mod_f2(carry);
-      for (int k = 1; k < 4; ++k) op.m[k] = make_float2(1.f, 0.f);
-      for (float2& v : op.lo) v = make_float2(1.f, 0.f);
-      P.ops.insert(P.ops.begin() + P.passes[0].op_begin, op);
-      ++P.passes[0].op_count;
-      for (size_t i = 1; i < P.passes.size(); ++i)
-        if (P.passes[i].L[0] != kInstrPass && P.passes[i].L[0] != kWidePass) ++P.passes[i].op_begin;
+      FusedOp* first = nullptr;
+      if (from_basis) {
+        op.code = OPC_DLIST;
+        op.t = 4;
+        op.c = 1;
+        std::memset(&op.hc, 0xFF, sizeof(op.hc));  // every factor always on
+        op.m[0] = to_mod_f2(carry);
+        for (int k = 1; k < 4; ++k) op.m[k] = make_float2(1.f, 0.f);
+        for (float2& v : op.lo) v = make_float2(1.f, 0.f);
+      } else {
+        for (FusedOp& o : P.ops)
+          if (o.code >= OPC_DENSE && o.code < OPC_CDENSE) {
+            first = &o;
+            break;
+          }
+        op.code = static_cast<uint8_t>(OPC_CDENSE + (first ? first->code - OPC_DENSE : 0));
+        cd tau = 0.0, beta = 1.0;
+        if (first) {
+          tau = double(first->hc.x) + double(first->hc.y);
+          beta = cd(first->m[3].x, first->m[3].y) + cd(first->lo[3].x, first->lo[3].y);
+        }
+        set_dense(op, {{carry, -carry * tau * beta, carry * tau, carry * beta}});
+      }
+      if (first) {
+        *first = op;
+      } else {
+        P.ops.insert(P.ops.begin() + P.passes[0].op_begin, op);
+        ++P.passes[0].op_count;
+        for (size_t i = 1; i < P.passes.size(); ++i)
+          if (P.passes[i].L[0] != kInstrPass && P.passes[i].L[0] != kWidePass) ++P.passes[i].op_begin;
+      }
       carry = 1.0;
     }
   }

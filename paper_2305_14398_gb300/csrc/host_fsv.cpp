@@ -130,7 +130,7 @@ static tqs_status compile_fsv(int n, const std::vector<Gate>& circuit, int max_g
   for (const Gate& g : circuit) gates.push_back(&g);
   std::deque<Gate> store;
   cd carry = 1.0;
-  const bool split = max_gates == 0 && prepare_gates(n, gates, store, carry, nullptr);
+  const bool split = max_gates == 0 && prepare_gates(n, gates, store, carry, nullptr, false);
   if (max_gates == 0 && !split) {
     gates.clear();
     for (const Gate& g : circuit) gates.push_back(&g);
@@ -245,7 +245,7 @@ tqs_status tqs_simulate_fsv(tqs_circuit* c, tqs_c64* d_state, void* stream) {
     F.nfar = info.nfar;
     std::memcpy(F.far, info.far, sizeof(F.far));
     L.circs = circs + k;
-    L.no_rot = !c->fsv.progs[k].rotations;
+    L.rot = c->fsv.progs[k].rot;
     TQS_CUDA(launch_fsv_tile(L, F, s), "tqs_simulate_fsv: launch");
   }
   return TQS_OK;

@@ -109,6 +109,8 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
   }
   const size_t amps = static_cast<size_t>(sl.offsets.back());
   LaunchPlan plans[3];
+  int rot[3] = {0, 0, 0};  // FusedLaunch::rot
+  for (const SrvReq& r : sl.reqs) rot[team_for(r.prog.nint)] = std::max(rot[team_for(r.prog.nint)], r.prog.rot);
   for (int t = 0; t < 3; ++t) plans[t] = plan_for(t, max_nint[t], n_team[t], 0);
   // Few global-class requests: K cooperating CTAs each (TEAM_MULTI),
   // bitwise the same results as one CTA each.  The J K CTAs take at most an
@@ -195,6 +197,7 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
     L.slice_q = plans[t].slice_q;
     L.grid = plans[t].grid;
     L.norm_width = plans[t].norm_width;
+    L.rot = rot[t];
     if (t == TEAM_GLOBAL && multi_k) {
       L.team = TEAM_MULTI;
       L.ctas_per_job = multi_k * kMultiSplit;

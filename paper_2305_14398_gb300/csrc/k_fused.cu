@@ -111,16 +111,21 @@ __device__ __forceinline__ void dense_t(float2 (&a)[16], const Coef& m, unsigned
 // qubits 960 -> 694 us, a 26-qubit tiled state 23.8 -> 20.5 ms; error against
 // FP64 2.1e-7 -> 1.6e-7, 2.8e-7 -> 2.2e-7, 6.3e-7 -> 5.7e-7 (phases in FP32
 // without lo: 6.9e-7).
-template <int T>
-__device__ __forceinline__ void rot_t(float2 (&a)[16], float tau) {
-  const float2 p = make_float2(tau, tau), m = make_float2(-tau, -tau);
+// TWO: tau = t.x + t.y (TauParts), the smaller part first: another multiply-add
+// (the batches 483 -> 503 and 695 -> 723 us where all programs take it, the tiled
+// state 18.4 -> 18.9 ms).  The parts have one sign, so where t.y
+// is zero both forms give the same bits.
+template <int T, bool TWO>
+__device__ __forceinline__ void rot_t(float2 (&a)[16], float2 t) {
+  const float2 px = make_float2(t.x, t.x), mx = make_float2(-t.x, -t.x);
+  const float2 py = make_float2(t.y, t.y), my = make_float2(-t.y, -t.y);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int j0 = ((k >> T) << (T + 1)) | (k & ((1 << T) - 1));
     const int j1 = j0 | (1 << T);
     const float2 x0 = a[j0], x1 = a[j1];
-    a[j0] = __ffma2_rn(m, x1, x0);
-    a[j1] = __ffma2_rn(p, x0, x1);
+    a[j0] = __ffma2_rn(mx, x1, TWO ? __ffma2_rn(my, x1, x0) : x0);
+    a[j1] = __ffma2_rn(px, x0, TWO ? __ffma2_rn(py, x0, x1) : x1);
   }
 }
 
@@ -280,9 +285,9 @@ __device__ __forceinline__ float2 f2(unsigned x, unsigned y) {
 // one place each 314 us).  SMALL keeps also the hi + lo phase in one place;
 // the other teams' warps run the same ops at about the same time and take one
 // branch less instead (n = 14 batch 702 -> 694 us).
-// ROT: the programs may hold rotations.  Those that hold none (the paper's) take
-// kernels without their code.
-template <bool SMALL, bool ROT>
+// ROT: what rotations the programs may hold: 0 none (the paper's programs; the
+// kernels go without their code), 1 with tau in one part, 2 any.
+template <bool SMALL, int ROT>
 __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restrict__ ops,
                                         uint32_t count, int base, float scale) {
   Pending pd;
@@ -300,14 +305,14 @@ __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restri
     const int fbit = (q0.y >> 8) & 0xff;
     if (fbit != 0xff && !((base >> fbit) & 1)) continue;  // a far control is 0 here
     // a phase that a rotation left on its target: hi + lo, at once
-    const bool phase_op = ROT && code >= OPC_DLN && code < OPC_DFL && ((q0.x >> 16) & 0xff);
+    const bool phase_op = ROT != 0 && code >= OPC_DLN && code < OPC_DFL && ((q0.x >> 16) & 0xff);
     if (code < OPC_DLN || phase_op) {
       // target local position t, or the mask hm of a Hadamard's positions;
       // exchanges act on the pairs in `act`
       int t = code & 3;
       unsigned act = q0.y >> 16;
       const bool had = code < OPC_X || code == OPC_HMASK;
-      const bool rot = ROT && code >= OPC_DENSE && code < OPC_CDENSE;
+      const bool rot = ROT != 0 && code >= OPC_DENSE && code < OPC_CDENSE;
       unsigned hm = 1u << t;
       if (code == OPC_HMASK) hm = (q0.x >> 8) & 15;
       if (code >= OPC_XL && code < OPC_ANTI) {
@@ -342,16 +347,16 @@ __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restri
           default: swap_t<3>(a, act); break;
         }
       } else if (!SMALL && rot) {
-        const float tau = __uint_as_float(q0.z);
+        const float2 tau = f2(q0.z, q0.w);
         switch (kind == 0 ? 4 + t : t) {
-          case 0: rot_t<0>(a, tau); break;
-          case 1: rot_t<1>(a, tau); break;
-          case 2: rot_t<2>(a, tau); break;
-          case 3: rot_t<3>(a, tau); break;
-          case 4: phase_hl_t<0>(a, bh, bl); rot_t<0>(a, tau); break;
-          case 5: phase_hl_t<1>(a, bh, bl); rot_t<1>(a, tau); break;
-          case 6: phase_hl_t<2>(a, bh, bl); rot_t<2>(a, tau); break;
-          default: phase_hl_t<3>(a, bh, bl); rot_t<3>(a, tau); break;
+          case 0: rot_t<0, ROT == 2>(a, tau); break;
+          case 1: rot_t<1, ROT == 2>(a, tau); break;
+          case 2: rot_t<2, ROT == 2>(a, tau); break;
+          case 3: rot_t<3, ROT == 2>(a, tau); break;
+          case 4: phase_hl_t<0>(a, bh, bl); rot_t<0, ROT == 2>(a, tau); break;
+          case 5: phase_hl_t<1>(a, bh, bl); rot_t<1, ROT == 2>(a, tau); break;
+          case 6: phase_hl_t<2>(a, bh, bl); rot_t<2, ROT == 2>(a, tau); break;
+          default: phase_hl_t<3>(a, bh, bl); rot_t<3, ROT == 2>(a, tau); break;
         }
       } else if (rot || phase_op) {
         if (kind == 0) {
@@ -367,12 +372,12 @@ __device__ __forceinline__ void run_ops(float2 (&a)[16], const FusedOp* __restri
           }
         }
         if (SMALL && rot) {
-          const float tau = __uint_as_float(q0.z);
+          const float2 tau = f2(q0.z, q0.w);
           switch (t) {
-            case 0: rot_t<0>(a, tau); break;
-            case 1: rot_t<1>(a, tau); break;
-            case 2: rot_t<2>(a, tau); break;
-            default: rot_t<3>(a, tau); break;
+            case 0: rot_t<0, ROT == 2>(a, tau); break;
+            case 1: rot_t<1, ROT == 2>(a, tau); break;
+            case 2: rot_t<2, ROT == 2>(a, tau); break;
+            default: rot_t<3, ROT == 2>(a, tau); break;
           }
         }
       } else {
@@ -731,7 +736,7 @@ __device__ __noinline__ void wide_pass(const FusedLaunch& L, int nint, int k, ui
   team_sync<TEAM>();
 }
 
-template <int TEAM, bool ROT>
+template <int TEAM, int ROT>
 __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, int size,
                             double* s_red, int& next_job, int& next_ci, int* s_slot,
                             GridBar* bar = nullptr, float* blk_sum = nullptr) {
@@ -963,7 +968,7 @@ __device__ void run_circuit(const FusedLaunch& L, int ci, float2* st, int rank, 
 // TEAM_SOLO: sums of 8 pairs of amplitudes, 2^kCtaMaxQ amplitudes at most.
 constexpr int kSoloSums = (1 << kCtaMaxQ) / 16;
 
-template <int TEAM, bool ROT>
+template <int TEAM, int ROT>
 __global__ void __launch_bounds__(TEAM == TEAM_SOLO    ? kCtaThreads
                                   : TEAM == TEAM_MULTI ? kMultiThreads
                                   : TEAM == TEAM_CTA   ? kCtaThreads
@@ -1079,7 +1084,7 @@ constexpr int kFsvHighQ = kFsvTileQ - kFsvLowQ;
 // instruction; 26 qubits, 10 layers 21.4 ms, now 18.9 ms; with 8 in flight, 19.8).
 constexpr int kFsvBatch = 4;
 
-template <bool ROT>
+template <int ROT>
 __global__ void __launch_bounds__(kFsvThreads, 2)
     fsv_tile_kernel(const __grid_constant__ FusedLaunch L, const __grid_constant__ FsvTile F) {
   extern __shared__ float4 smem_raw[];
@@ -1187,7 +1192,7 @@ int fused_threads(int team, int warps_per_cta) {
   return team == TEAM_MULTI ? kMultiThreads : kGlobalThreads;
 }
 
-template <bool ROT>
+template <int ROT>
 const void* fused_kernel_of(int team) {
   switch (team) {
     case TEAM_WARP: return reinterpret_cast<const void*>(fused_kernel<TEAM_WARP, ROT>);
@@ -1200,8 +1205,8 @@ const void* fused_kernel_of(int team) {
 }
 
 // The kernel of a launch, ready for `smem` bytes of dynamic shared memory.
-cudaError_t fused_kernel_for(int team, bool no_rot, size_t smem, const void** fn) {
-  *fn = no_rot ? fused_kernel_of<false>(team) : fused_kernel_of<true>(team);
+cudaError_t fused_kernel_for(int team, int rot, size_t smem, const void** fn) {
+  *fn = rot == 0 ? fused_kernel_of<0>(team) : rot == 1 ? fused_kernel_of<1>(team) : fused_kernel_of<2>(team);
   if (smem <= 40 * 1024) return cudaSuccess;  // (48 KiB with the kernels' static arrays, 5 KiB at most)
   return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
 }
@@ -1212,14 +1217,14 @@ int fused_max_ctas_per_sm(int team, int warps_per_cta, int slice_q) {
   const size_t smem = fused_smem_bytes(team, warps_per_cta, slice_q);
   const void* fn = nullptr;
   int blocks = 0;
-  if (fused_kernel_for(team, false, smem, &fn) != cudaSuccess ||
+  if (fused_kernel_for(team, 2, smem, &fn) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, fused_threads(team, warps_per_cta), smem) !=
           cudaSuccess)
     return 0;
   return blocks;
 }
 
-template <bool ROT>
+template <int ROT>
 static cudaError_t launch_fsv(const FusedLaunch& L, const FsvTile& F, cudaStream_t s) {
   static int per_sm = 0, sms = 0;
   const int smem_max = static_cast<int>((size_t(1) << kFsvTileQ) * sizeof(float2));
@@ -1243,7 +1248,7 @@ static cudaError_t launch_fsv(const FusedLaunch& L, const FsvTile& F, cudaStream
 }
 
 cudaError_t launch_fsv_tile(const FusedLaunch& L, const FsvTile& F, cudaStream_t s) {
-  return L.no_rot ? launch_fsv<false>(L, F, s) : launch_fsv<true>(L, F, s);
+  return L.rot == 0 ? launch_fsv<0>(L, F, s) : L.rot == 1 ? launch_fsv<1>(L, F, s) : launch_fsv<2>(L, F, s);
 }
 
 TQS_DEFINE_VIOLATIONS(violations_fused)
@@ -1253,7 +1258,7 @@ cudaError_t launch_fused(const FusedLaunch& L, cudaStream_t s) {
   const size_t smem = fused_smem_bytes(L.team, L.warps_per_cta, L.slice_q);
   const int threads = fused_threads(L.team, L.warps_per_cta);
   const void* fn = nullptr;
-  cudaError_t e = fused_kernel_for(L.team, L.no_rot != 0, smem, &fn);
+  cudaError_t e = fused_kernel_for(L.team, L.rot, smem, &fn);
   if (e != cudaSuccess) return e;
   FusedLaunch arg = L;
   void* args[] = {&arg};

@@ -233,7 +233,7 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
                                      "tqs_simulate: upload program");
   if (st != TQS_OK) return st;
   L.n_jobs = 1;
-  L.no_rot = !P.rotations;
+  L.rot = P.rot;
   L.out = reinterpret_cast<float2*>(d_out);
   L.probs = d_probs;
   L.exact_probs = g_exact_probs.load();
@@ -250,7 +250,7 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
   constexpr size_t kCoopPasses = 8;
   const int multi = multi_ctas_for(P);
   const bool coop = multi >= 2 && (team == TEAM_GLOBAL ||
-                                   (P.nint == kCtaMaxQ && P.rotations && P.passes.size() >= kCoopPasses));
+                                   (P.nint == kCtaMaxQ && P.rot != 0 && P.passes.size() >= kCoopPasses));
   if (!coop && team != TEAM_GLOBAL && P.n_instr == 0 && P.coef.empty()) {
     // alone on the GPU: a thread per group instead of a warp for all, no job counter
     L.team = TEAM_SOLO;

@@ -37,11 +37,13 @@ namespace tqs {
 //                    control positions (a run of X / CNOT factors on one target)
 //   OPC_DENSE + t    uncontrolled 2x2 as a rotation after a phase (the rest of
 //                    the gate, its outer phase, X and scale, is carried by the
-//                    compiler): [[1, -tau], [tau, 1]] diag(1, beta); tau in
-//                    hc.x; `d0one` = 1 when beta is exactly 1, 2 when FP32
+//                    compiler): [[1, -tau], [tau, 1]] diag(1, beta); tau =
+//                    hc.x + hc.y; `d0one` = 1 when beta is exactly 1, 2 when FP32
 //                    holds it, else 0; beta as hi + lo in m[3], lo[3]; m holds
 //                    the product
-//   OPC_CDENSE + t   controlled 2x2 (`act` mask for a local control, `fbit` far)
+//   OPC_CDENSE + t   2x2 with FP32 hi + lo coefficients, controlled (`act` mask for
+//                    a local control, `fbit` far) or, once in a program that
+//                    starts from a caller's state, not
 //   OPC_DLN + t      diag(d0, d1), local target, uncontrolled; field c = 1:
 //                    diag(1, d1) with d1 as hi + lo (hc, lo[0])
 //   OPC_DLF + t      diag(d0, d1), local target, far control `fbit`
@@ -100,7 +102,7 @@ struct alignas(16) FusedOp {
   float2 hc;       // diagonal ops, in the header so no further load is needed in the
                    // common case: d1/d0 (DLN, DLF) or d1 (DFL, DFF, DLL)
   float2 m[4];     // DENSE: m00 m01 m10 m11 | ANTI: -, m01, m10, - | DIAG: d0, d1, d1/d0, -
-  float2 lo[4];    // CDENSE: m - m_fp32 rounded to FP32 (the FP64 matrix is m + lo)
+  float2 lo[4];    // DENSE, CDENSE: m - m_fp32 rounded to FP32 (the FP64 matrix is m + lo)
 };
 static_assert(sizeof(FusedOp) == 80, "FusedOp layout");
 
@@ -202,7 +204,8 @@ struct FusedLaunch {
   const double* uniforms;   // instructions: one uniform each (nullable without instructions)
   int32_t* outcomes;        // instructions: one outcome each (nullable)
   int32_t* err;             // TEAM_MULTI: set to 1 when a grid barrier timed out
-  int32_t no_rot;           // 1: no program of the launch holds a rotation (OPC_DENSE) or its phase
+  int32_t rot;              // the most that a program of the launch holds: 0 no rotation (OPC_DENSE) nor
+                            // its phase, 1 rotations with tau in one part, 2 any
   int32_t exact_probs;      // probs: 1 exact squares rounded once in FP64, 0 FP32 |psi|^2
   int32_t ctas_per_job;     // TEAM_MULTI: CTAs per circuit; job j runs on CTAs
                             // [j K, (j + 1) K), its barrier counter is counter[j],
