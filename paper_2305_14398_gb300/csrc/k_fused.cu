@@ -1208,7 +1208,8 @@ const void* fused_kernel_of(int team) {
 cudaError_t fused_kernel_for(int team, int rot, size_t smem, const void** fn) {
   *fn = rot == 0 ? fused_kernel_of<0>(team) : rot == 1 ? fused_kernel_of<1>(team) : fused_kernel_of<2>(team);
   if (smem <= 40 * 1024) return cudaSuccess;  // (48 KiB with the kernels' static arrays, 5 KiB at most)
-  return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  static std::atomic<uint64_t> done[kTeamKinds][3];
+  return allow_all_smem(*fn, done[team][rot]);
 }
 
 }  // namespace

@@ -401,14 +401,15 @@ cudaError_t launch_sample(const SampleLaunch& L, cudaStream_t s) {
     int threads = 32;
     while (threads < kThreads && (threads < nc || threads < L.shots)) threads *= 2;
     const int smem = nc * (kChunkPad + 1) * static_cast<int>(sizeof(double));
-    auto launch = [&](auto kernel) -> cudaError_t {
-      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static std::atomic<uint64_t> done[3];
+    auto launch = [&](auto kernel, std::atomic<uint64_t>& d) -> cudaError_t {
+      const cudaError_t e = allow_all_smem(reinterpret_cast<const void*>(kernel), d);
       if (e == cudaSuccess) kernel<<<L.n_sseg, threads, smem, s>>>(L);
       return e;
     };
-    const cudaError_t e = nc <= threads       ? launch(segment_smem_kernel<1>)
-                          : nc <= 2 * threads ? launch(segment_smem_kernel<2>)
-                                              : launch(segment_smem_kernel<4>);
+    const cudaError_t e = nc <= threads       ? launch(segment_smem_kernel<1>, done[0])
+                          : nc <= 2 * threads ? launch(segment_smem_kernel<2>, done[1])
+                                              : launch(segment_smem_kernel<4>, done[2]);
     if (e != cudaSuccess) return e;
     ++k;
   }

@@ -2,6 +2,7 @@
 // sm_103a kernels.  Not part of the public ABI.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -144,6 +145,7 @@ static_assert(sizeof(FusedPass) == 16, "FusedPass layout");
 enum TeamKind : int32_t {
   TEAM_WARP = 0, TEAM_CTA = 1, TEAM_GLOBAL = 2, TEAM_PAIR = 3, TEAM_MULTI = 4, TEAM_SOLO = 5
 };
+constexpr int kTeamKinds = 6;
 
 // Grid barrier of TEAM_MULTI: spins at most this many SM cycles (about 1 s),
 // then records a time-out in FusedLaunch::err and stops waiting.
@@ -359,6 +361,25 @@ cudaError_t violations_probs(unsigned int* count, bool reset);
 cudaError_t violations_sample(unsigned int* count, bool reset);
 cudaError_t violations_columns(unsigned int* count, bool reset);
 cudaError_t violations_chain_tc(unsigned int* count, bool reset);
+
+// Raises a kernel's limit of dynamic shared memory to all that the current device
+// has beside the kernel's static arrays, once per device (`done`: a bit each).
+// With the limit set to each launch's own size, threads that launched one kernel
+// with different sizes made one another's launches fail.
+inline cudaError_t allow_all_smem(const void* kernel, std::atomic<uint64_t>& done) {
+  int dev = 0, all = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = uint64_t(1) << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  cudaFuncAttributes at;
+  if ((e = cudaFuncGetAttributes(&at, kernel)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           all - static_cast<int>(at.sharedSizeBytes));
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
 
 // Process-wide count of kernel launches enqueued by this library.
 void count_launches(int64_t k);
