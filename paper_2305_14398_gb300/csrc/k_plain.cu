@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kMatThreads)
                        float2* __restrict__ S) {
   __shared__ StepFactor fs[kMaxFactors];
   __shared__ int level[16];
-  __shared__ float2 mid[kMatMid];
+  __shared__ alignas(16) float2 mid[kMatMid];  // read two entries at a time
   const int t = threadIdx.x;
   for (int i = t; i < nf * static_cast<int>(sizeof(StepFactor) / 8); i += blockDim.x)
     reinterpret_cast<float2*>(fs)[TQS_IX(i, int(sizeof(fs) / 8))] =
