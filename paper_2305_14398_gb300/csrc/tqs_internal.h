@@ -261,7 +261,7 @@ size_t chain_tc_scratch_bytes(int n, int prec, int ncols);
 // group: output-tile rows per raster band of the GEMM grid (L2 reuse).
 cudaError_t chain_tc(const StepFactor* d_factors, const StepDesc* steps, int nsteps, int n,
                      int prec, int col0, int ncols, float2* d_U, int64_t ldu, void* scratch,
-                     int* d_err, int group, int kchunk, int pair, cudaStream_t s);
+                     int* d_err, int group, int kchunk, cudaStream_t s);
 // FP32 form: the columns as a batch of the circuit's fused program, whose
 // arrays L names (L.circs its descriptor).
 size_t columns_scratch_bytes(int n, int ncols);
