@@ -918,7 +918,8 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
       p.flip = r.flip;
     }
     p.rot = true;
-    put(TQS_U3, q, rotation_part(r));
+    if (r.tau == 0.0) put_phase(kPhaseKind, q, r.beta);  // nothing to turn
+    else put(TQS_U3, q, rotation_part(r));
     if (last) stop_phase(q);
   };
   // make the pending factor of q one that passes what the flags name: gates

@@ -54,6 +54,29 @@ def test_repeated_angles_do_not_drift(name, theta):
     assert np.max(np.abs(got - fsv_route.simulate(2, ops))) < 2e-7
 
 
+def with_low_parts(prog):
+    """The program with the hi + lo phases that follow rotations (field c of an
+    uncontrolled local diagonal op) as FP64, which the replay reads as hi alone."""
+    ops = prog[1]
+    wide = np.zeros(len(ops), dtype=[(k, (np.complex128, (4,))) if k == "m" else (k,) + (
+        ops.dtype[k].subdtype if ops.dtype[k].subdtype else (ops.dtype[k],)) for k in ops.dtype.names])
+    for k in ops.dtype.names:
+        wide[k] = ops[k]
+    hl = (ops["code"] >= 40) & (ops["code"] < 44) & (ops["c"] == 1)
+    wide["m"][hl, 1] += ops["lo"][hl, 0]
+    wide["m"][hl, 2] = wide["m"][hl, 1]
+    return (prog[0], wide) + tuple(prog[2:])
+
+
+@pytest.mark.parametrize("theta", [0.7, 2.0, math.pi, math.pi - 1e-15])
+def test_repeated_phases_do_not_drift(theta):
+    # phases before controls, targets and half turns: as for the angles
+    ops = [("u3", (q,), (theta, 0.3, 0.9)) for q in range(3)]
+    ops = (ops + [("cx", (0, 1), ()), ("ry", (0,), (0.5,)), ("cx", (1, 2), ()), ("rz", (2,), (0.4,))]) * 700
+    got = hp.replay(3, *with_low_parts(hp.compiled(3, ops)))
+    assert np.max(np.abs(got - fsv_route.simulate(3, ops))) < 2e-7
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("theta", [0.7, 0.9274, 1.0, 2.0])
 def test_gpu_repeated_angles(theta):
