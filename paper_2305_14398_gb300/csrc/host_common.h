@@ -221,6 +221,9 @@ constexpr int kCustomKind = 64;
 // Internal kind of the phase diag(1, phi) that prepare_gates puts before the
 // target of a CNOT: it runs in a pass where its qubit is local, as hi + lo.
 constexpr int kPhaseKind = 65;
+// Internal kind of a rotation that prepare_gates took out of a factor: u =
+// scale [[1, -tau], [tau, 1]] diag(1, beta), p[0] = tau, p[1] + i p[2] = beta.
+constexpr int kRotKind = 66;
 
 // One recorded operation.
 struct Gate {
@@ -231,6 +234,28 @@ struct Gate {
   Mat2 u;     // single-qubit matrix, the controlled U, or a 1-qubit custom matrix
   int step;   // step index (ASAP)
   std::shared_ptr<const CustomMat> cm;  // custom unitaries with k >= 2
+};
+
+// Gates made by the compiler.  The memory of the first 4096 is kept for the next
+// circuit (a deque allocates for every two).
+class GateStore {
+ public:
+  void clear() {
+    n_ = 0;
+    if (chunks_.size() > kKept) chunks_.resize(kKept);
+  }
+  Gate& add() {
+    if (n_ == chunks_.size() * kChunk) chunks_.emplace_back(new Gate[kChunk]);
+    Gate& g = chunks_[n_ / kChunk][n_ % kChunk];
+    ++n_;
+    g.cm.reset();
+    return g;
+  }
+
+ private:
+  static constexpr size_t kChunk = 64, kKept = 64;
+  std::vector<std::unique_ptr<Gate[]>> chunks_;
+  size_t n_ = 0;
 };
 
 inline bool is_wide(const Gate& g) { return g.kind == kCustomKind && g.nq >= 2; }
@@ -306,6 +331,7 @@ struct Program {
 
 // A scheduled factor of the pass being built (compile_program).
 struct CompileRaw {
+  const Gate* g;
   Mat2 u;
   GClass cls;
   bool is_h;    // unfused uncontrolled Hadamard
@@ -350,7 +376,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
 
 // Fusion of a circuit's single-qubit factors and the move of its phases past
 // one another, in place of gs (new gates live in `store`); see host_compile.cpp.
-bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store, cd& global,
+bool prepare_gates(int n, std::vector<const Gate*>& gs, GateStore& store, cd& global,
                    uint32_t* flips, bool from_basis);
 
 inline int team_for(int nint) {

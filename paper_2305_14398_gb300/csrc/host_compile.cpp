@@ -1,8 +1,6 @@
 // The fused-pass compiler (compile_program): a circuit's steps into passes of 4
 // local qubit bits with their ops (declared, with its description, in
 // host_common.h).
-#include <deque>
-
 #include "host_common.h"
 
 namespace tqs {
@@ -202,10 +200,15 @@ struct RotSplit {
 };
 
 // A phase within 1e-14 of 1, -1, i or -i is that value.
-cd snap_phase(cd z) {
-  const double re = std::round(z.real()), im = std::round(z.imag());
-  return std::abs(z - cd(re, im)) <= 1e-14 ? cd(re, im) : z / std::abs(z);
+cd snap_unit(cd z) {
+  if (std::abs(z.real()) <= 1e-14 || std::abs(z.imag()) <= 1e-14) {
+    const cd s(std::round(z.real()), std::round(z.imag()));
+    if (std::norm(z - s) <= 1e-28) return s;
+  }
+  return z;
 }
+cd unit(cd z) { return z * (1.0 / std::sqrt(std::norm(z))); }
+cd snap_phase(cd z) { return snap_unit(unit(z)); }
 
 // tau as the record holds it, a + b in FP32.  One FP32 value is off by up to
 // 2^-25, the same way for the same angle, and a circuit that repeats an angle adds
@@ -279,7 +282,9 @@ class SeenAngles {
 // seen: the circuit's angles, if one FP32 value may do for tau.
 RotSplit split_rotation(const Mat2& u, bool real_column, SeenAngles* seen = nullptr) {
   RotSplit r;
-  double c = std::abs(u.m[0]), s = std::abs(u.m[2]);
+  // (moduli as roots of sums of squares and phases multiplied by conjugates: the
+  // entries are at most 1, and hypot and complex division took most of a circuit's compile)
+  double c = std::sqrt(std::norm(u.m[0])), s = std::sqrt(std::norm(u.m[2]));
   if (s <= 1e-14) s = 0.0;  // rounding of a zero: its phase means nothing
   if (c <= 1e-14) c = 0.0;
   r.flip = s > c;
@@ -288,19 +293,19 @@ RotSplit split_rotation(const Mat2& u, bool real_column, SeenAngles* seen = null
   cd p0, p1;  // the phases of the first column, row 0 and row 1
   const bool minus = real_column && (u.m[2] * std::conj(u.m[0])).real() < 0.0;
   if (!r.flip) {
-    p0 = u.m[0] / c;
-    p1 = s == 0.0 ? p0 : !real_column ? u.m[2] / s : minus ? -p0 : p0;
+    p0 = u.m[0] * (1.0 / c);
+    p1 = s == 0.0 ? p0 : !real_column ? u.m[2] * (1.0 / s) : minus ? -p0 : p0;
     r.tau = s / c;
-    r.beta = u.m[3] / (p1 * std::abs(u.m[3]));
+    r.beta = u.m[3] * std::conj(p1);
   } else {
-    p1 = u.m[2] / s;
-    p0 = c == 0.0 ? p1 : !real_column ? u.m[0] / c : minus ? -p1 : p1;
+    p1 = u.m[2] * (1.0 / s);
+    p0 = c == 0.0 ? p1 : !real_column ? u.m[0] * (1.0 / c) : minus ? -p1 : p1;
     r.tau = c / s;
-    r.beta = u.m[1] / (p0 * std::abs(u.m[1]));
+    r.beta = u.m[1] * std::conj(p0);
   }
   r.beta = snap_phase(r.beta);
-  r.gamma = snap_phase(p0);
-  r.alpha = snap_phase(p1 / p0);
+  r.gamma = snap_unit(p0);
+  r.alpha = snap_unit(p1 * std::conj(p0));
   if (r.alpha == cd(-1.0)) {  // a sign: the rotation the other way
     r.alpha = 1.0;
     r.tau = -r.tau;
@@ -780,7 +785,7 @@ void group_hadamards(std::vector<FusedOp>& ops, size_t begin) {
 // a coefficient's error adds up as a repeated gate's would: no angle counts as
 // seldom used (SeenAngles), and the phases of a qubit's last rotation are
 // applied behind it as FP32 hi + lo, not at the end in FP32.
-bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store, cd& global,
+bool prepare_gates(int n, std::vector<const Gate*>& gs, GateStore& store, cd& global,
                    uint32_t* flips, bool from_basis) {
   static thread_local std::vector<const Gate*> fl_tls;
   std::vector<const Gate*>& fl = fl_tls;
@@ -805,8 +810,8 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
           open[q] = -1;
           continue;
         }
-        store.push_back(*pg);
-        Gate& f = store.back();
+        Gate& f = store.add();
+        f = *pg;
         f.u = uf;
         f.cm.reset();
         const bool is_x = uf.m[0] == cd(0.0) && uf.m[3] == cd(0.0) && uf.m[1] == cd(1.0) && uf.m[2] == cd(1.0);
@@ -873,23 +878,30 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
   static thread_local SeenAngles seen;
   seen.clear();
   const Mat2 mat_x = {{0.0, 1.0, 1.0, 0.0}};
-  auto put = [&](int kind, int q, const Mat2& u) {
-    store.emplace_back();
-    Gate& g = store.back();
+  auto put = [&](int kind, int q, const Mat2& u) -> Gate* {
+    Gate& g = store.add();
     g.kind = kind;
     for (int& v : g.q) v = q;
     g.nq = 1;
+    g.step = 0;
     g.u = u;
     gs.push_back(&g);
+    return &g;
   };
   auto put_phase = [&](int kind, int q, cd phi) {
     if (phi != cd(1.0)) put(kind, q, {{1.0, 0.0, 0.0, phi}});
   };
-  auto pend_mat = [&](const Pend& p) -> Mat2 {
-    if (!p.x) return p.flip ? Mat2{{0.0, 1.0, p.phi, 0.0}} : Mat2{{1.0, 0.0, 0.0, p.phi}};
-    const cd a = 0.5 * (1.0 + p.phi), b = 0.5 * (1.0 - p.phi);
-    return {{a, b, b, a}};
+  // u times a pending factor
+  auto times_pend = [&](const Mat2& u, const Pend& p) -> Mat2 {
+    if (p.x) {
+      const cd a0 = u.m[0] + u.m[1], a1 = (u.m[0] - u.m[1]) * p.phi;
+      const cd b0 = u.m[2] + u.m[3], b1 = (u.m[2] - u.m[3]) * p.phi;
+      return {{0.5 * (a0 + a1), 0.5 * (a0 - a1), 0.5 * (b0 + b1), 0.5 * (b0 - b1)}};
+    }
+    const cd a1 = u.m[1] * p.phi, b1 = u.m[3] * p.phi;
+    return p.flip ? Mat2{{a1, u.m[0], b1, u.m[2]}} : Mat2{{u.m[0], a1, u.m[2], b1}};
   };
+  const Mat2 one = {{1.0, 0.0, 0.0, 1.0}};
   // a pending Z's phase becomes a gate: diag(1, phi) X = X phi diag(1, conj phi)
   auto stop_phase = [&](int q) {
     Pend& p = pend[q];
@@ -905,9 +917,11 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
     if (left_x) {
       // the X factor that makes the first column real up to a phase, its larger part first
       const cd w0 = u.m[0] + u.m[2], w1 = u.m[0] - u.m[2];
-      if (std::abs(w0) > 0.0 && std::abs(w1) > 0.0) p.phi = snap_phase((w1 / std::abs(w1)) / (w0 / std::abs(w0)));
+      const cd v0 = u.m[1] + u.m[3], v1 = u.m[1] - u.m[3];
+      if (std::norm(w0) > 0.0 && std::norm(w1) > 0.0) p.phi = snap_unit(unit(w1) * std::conj(unit(w0)));
       p.x = true;
-      u = mat_mul(pend_mat({std::conj(p.phi), true, false}), u);
+      const cd x1 = std::conj(p.phi) * w1, y1 = std::conj(p.phi) * v1;
+      u = {{0.5 * (w0 + x1), 0.5 * (v0 + y1), 0.5 * (w0 - x1), 0.5 * (v0 - y1)}};
     }
     const RotSplit r = split_rotation(u, left_x, from_basis ? &seen : nullptr);
     global *= r.gamma;
@@ -918,8 +932,14 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
       p.flip = r.flip;
     }
     p.rot = true;
-    if (r.tau == 0.0) put_phase(kPhaseKind, q, r.beta);  // nothing to turn
-    else put(TQS_U3, q, rotation_part(r));
+    if (r.tau == 0.0) {  // nothing to turn
+      put_phase(kPhaseKind, q, r.beta);
+    } else {
+      Gate* g = put(kRotKind, q, rotation_part(r));
+      g->p[0] = r.tau;
+      g->p[1] = r.beta.real();
+      g->p[2] = r.beta.imag();
+    }
     if (last) stop_phase(q);
   };
   // make the pending factor of q one that passes what the flags name: gates
@@ -928,7 +948,7 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
     Pend& p = pend[q];
     if (p.x) {
       if (p.phi == cd(1.0)) p = Pend();
-      else if (!x) rotate(q, pend_mat(p), false, false);
+      else if (!x) rotate(q, times_pend(one, p), false, false);
     }
     if (p.x || z) return;
     if (x) {
@@ -984,10 +1004,11 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
           global *= std::conj(w);
           gs.push_back(g);
         } else {
-          store.push_back(*g);
-          store.back().kind = TQS_CP;
-          store.back().u.m[3] = std::conj(w);
-          gs.push_back(&store.back());
+          Gate& cp = store.add();
+          cp = *g;
+          cp.kind = TQS_CP;
+          cp.u.m[3] = std::conj(w);
+          gs.push_back(&cp);
         }
       }
       continue;
@@ -1022,7 +1043,7 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, std::deque<Gate>& store,
       gs.push_back(g);
     } else {
       const bool last = !from_basis && final[i];
-      rotate(q, mat_mul(g->u, pend_mat(p)), after[i] == kXOnly && !last, last);
+      rotate(q, times_pend(g->u, p), after[i] == kXOnly && !last, last);
     }
   }
   if (flips) *flips = 0;
@@ -1107,7 +1128,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     }
     gs.swap(xf);
   }
-  static thread_local std::deque<Gate> fused_tls;
+  static thread_local GateStore fused_tls;
   const bool from_basis = absorb && fold_x;
   bool split = prepared;  // the program runs rotations (split_rotation)
   uint32_t flips = 0;     // qubits with an X left after the program's gates
@@ -1156,6 +1177,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
         const Mat2 uf = mat_mul(g.u, r.u);
         if (single_cost(uf, false) <= single_cost(r.u, r.is_h) + single_cost(g.u, g.kind == TQS_H)) {
           if (r.is_h) --h_in_pass;
+          r.g = nullptr;
           r.u = uf;
           r.is_h = false;
           r.cls = classify_mat(r.u);
@@ -1165,7 +1187,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     }
     const bool is_h = single && g.kind == TQS_H && h_in_pass < kMaxHPerPass;
     if (is_h) ++h_in_pass;
-    raw.push_back({g.u, cls, is_h, single, t, c, g.kind == kPhaseKind});
+    raw.push_back({&g, g.u, cls, is_h, single, t, c, g.kind == kPhaseKind});
     last_touch[t] = static_cast<int>(raw.size()) - 1;
     if (c >= 0) last_touch[c] = static_cast<int>(raw.size()) - 1;
   };
@@ -1226,7 +1248,13 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
           else op.code = static_cast<uint8_t>(OPC_XL + 4 * tl + cl);
           pass_cost += 0.5;
         } else if (r.c < 0) {  // dense, or anti-diagonal other than X: a rotation
-          const RotSplit rs = split_rotation(u, false);
+          RotSplit rs;
+          if (r.g != nullptr && r.g->kind == kRotKind) {
+            const double tau = r.g->p[0];
+            rs = {false, tau, 1.0 / std::sqrt(1.0 + tau * tau), 1.0, cd(r.g->p[1], r.g->p[2]), 1.0};
+          } else {
+            rs = split_rotation(u, false);
+          }
           const TauParts tp = split_tau(rs.tau);
           const cd u01 = -rs.tau * rs.beta;
           carry *= rs.gamma * rs.scale;
@@ -1243,7 +1271,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
           op.d0one = rs.beta == cd(1.0) ? 1 : op.lo[3].x == 0.f && op.lo[3].y == 0.f ? 2 : 0;
           pass_cost += 1.0;
           P.ops.push_back(op);
-          if (rs.flip) emit_raw({gate_matrix(TQS_X, nullptr), G_ANTI, false, true, r.t, -1, false}, emit_raw);
+          if (rs.flip) emit_raw({nullptr, gate_matrix(TQS_X, nullptr), G_ANTI, false, true, r.t, -1, false}, emit_raw);
           if (rs.alpha != cd(1.0)) emit_phase(rs.alpha, tl);
           return;
         } else {  // controlled: hi + lo coefficients
@@ -1286,9 +1314,9 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
       Mat2 d1, d2;
       if (!split && r.single && !r.is_h && r.cls != G_DIAG && h_count < kMaxHPerPass &&
           hadamard_split(r.u, d2, d1)) {
-        emit_raw({d2, G_DIAG, false, true, r.t, -1, false}, emit_raw);
-        emit_raw({gate_matrix(TQS_H, nullptr), G_DENSE, true, true, r.t, -1, false}, emit_raw);
-        emit_raw({d1, G_DIAG, false, true, r.t, -1, false}, emit_raw);
+        emit_raw({nullptr, d2, G_DIAG, false, true, r.t, -1, false}, emit_raw);
+        emit_raw({nullptr, gate_matrix(TQS_H, nullptr), G_DENSE, true, true, r.t, -1, false}, emit_raw);
+        emit_raw({nullptr, d1, G_DIAG, false, true, r.t, -1, false}, emit_raw);
         continue;
       }
       // An uncontrolled anti-diagonal factor [[0, b], [c, 0]] other than X
@@ -1296,8 +1324,8 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
       // exchange.
       if (!split && r.single && !r.is_h && r.cls == G_ANTI && !(r.u.m[1] == cd(1.0) && r.u.m[2] == cd(1.0)) &&
           exact_phase(r.u.m[1]) && exact_phase(r.u.m[2])) {
-        emit_raw({Mat2{{r.u.m[2], 0.0, 0.0, r.u.m[1]}}, G_DIAG, false, true, r.t, -1, false}, emit_raw);
-        emit_raw({gate_matrix(TQS_X, nullptr), G_ANTI, false, true, r.t, -1, false}, emit_raw);
+        emit_raw({nullptr, Mat2{{r.u.m[2], 0.0, 0.0, r.u.m[1]}}, G_DIAG, false, true, r.t, -1, false}, emit_raw);
+        emit_raw({nullptr, gate_matrix(TQS_X, nullptr), G_ANTI, false, true, r.t, -1, false}, emit_raw);
         continue;
       }
       emit_raw(r, emit_raw);
@@ -1374,7 +1402,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
       push_raw(g, cls, t, c);
       grow_in_pass += grows;
     }
-    for (; idx < pending.size(); ++idx) still.push_back(pending[idx]);
+    still.insert(still.end(), pending.begin() + static_cast<std::ptrdiff_t>(idx), pending.end());
     emit_pass(Lmask, nL, still.empty());
     pending.swap(still);
   }

@@ -128,7 +128,8 @@ static tqs_status compile_fsv(int n, const std::vector<Gate>& circuit, int max_g
   // with a bound on the gates per pass counts the circuit's own gates).
   std::vector<const Gate*> gates;
   for (const Gate& g : circuit) gates.push_back(&g);
-  std::deque<Gate> store;
+  static thread_local GateStore store;
+  store.clear();
   cd carry = 1.0;
   const bool split = max_gates == 0 && prepare_gates(n, gates, store, carry, nullptr, false);
   if (max_gates == 0 && !split) {
