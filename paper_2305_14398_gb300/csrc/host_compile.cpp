@@ -932,8 +932,15 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, GateStore& store, cd& gl
       p.flip = r.flip;
     }
     p.rot = true;
-    if (r.tau == 0.0) {  // nothing to turn
-      put_phase(kPhaseKind, q, r.beta);
+    if (r.tau == 0.0) {
+      // nothing to turn: a phase alone, pending as well where Z is (X diag(1, beta) =
+      // beta diag(1, conj beta) X)
+      if (left_x) {
+        put_phase(exact_phase(r.beta) ? TQS_R : kPhaseKind, q, r.beta);
+      } else {
+        if (r.flip) global *= r.beta;
+        p.phi = snap_phase(r.alpha * (r.flip ? std::conj(r.beta) : r.beta));
+      }
     } else {
       Gate* g = put(kRotKind, q, rotation_part(r));
       g->p[0] = r.tau;
