@@ -221,8 +221,8 @@ constexpr int kCustomKind = 64;
 // Internal kind of the phase diag(1, phi) that prepare_gates puts before the
 // target of a CNOT: it runs in a pass where its qubit is local, as hi + lo.
 constexpr int kPhaseKind = 65;
-// Internal kind of a rotation that prepare_gates took out of a factor: u =
-// scale [[1, -tau], [tau, 1]] diag(1, beta), p[0] = tau, p[1] + i p[2] = beta.
+// Internal kind of a rotation that prepare_gates took out of a factor: u is
+// [[1, -tau], [tau, 1]] diag(1, beta), unscaled, p[0] = tau, p[1] + i p[2] = beta.
 constexpr int kRotKind = 66;
 
 // One recorded operation.

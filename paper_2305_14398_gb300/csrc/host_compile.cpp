@@ -190,12 +190,11 @@ double single_cost(const Mat2& u, bool is_h) {
 //   u = gamma diag(1, alpha) X^flip scale R diag(1, beta),  R = [[1, -tau], [tau, 1]],
 // with phases alpha, beta, gamma and |tau| the ratio of the small to the large
 // entry, at most 1.  R costs two multiply-adds per real part (the dense product
-// with hi + lo coefficients: eight), and scale = (1 + tau^2)^-1/2 is taken
+// with hi + lo coefficients: eight).  The emitter takes scale = (1 + tau^2)^-1/2
 // from tau as the record holds it (TauParts), so scale R is a rotation exactly.
 struct RotSplit {
   bool flip;
   double tau;
-  double scale;
   cd alpha, beta, gamma;
 };
 
@@ -207,8 +206,9 @@ cd snap_unit(cd z) {
   }
   return z;
 }
-cd unit(cd z) { return z * (1.0 / std::sqrt(std::norm(z))); }
-cd snap_phase(cd z) { return snap_unit(unit(z)); }
+// A product of phases, of modulus 1 but for rounding (a custom unitary's entries:
+// 1e-9): one Newton step to modulus 1.
+cd snap_phase(cd z) { return snap_unit(z * (1.5 - 0.5 * std::norm(z))); }
 
 // tau as the record holds it, a + b in FP32.  One FP32 value is off by up to
 // 2^-25, the same way for the same angle, and a circuit that repeats an angle adds
@@ -249,10 +249,10 @@ class SeenAngles {
   // Whether one FP32 value will do for this use.
   bool one_will_do(double tau) {
     const float t = static_cast<float>(std::abs(tau));
-    const float off = static_cast<float>(std::abs(std::abs(tau) - double(t)) / (1.0 + tau * tau));
+    const float off = static_cast<float>(std::abs(std::abs(tau) - double(t)));
     uint32_t key;
     std::memcpy(&key, &t, 4);
-    uint32_t h = (key * 0x9E3779B1u) >> 20;
+    uint32_t h = (key * 0x9E3779B1u) >> 21;
     for (int i = 0; i < 8; ++i, h = (h + 1) & (kSlots - 1)) {
       Slot& s = slots_[h];
       if (s.epoch != epoch_) s = {epoch_, key, 0.f};
@@ -265,7 +265,7 @@ class SeenAngles {
   }
 
  private:
-  static constexpr uint32_t kSlots = 4096;  // 2^(32 - 20)
+  static constexpr uint32_t kSlots = 2048;  // 2^(32 - 21)
   struct Slot {
     uint32_t epoch = 0, key = 0;
     float off = 0.f;
@@ -282,50 +282,39 @@ class SeenAngles {
 // seen: the circuit's angles, if one FP32 value may do for tau.
 RotSplit split_rotation(const Mat2& u, bool real_column, SeenAngles* seen = nullptr) {
   RotSplit r;
-  // (moduli as roots of sums of squares and phases multiplied by conjugates: the
-  // entries are at most 1, and hypot and complex division took most of a circuit's compile)
-  double c = std::sqrt(std::norm(u.m[0])), s = std::sqrt(std::norm(u.m[2]));
-  if (s <= 1e-14) s = 0.0;  // rounding of a zero: its phase means nothing
-  if (c <= 1e-14) c = 0.0;
-  r.flip = s > c;
+  // Moduli as roots of sums of squares and phases multiplied by conjugates (the
+  // entries are at most 1): hypot and complex division took a third of a
+  // circuit's compile.
+  const double n0 = std::norm(u.m[0]), n1 = std::norm(u.m[2]);
+  r.flip = n1 > n0;
   // u = gamma diag(p0, p1) [[c, -s beta], [s, c beta]]; with s > c the bracket
   // is X [[s, c beta], [c, -s beta]] = X [[s, -c beta'], [c, s beta']], beta' = -beta
-  cd p0, p1;  // the phases of the first column, row 0 and row 1
-  const bool minus = real_column && (u.m[2] * std::conj(u.m[0])).real() < 0.0;
-  if (!r.flip) {
-    p0 = u.m[0] * (1.0 / c);
-    p1 = s == 0.0 ? p0 : !real_column ? u.m[2] * (1.0 / s) : minus ? -p0 : p0;
-    r.tau = s / c;
-    r.beta = u.m[3] * std::conj(p1);
-  } else {
-    p1 = u.m[2] * (1.0 / s);
-    p0 = c == 0.0 ? p1 : !real_column ? u.m[0] * (1.0 / c) : minus ? -p1 : p1;
-    r.tau = c / s;
-    r.beta = u.m[1] * std::conj(p0);
-  }
-  r.beta = snap_phase(r.beta);
-  r.gamma = snap_unit(p0);
-  r.alpha = snap_unit(p1 * std::conj(p0));
-  if (r.alpha == cd(-1.0)) {  // a sign: the rotation the other way
-    r.alpha = 1.0;
-    r.tau = -r.tau;
-    r.beta = -r.beta;
-    if (r.flip) r.gamma = -r.gamma;
-  }
+  const cd mb = r.flip ? u.m[2] : u.m[0], ms = r.flip ? u.m[0] : u.m[2];  // the first column by size
+  const cd ob = r.flip ? u.m[1] : u.m[3];                                // the other large entry
+  const double w = 1.0 / std::sqrt(r.flip ? n1 : n0);
+  double s = std::sqrt(r.flip ? n0 : n1);
+  const cd pb = mb * w;  // their phases, the large one's and the small one's
+  cd ps = pb;
+  if (s <= 1e-14) s = 0.0;  // rounding of a zero: its phase means nothing
+  else if (!real_column) ps = ms * (1.0 / s);
+  else if ((ms * std::conj(mb)).real() < 0.0) ps = -pb;
+  r.tau = s * w;
+  r.beta = snap_phase(ob * std::conj(ps) * w);
+  r.gamma = snap_unit(r.flip ? ps : pb);
+  const cd a = ps * std::conj(pb);
+  r.alpha = snap_unit(r.flip ? std::conj(a) : a);
+  const bool minus = r.alpha == cd(-1.0);  // a sign: the rotation the other way
+  r.alpha = minus ? cd(1.0) : r.alpha;
+  r.tau = minus ? -r.tau : r.tau;
+  r.beta = minus ? -r.beta : r.beta;
+  r.gamma = minus && r.flip ? -r.gamma : r.gamma;
   if (seen != nullptr && seen->one_will_do(r.tau)) {
     r.tau = static_cast<float>(r.tau);
   } else {
     const TauParts p = split_tau(r.tau);
     r.tau = double(p.a) + double(p.b);
   }
-  r.scale = 1.0 / std::sqrt(1.0 + r.tau * r.tau);
   return r;
-}
-
-// scale R diag(1, beta): what is left of u with gamma, alpha and X taken out.
-Mat2 rotation_part(const RotSplit& r) {
-  const double c = r.scale, s = r.scale * r.tau;
-  return {{c, -s * r.beta, s, c * r.beta}};
 }
 
 // The FP32 pair near z whose modulus is nearest |z|: a value that multiplies
@@ -918,7 +907,8 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, GateStore& store, cd& gl
       // the X factor that makes the first column real up to a phase, its larger part first
       const cd w0 = u.m[0] + u.m[2], w1 = u.m[0] - u.m[2];
       const cd v0 = u.m[1] + u.m[3], v1 = u.m[1] - u.m[3];
-      if (std::norm(w0) > 0.0 && std::norm(w1) > 0.0) p.phi = snap_unit(unit(w1) * std::conj(unit(w0)));
+      const double nn = std::norm(w0) * std::norm(w1);
+      if (nn > 0.0) p.phi = snap_unit(w1 * std::conj(w0) * (1.0 / std::sqrt(nn)));
       p.x = true;
       const cd x1 = std::conj(p.phi) * w1, y1 = std::conj(p.phi) * v1;
       u = {{0.5 * (w0 + x1), 0.5 * (v0 + y1), 0.5 * (w0 - x1), 0.5 * (v0 - y1)}};
@@ -942,7 +932,7 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, GateStore& store, cd& gl
         p.phi = snap_phase(r.alpha * (r.flip ? std::conj(r.beta) : r.beta));
       }
     } else {
-      Gate* g = put(kRotKind, q, rotation_part(r));
+      Gate* g = put(kRotKind, q, {{1.0, -r.tau * r.beta, r.tau, r.beta}});
       g->p[0] = r.tau;
       g->p[1] = r.beta.real();
       g->p[2] = r.beta.imag();
@@ -1144,6 +1134,8 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     split = prepare_gates(n, gs, fused_tls, P.carry, absorb ? &flips : nullptr, from_basis);
   }
 
+  P.ops.reserve(P.ops.size() + gs.size() + gs.size() / 4 + 16);
+
   std::vector<uint32_t>& qmask = qmask_tls;
   std::vector<GClass>& gcls = cls_tls;
   qmask.resize(gs.size());
@@ -1211,6 +1203,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     ps.op_begin = static_cast<uint32_t>(P.ops.size());
     double pass_cost = 6.0;
     int h_count = 0;
+    double grown = 1.0;  // the square of what the pass's rotations scale by
     // the phase diag(1, alpha) that a rotation leaves on its own target
     auto emit_phase = [&](cd alpha, int tl) {
       FusedOp op{};
@@ -1246,7 +1239,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
         if (cl >= 0) op.act = kLocalControlMask[cl];
         if (r.is_h) {
           op.code = static_cast<uint8_t>(OPC_H + tl);
-          if (split) carry *= std::sqrt(0.5);
+          if (split) grown *= 2.0;
           else ++h_count;
           pass_cost += 0.5;
         } else if (r.cls == G_ANTI && u.m[1] == cd(1.0) && u.m[2] == cd(1.0)) {
@@ -1257,14 +1250,14 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
         } else if (r.c < 0) {  // dense, or anti-diagonal other than X: a rotation
           RotSplit rs;
           if (r.g != nullptr && r.g->kind == kRotKind) {
-            const double tau = r.g->p[0];
-            rs = {false, tau, 1.0 / std::sqrt(1.0 + tau * tau), 1.0, cd(r.g->p[1], r.g->p[2]), 1.0};
+            rs = {false, r.g->p[0], 1.0, cd(r.g->p[1], r.g->p[2]), 1.0};
           } else {
             rs = split_rotation(u, false);
           }
           const TauParts tp = split_tau(rs.tau);
           const cd u01 = -rs.tau * rs.beta;
-          carry *= rs.gamma * rs.scale;
+          carry *= rs.gamma;
+          grown *= 1.0 + rs.tau * rs.tau;
           P.rot = std::max(P.rot, tp.b != 0.f ? 2 : 1);
           op.code = static_cast<uint8_t>(OPC_DENSE + tl);
           op.hc = make_float2(tp.a, tp.b);
@@ -1345,6 +1338,7 @@ void compile_program(int n, const std::vector<const Gate*>& gs_in, Program& P,
     const int tot = h_carry + h_count;
     ps.scale = std::ldexp(1.0f, -(tot / 2));
     h_carry = tot % 2;
+    if (grown != 1.0) carry *= 1.0 / std::sqrt(grown);
     // rotations: rescaled only once the factor held back is below 2^-20
     if (const double left = std::abs(carry); left < 0x1p-20) {
       const int k = -std::ilogb(left) - 1;
