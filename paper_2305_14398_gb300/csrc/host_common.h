@@ -884,9 +884,10 @@ inline std::atomic<int> g_chain_kchunk{0};
 // TQS_OPT_CHAIN_PAIR: kept and returned, without effect.
 inline std::atomic<int> g_chain_pair{0};
 
-// instr: the circuits hold instructions (their reductions are summed in a
-// partition that depends on the CTA's threads, which then stay the option's).
-inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint, bool instr = false) {
+// rot: FusedLaunch::rot of the launch.  instr: the circuits hold instructions
+// (their reductions are summed in a partition that depends on the CTA's
+// threads, which then stay the option's).
+inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint, int rot, bool instr = false) {
   LaunchPlan lp{team, 1, 4, 1};
   if (team == TEAM_WARP) {
     lp.slice_q = std::max(4, max_nint);
@@ -923,8 +924,11 @@ inline LaunchPlan plan_for(int team, int max_nint, int jobs, int warps_hint, boo
     // outputs than from a second set of threads: 1024 random circuits of 12
     // qubits 408 -> 194 us, of 13 qubits 546 -> 312 us, QFT and the like 267 ->
     // 166 us (4096 of 12) and 176 -> 118 us (2048 of 13).
-    // (One circuit alone writes its outputs faster with all.)
-    if (!instr && jobs > 1 && (lp.slice_q <= 12 || (lp.slice_q == 13 && jobs > device_sms())))
+    // Without general gates a circuit's time is mostly its outputs, which all the
+    // threads write faster: up to two rounds of the GPU (250 programs of 12 and 13
+    // qubits 19.9 and 26.7 us, with half 23.2 and 33.7; 400: 28.7 and 35.9
+    // against 23.2 and 33.7).  One circuit alone takes all, too.
+    if (!instr && jobs > (rot != 0 ? 1 : 2 * device_sms()) && (lp.slice_q <= 12 || (lp.slice_q == 13 && jobs > device_sms())))
       lp.warps = std::min(lp.warps, 8);
     const int per_sm = std::max(1, fused_max_ctas_per_sm(TEAM_CTA, lp.warps, lp.slice_q));
     lp.grid = std::max(1, std::min(jobs, per_sm * device_sms()));
@@ -1274,7 +1278,7 @@ struct tqs_batch {
   bool one_each(int kind) const { return team_of(kind) == TEAM_SOLO && plans[kind].grid == n_kind[kind]; }
   void make_plans() {
     for (int t = 0; t < kKinds; ++t)
-      plans[t] = plan_for(team_of(t), max_nint[t], n_kind[t], 0, instr_off.back() > 0);
+      plans[t] = plan_for(team_of(t), max_nint[t], n_kind[t], 0, rot[t], instr_off.back() > 0);
   }
   // graph cache
   cudaStream_t cap_stream = nullptr;

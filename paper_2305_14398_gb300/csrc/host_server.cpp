@@ -111,7 +111,7 @@ static tqs_status server_launch(tqs_server* sv, SrvSlot& sl) {
   LaunchPlan plans[3];
   int rot[3] = {0, 0, 0};  // FusedLaunch::rot
   for (const SrvReq& r : sl.reqs) rot[team_for(r.prog.nint)] = std::max(rot[team_for(r.prog.nint)], r.prog.rot);
-  for (int t = 0; t < 3; ++t) plans[t] = plan_for(t, max_nint[t], n_team[t], 0);
+  for (int t = 0; t < 3; ++t) plans[t] = plan_for(t, max_nint[t], n_team[t], 0, rot[t]);
   // Few global-class requests: K cooperating CTAs each (TEAM_MULTI),
   // bitwise the same results as one CTA each.  The J K CTAs take at most an
   // equal share of the SMs per slot in flight, counted in CTAs of kGlobalThreads

@@ -278,7 +278,7 @@ static tqs_status simulate_impl(tqs_circuit* c, const tqs_c64* d_init, tqs_c64* 
     TQS_CUDA(launch_fused(L, s), "tqs_simulate: launch");
     return TQS_OK;
   }
-  const LaunchPlan lp = plan_for(team, P.nint, 1, 1, P.n_instr > 0);
+  const LaunchPlan lp = plan_for(team, P.nint, 1, 1, P.rot, P.n_instr > 0);
   L.team = lp.team;
   L.norm_width = lp.norm_width;
   L.warps_per_cta = lp.warps;
