@@ -15,7 +15,7 @@ namespace {
 constexpr int kMatThreads = 256;
 constexpr int kMaxFactors = 16;
 
-// Small matrices (n < kMatExpandQ): one product over the factors per entry.
+// Small matrices and few factors (expansion_pays): one product over the factors per entry.
 __global__ void __launch_bounds__(kMatThreads)
     materialize_small_kernel(const StepFactor* __restrict__ factors, int nf, uint32_t idle, int n,
                        float2* __restrict__ S) {
@@ -50,7 +50,11 @@ __global__ void __launch_bounds__(kMatThreads)
 // then expands 8 of those by the top 3 qubits into the matrix, two neighbours
 // at once, so that a warp's store covers 512 contiguous bytes.  Same matrix:
 // 29 us, and n = 14 at 6.9 TB/s, the measured copy rate (n = 12, 13: 4.7, 6.3 TB/s).
-constexpr int kMatExpandQ = 10;  // below, 16 or fewer blocks are slower than the small kernel (9 us against 12)
+// Where expansion is the faster: its time hardly depends on the factors (n = 10
+// 9..11 us, n = 11 11..13 us, n = 12 25..29 us), the small kernel's grows with their
+// number (n = 10, 2 to 6 factors 8.2..8.6 us, 8 9.9, 10 16.6; n = 11, 2 and 3 9.5 us, 4 12.0, 6
+// 18.7; n = 12, 3 25.9 us, 6 60); n = 9 9 us against 12.
+inline bool expansion_pays(int n, int factors) { return n >= 12 || (n == 11 && factors > 4) || (n == 10 && factors > 8); }
 constexpr int kMatMid = 2048;  // entries of the 2^(n-3)-entry row parts of a block
 
 // How the expansion by qubit q multiplies: the index of the factor whose
@@ -216,7 +220,7 @@ int sm_count() {
 cudaError_t launch_materialize(const StepFactor* d_factors, StepDesc step, int n, float2* d_S,
                                cudaStream_t s) {
   if (step.f_count > kMaxFactors) return cudaErrorInvalidValue;
-  if (n >= kMatExpandQ) {
+  if (expansion_pays(n, step.f_count)) {
     materialize_kernel<<<1 << (2 * n - 14), kMatThreads, 0, s>>>(d_factors + step.f_begin, step.f_count,
                                                                  step.idle, n, d_S);
     count_launches(1);
