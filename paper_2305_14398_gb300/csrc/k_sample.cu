@@ -395,11 +395,15 @@ cudaError_t launch_sample(const SampleLaunch& L, cudaStream_t s) {
     }
   }
   if (L.n_sseg > 0 && L.shots > 0) {
-    // a thread per chunk of the largest segment, or per shot where there are
-    // more, up to kThreads; from 2^12 entries on two or four chunks a thread
+    // A thread per chunk of the largest segment, or per two shots (from 256 shots on
+    // four, from 512 on more) where that is more, up to kThreads; from 2^12
+    // entries on two or four chunks a thread.  With a thread per shot the blocks of
+    // small segments hold more warps than their tables are worth: 16000 states
+    // of 2^5, 64, 200 and 500 shots 24.7, 80 and 107 us, so 18.6, 49 and 76 us; 1000 states of
+    // 2^6, 200 shots 10.3 and 7.2 us.
     const int nc = L.smem_q > 3 ? 1 << (L.smem_q - 3) : 1;
     int threads = 32;
-    while (threads < kThreads && (threads < nc || threads < L.shots)) threads *= 2;
+    while (threads < kThreads && (threads < nc || (threads < 128 ? 2 : 4) * threads < L.shots)) threads *= 2;
     const int smem = nc * (kChunkPad + 1) * static_cast<int>(sizeof(double));
     static std::atomic<uint64_t> done[3];
     auto launch = [&](auto kernel, std::atomic<uint64_t>& d) -> cudaError_t {
