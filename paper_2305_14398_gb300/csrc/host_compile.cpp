@@ -878,7 +878,11 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, GateStore& store, cd& gl
     return &g;
   };
   auto put_phase = [&](int kind, int q, cd phi) {
-    if (phi != cd(1.0)) put(kind, q, {{1.0, 0.0, 0.0, phi}});
+    if (phi == cd(1.0)) return;
+    // a phase that FP32 holds is a diagonal gate like any other: it needs no
+    // local position and merges with its neighbours
+    if (kind == kPhaseKind && exact_phase(phi)) kind = TQS_R;
+    put(kind, q, {{1.0, 0.0, 0.0, phi}});
   };
   // u times a pending factor
   auto times_pend = [&](const Mat2& u, const Pend& p) -> Mat2 {
@@ -897,6 +901,7 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, GateStore& store, cd& gl
     if (p.flip) global *= p.phi;
     put_phase(kPhaseKind, q, p.flip ? std::conj(p.phi) : p.phi);
     p.phi = 1.0;
+    p.rot = false;
   };
   // the rotation of u into the circuit, its left factor pending; its phase too
   // if none is to be left at the end (`last`)
@@ -926,7 +931,7 @@ bool prepare_gates(int n, std::vector<const Gate*>& gs, GateStore& store, cd& gl
       // nothing to turn: a phase alone, pending as well where Z is (X diag(1, beta) =
       // beta diag(1, conj beta) X)
       if (left_x) {
-        put_phase(exact_phase(r.beta) ? TQS_R : kPhaseKind, q, r.beta);
+        put_phase(kPhaseKind, q, r.beta);
       } else {
         if (r.flip) global *= r.beta;
         p.phi = snap_phase(r.alpha * (r.flip ? std::conj(r.beta) : r.beta));
