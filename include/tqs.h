@@ -169,7 +169,8 @@ tqs_status tqs_circuit_steps(const tqs_circuit* c, int* h_step_of_gate);
  *               (their FP32 rounding residues, dense ops)}.  code: 0-3
  *               Hadamard without its 2^-1/2, 4-7 X, 8-11 X under a far
  *               control, 12-27 X under a local control (12 + 4 t + c), 28-31
- *               anti-diagonal, 32-35 dense, 36-39 controlled dense, each + the
+ *               anti-diagonal, 32-35 a rotation after a phase
+ *               (m + lo: their product), 36-39 dense, controlled or not, each + the
  *               local target position t; diagonal: 40-43 local target, 44-47
  *               local target + far control, 48-51 far target + local control
  *               c, 52 far target, 53 both local (fields t, c).  fbit: far
@@ -201,7 +202,8 @@ tqs_status tqs_circuit_program(tqs_circuit* c, int* n_passes, int* n_ops, void* 
  *             in FP64 under TQS_OPT_EXACT_PROBS), or NULL.
  *   d_norm  : 1 double, receives sum_i |psi_i|^2 (FP64), or NULL.
  * n <= TQS_MAX_QUBITS.  Arithmetic: FP32 amplitudes, probabilities stored as
- * FP64, FP64 norm.  The circuit's device program is uploaded on the first
+ * FP64, FP64 norm.  General gates as in tqs_simulate_fsv; from |0...0> an angle
+ * takes one FP32 part as long as its uses are together off by at most 2^-24.  The circuit's device program is uploaded on the first
  * call and kept until the circuit or the d_init pointer changes; a 15-16
  * qubit circuit runs on several cooperating CTAs
  * (TQS_OPT_MULTI_CTAS).  A circuit handle is used by one stream at a time. */
@@ -265,7 +267,10 @@ tqs_status tqs_circuit_unitary_cols(tqs_circuit* c, int prec, int col0, int ncol
  * act on non-diagonally; controls and diagonal gates may sit on any qubit),
  * so the state crosses HBM twice per pass.  Custom unitaries are supported; measure/reset instructions return
  * TQS_ERR_UNSUPPORTED.  Scratch (cached on the circuit): the pass program.
- * FP32 amplitudes, FP32 hi + lo coefficients. */
+ * FP32 amplitudes.  A general single-qubit gate runs as a phase (FP32 hi + lo) and a
+ * rotation (its tangent to 2^-37, in two FP32 parts), other dense factors with FP32
+ * hi + lo coefficients; plain phases are FP32.  So the state may be taken through
+ * the same circuit many times: only plain phases' rounding adds up. */
 tqs_status tqs_simulate_fsv(tqs_circuit* c, tqs_c64* d_state, void* stream);
 
 /* Pass count and tile bits of the circuit's full-state-vector program (host
@@ -402,9 +407,11 @@ tqs_status tqs_batch_sample(tqs_batch* b, const double* d_probs, int shots, cons
 tqs_status tqs_batch_instructions(const tqs_batch* b, int64_t* h_off);
 
 /* Launch shape of a batch's persistent kernel for one size class (0: circuits
- * of n <= 11, run by one or two warps each; 1: n = 12..14, one CTA each with
- * the state in shared memory, launched size by size: the numbers are those of
- * all sizes, the threads the largest's; 2: n = 15..16, one CTA each on global scratch),
+ * of n <= 11, run by one or two warps each, or a CTA each where they are few or
+ * hold general gates; 1: n = 12..14, one CTA each with the state in shared
+ * memory, launched size by size; 2: n = 15..16, one CTA each on global scratch;
+ * where a class takes several launches, jobs, CTAs and teams are summed and the
+ * threads are the largest's),
  * as the last tqs_batch_run chose it from the options in force then (a
  * scheduling fact: results do not depend on it).  Outputs (each may be
  * NULL): jobs = circuits of that class, grid = CTAs, threads = threads per
@@ -540,8 +547,8 @@ tqs_status tqs_check_violations(uint32_t* count, int reset);
  * in HBM per gate.  Read by tqs_simulate_fsv and tqs_fsv_passes (a circuit's
  * cached passes are rebuilt when it changed).
  * TQS_OPT_MULTI_CTAS, key = 0, value = CTAs at most for one circuit of 15 or
- * 16 qubits (or 14, with general gates) in tqs_simulate, and for each request of 15 or 16 qubits of a server batch that
- * holds few of them (together at most the SMs divided by the server's batches
+ * 16 qubits (or of 14 with general gates and 8 passes or more) in tqs_simulate, and
+ * for each request of 15 or 16 qubits of a server batch that holds few of them (together at most the SMs divided by the server's batches
  * in flight) (0 or 1: one CTA; default 8; at most 64), counted in CTAs of 512
  * threads: each is launched as four of 128.  The CTAs (a cooperative launch)
  * share the circuit's passes, one thread per amplitude group, meet at a grid

@@ -1252,6 +1252,7 @@ struct tqs_batch {
   //   * Up to twice as many (16 CTAs of 32 threads to an SM), those without
   //     general gates (2000 of 9 qubits 23.3 -> 14.7 us, of 11 qubits 44.5 ->
   //     40.4 us; random ones of 8 qubits 93 against 109 us).
+  // (kSoloFew: 8 CTAs of 128 threads on each of the GB300's 152 SMs.)
   // Beyond, the paper's programs work few groups until their last passes and
   // are bound by their outputs (16384 of 11 qubits: 146 us on warps, 274 us on CTAs).
   static constexpr int kSoloFew = 1216;

@@ -13,11 +13,14 @@
 // pass, only the groups of 16 amplitudes that can be nonzero by then (the
 // support rule in run_circuit); the rest of its state is zero.
 //
-// Teams: one warp or a pair of warps per circuit (n <= 11), one 512-thread CTA
-// per circuit (n <= 14), one CTA on global scratch (n <= 16), or several
-// cooperating CTAs on global scratch for a few 15-16 qubit circuits
-// (TEAM_MULTI).  Warps/CTAs pull circuits from an atomic job counter
-// (costliest first), so one persistent launch runs a whole batch.
+// Teams: one warp or a pair of warps per circuit (n <= 11), or a CTA with a
+// thread per group where circuits are alone, few or hold general gates
+// (TEAM_SOLO; one alone also up to n = 14); one CTA of 256 or 512 threads per
+// circuit (n <= 14), one CTA on global scratch (n <= 16), or cooperating CTAs of 128
+// threads on global scratch for a few 15-16 qubit circuits and a lone one of 14
+// with general gates and 8 passes or more (TEAM_MULTI).  Where circuits queue,
+// warps/CTAs pull them from an atomic job counter (costliest first), so one
+// persistent launch runs a whole size class.
 #include "checked.h"
 #include "exact_sq.h"
 #include "tqs_internal.h"

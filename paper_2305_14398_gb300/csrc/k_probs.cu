@@ -14,7 +14,7 @@
 // (the squares added in FP64) a 2^24 state was bound by that pipe, 88 us, now 59
 // us; four loads in flight per thread give 10 of these.  2^25 amplitudes move
 // at 5.3 TB/s, 78 % of the copy rate; bound by instruction issue (71
-// instructions per amplitude, 62 % of the issue slots).
+// instructions per amplitude, 61 % of the issue slots, the ALU pipe 75 % busy).
 #include <mutex>
 
 #include "../../include/tqs.h"

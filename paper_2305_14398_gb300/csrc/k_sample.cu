@@ -201,15 +201,15 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // ------------------------------------------------------ shared-memory path
-// One CTA per segment (n <= kSampleSmemMaxQ).  Dynamic shared memory holds
-// the 2^smem_q entries, then the chunk prefixes (32 per block: at least 32).
+// One CTA per segment (n <= kSampleSmemMaxQ).  Dynamic shared memory holds the
+// segment's entries, 9 words to a chunk of 8 (kChunkPad), then a base per chunk.
 //
 // Here the cumulative sums are exact: each probability p becomes the 64-bit
 // integer floor(p 2^S), with S chosen from an FP32 estimate of the segment's
 // total T so that T 2^S stays below 2^61 (each entry then loses less than
 // 2^-60 T, all of them together less than 2^(n - 60) T: 4e-15 T at n = 13; a
-// probability below 2^-S counts as 0); the sums are integer additions in the
-// fixed order above, and a shot's target is floor(u T 2^S).  The FP64 pipe
+// probability below 2^-S counts as 0); the sums are integer additions, the
+// same in any order, and a shot's target is floor(u T 2^S).  The FP64 pipe
 // (1/64 of the FP32 rate on this GPU) is left to one multiply per shot.
 
 // p as FP32 (truncated; 0 below the FP32 range), from the FP64 bits with

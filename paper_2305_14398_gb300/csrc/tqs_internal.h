@@ -30,7 +30,7 @@ namespace tqs {
 //   OPC_HMASK        unscaled Hadamards on the local positions of the bit mask
 //                    in field t (two or more, in position order; they commute);
 //                    anti-diagonal factors other than X run as DENSE (fewer
-//                    kernel code paths, and their coefficients get hi + lo)
+//                    kernel code paths)
 //   OPC_XP           exchanges on local position t (field t) that commute and
 //                    compose: the pair (j, j ^ 2^t) swaps when bit j of `act`
 //                    XOR the parity of the group's physical bits in the far
